@@ -1,8 +1,10 @@
 // FP64 / complex-FP64 GEMM on the CUDA cores: C = alpha op(A) op(B) + beta C.
-// 64 x 64 output tile per 256-thread block, 4 x 4 outputs per thread, K
-// staged through shared memory in slices of 16. Long-K, small-output
-// products (Gram matrices, rho = Z_L^H Z_R) split K over blocks and reduce
-// the partials in a second, deterministic pass.
+// One output per thread in tiles of 16 x 8, K staged through shared memory in
+// slices of 16 and split over the CTAs of a cluster. Long-K,
+// small-output products (Gram matrices, rho = Z_L^H Z_R) with K >= 4096 take
+// a tall-skinny kernel whose partials a second, deterministic pass reduces.
+#include <cooperative_groups.h>
+
 #include "common.cuh"
 #include "kernels.h"
 
@@ -10,7 +12,13 @@ namespace ctm {
 
 namespace {
 
-constexpr int BM = 64, BN = 64, BK = 16;
+namespace cg = cooperative_groups;
+
+constexpr int TM = 16, TN = 8;   // outputs per CTA
+constexpr int GT = TM * TN;      // threads per CTA, one output each
+constexpr int BK = 16;           // K elements per staged slice
+constexpr int MAX_CTAS = 8;      // CTAs of a cluster that share the K splits of a tile
+constexpr int MAX_SPLITS = 64;
 
 struct GemmP {
   long M, N, K, kchunk;
@@ -18,8 +26,7 @@ struct GemmP {
   const void* B; long ldb, sB;
   void* C; long ldc, sC;
   double2 alpha, beta;
-  int splits;
-  void* work;
+  int splits, per_cta;   // K splits, and how many of them each CTA of the cluster takes
   int lower_only;
 };
 
@@ -29,47 +36,55 @@ template <> __device__ __forceinline__ cplx from2<cplx>(double2 v) { return v; }
 
 __device__ __forceinline__ bool is_zero(double2 v) { return v.x == 0.0 && v.y == 0.0; }
 
+// What bounds it: the fp64 pipe, about 1.6 multiply-adds per clock and SM (a
+// warp-wide one occupies its sub-partition for ~80 clocks). Operand traffic
+// is nothing beside that, so register tiles buy nothing; what counts is that
+// the multiply-adds are spread evenly over all SMs and that none is spent on
+// padding. Hence one output per thread in tiles of 16 x 8, four warps (one
+// per sub-partition), warps without a live row skipping the arithmetic, and
+// the K splits shared by the CTAs of a cluster, which add the partial sums
+// in split order through distributed shared memory (no second launch).
+// Against 64 x 64 tiles of 4 x 4 outputs a thread and a second launch for the
+// splits (same sums in the same order): 243 x 32 x 243 real 58-71 us -> 8-10,
+// 297 x 38 x 297 complex 230-264 us -> 25-33, 1024 x 69 x 1024 real 262 us ->
+// 173 (138 us at the pipe's rate).
 template <typename T, int OPA, int OPB>
-__global__ void __launch_bounds__(256) gemm_kernel(GemmP p) {
-  __shared__ T As[BK][BM + 1];
-  __shared__ T Bs[BK][BN + 1];
+__global__ void __launch_bounds__(GT) gemm_kernel(GemmP p) {
+  __shared__ T As[2][BK][TM + 1];
+  __shared__ T Bs[2][BK][TN + 1];
+  __shared__ T part[MAX_SPLITS / MAX_CTAS][GT];
   const int tid = threadIdx.x;
-  const int tx = tid & 15, ty = tid >> 4;
-  const long m0 = (long)blockIdx.y * BM, n0 = (long)blockIdx.x * BN;
-  if (p.lower_only && n0 > m0 + BM - 1) return;   // tile strictly above the diagonal
-  const int z = blockIdx.z;
-  const int b = z / p.splits, sp = z % p.splits;
-  const long kbeg = sp * p.kchunk;
-  const long kend = min(p.K, kbeg + p.kchunk);
+  const int tx = tid % TN, ty = tid / TN;
+  const unsigned ntn = (unsigned)((p.N + TN - 1) / TN);   // tiles in one grid axis: M may exceed 65535 tiles
+  const long m0 = (long)(blockIdx.x / ntn) * TM, n0 = (long)(blockIdx.x % ntn) * TN;
+  if (p.lower_only && n0 > m0 + TM - 1) return;   // tile strictly above the diagonal (whole cluster)
+  const int ctas = (p.splits + p.per_cta - 1) / p.per_cta;
+  const int b = blockIdx.y / ctas, rank = blockIdx.y % ctas;
   const T* A = static_cast<const T*>(p.A) + b * p.sA;
   const T* B = static_cast<const T*>(p.B) + b * p.sB;
   const T zero = zero_of(T());
-  T acc[4][4];
+  constexpr int NA = TM * BK / GT, NB = TN * BK / GT;
+  T ra[NA], rb[NB];
+  auto load = [&](long k0, long kend) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = zero;
-
-  for (long k0 = kbeg; k0 < kend; k0 += BK) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int e = tid + 256 * i;
+    for (int i = 0; i < NA; ++i) {
+      const int e = tid + GT * i;
       int mm, kk;
       if (OPA == OP_N || OPA == OP_R) { mm = e / BK; kk = e % BK; }
-      else { kk = e / BM; mm = e % BM; }
+      else { kk = e / TM; mm = e % TM; }
       const long gm = m0 + mm, gk = k0 + kk;
       T v = zero;
       if (gm < p.M && gk < kend) {
         v = (OPA == OP_N || OPA == OP_R) ? A[gm * p.lda + gk] : A[gk * p.lda + gm];
         if (OPA == OP_C || OPA == OP_R) v = conjv(v);
       }
-      As[kk][mm] = v;
+      ra[i] = v;
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int e = tid + 256 * i;
+    for (int i = 0; i < NB; ++i) {
+      const int e = tid + GT * i;
       int nn, kk;
-      if (OPB == OP_N || OPB == OP_R) { kk = e / BN; nn = e % BN; }
+      if (OPB == OP_N || OPB == OP_R) { kk = e / TN; nn = e % TN; }
       else { nn = e / BK; kk = e % BK; }
       const long gn = n0 + nn, gk = k0 + kk;
       T v = zero;
@@ -77,73 +92,83 @@ __global__ void __launch_bounds__(256) gemm_kernel(GemmP p) {
         v = (OPB == OP_N || OPB == OP_R) ? B[gk * p.ldb + gn] : B[gn * p.ldb + gk];
         if (OPB == OP_C || OPB == OP_R) v = conjv(v);
       }
-      Bs[kk][nn] = v;
+      rb[i] = v;
+    }
+  };
+  auto stage = [&](int buf) {
+#pragma unroll
+    for (int i = 0; i < NA; ++i) {
+      const int e = tid + GT * i;
+      if (OPA == OP_N || OPA == OP_R) As[buf][e % BK][e / BK] = ra[i];
+      else As[buf][e / TM][e % TM] = ra[i];
+    }
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+      const int e = tid + GT * i;
+      if (OPB == OP_N || OPB == OP_R) Bs[buf][e / TN][e % TN] = rb[i];
+      else Bs[buf][e % BK][e / BK] = rb[i];
+    }
+  };
+  // a warp covers 32 / TN rows: it computes only when its first row is live
+  const bool live = m0 + (tid & ~31) / TN < p.M;
+  T acc = zero;
+  int buf = 0;
+  const int s0 = rank * p.per_cta, s1 = min(p.splits, s0 + p.per_cta);
+  for (int sp = s0; sp < s1; ++sp) {
+    const long kbeg = sp * p.kchunk, kend = min(p.K, kbeg + p.kchunk);
+    acc = zero;
+    if (kbeg < kend) {
+      load(kbeg, kend);
+      stage(buf);
     }
     __syncthreads();
+    for (long k0 = kbeg; k0 < kend; k0 += BK, buf ^= 1) {
+      const bool more = k0 + BK < kend;
+      if (more) load(k0 + BK, kend);
+      const int kn = (int)min((long)BK, kend - k0);
+      if (live) {
+        if (kn == BK) {
 #pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      T a[4], bb[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) bb[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) fmav(acc[i][j], a[i], bb[j]);
+          for (int kk = 0; kk < BK; ++kk) fmav(acc, As[buf][kk][ty], Bs[buf][kk][tx]);
+        } else {
+          for (int kk = 0; kk < kn; ++kk) fmav(acc, As[buf][kk][ty], Bs[buf][kk][tx]);
+        }
+      }
+      if (more) stage(buf ^ 1);
+      __syncthreads();
     }
-    __syncthreads();
+    if (p.splits > 1) part[sp - s0][tid] = acc;
   }
-
+  T* C = static_cast<T*>(p.C) + b * p.sC;
+  auto put = [&](int e, T v) {
+    const long gm = m0 + e / TN, gn = n0 + e % TN;
+    if (gm >= p.M || gn >= p.N) return;
+    v = mulv(from2<T>(p.alpha), v);
+    if (!is_zero(p.beta)) v = addv(v, mulv(from2<T>(p.beta), C[gm * p.ldc + gn]));
+    C[gm * p.ldc + gn] = v;
+  };
   if (p.splits == 1) {
-    T* C = static_cast<T*>(p.C) + b * p.sC;
-    const T alpha = from2<T>(p.alpha), beta = from2<T>(p.beta);
-    const bool use_beta = !is_zero(p.beta);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const long gm = m0 + ty + 16 * i;
-      if (gm >= p.M) continue;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const long gn = n0 + tx + 16 * j;
-        if (gn >= p.N) continue;
-        T v = mulv(alpha, acc[i][j]);
-        if (use_beta) v = addv(v, mulv(beta, C[gm * p.ldc + gn]));
-        C[gm * p.ldc + gn] = v;
-      }
-    }
-  } else {
-    T* W = static_cast<T*>(p.work) + ((long)b * p.splits + sp) * p.M * p.N;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const long gm = m0 + ty + 16 * i;
-      if (gm >= p.M) continue;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const long gn = n0 + tx + 16 * j;
-        if (gn < p.N) W[gm * p.N + gn] = acc[i][j];
-      }
-    }
+    put(tid, acc);
+    return;
   }
-}
-
-template <typename T>
-__global__ void splitk_reduce(GemmP p, int batch) {
-  const long MN = p.M * p.N;
-  const T alpha = from2<T>(p.alpha), beta = from2<T>(p.beta);
-  const bool use_beta = !is_zero(p.beta);
-  for (long idx = blockIdx.x * (long)blockDim.x + threadIdx.x; idx < MN * batch;
-       idx += (long)gridDim.x * blockDim.x) {
-    const long b = idx / MN, e = idx % MN;
-    const T* W = static_cast<const T*>(p.work) + b * p.splits * MN + e;
-    T s = zero_of(T());
-    for (int k = 0; k < p.splits; ++k) s = addv(s, W[k * MN]);
-    T* C = static_cast<T*>(p.C) + b * p.sC;
-    const long m = e / p.N, n = e % p.N;
-    T v = mulv(alpha, s);
-    if (use_beta) v = addv(v, mulv(beta, C[m * p.ldc + n]));
-    C[m * p.ldc + n] = v;
+  if (ctas == 1) {   // every thread sums its own partial sums
+    T s = zero;
+    for (int sp = 0; sp < p.splits; ++sp) s = addv(s, part[sp][tid]);
+    put(tid, s);
+    return;
   }
+  // rank r of the cluster sums the outputs r per .. (r + 1) per - 1
+  cg::cluster_group cl = cg::this_cluster();
+  cl.sync();
+  const int per = (GT + ctas - 1) / ctas;
+  const int e = rank * per + tid;
+  if (tid < per && e < GT) {
+    T s = zero;
+    for (int sp = 0; sp < p.splits; ++sp)
+      s = addv(s, *cl.map_shared_rank(&part[sp % p.per_cta][e], sp / p.per_cta));
+    put(e, s);
+  }
+  cl.sync();   // no CTA leaves while another may read its partial sums
 }
 
 // ------------------------------------------- tall-skinny C = op(A) B
@@ -290,31 +315,47 @@ cudaError_t run_ts(const GemmDesc& g, const TsPlan& t, void* work, cudaStream_t 
   return cudaGetLastError();
 }
 
+// K splits of a product, from the number of 64 x 64 blocks of its result: at
+// least 64 K elements each. The splits fix the order of the sums.
 int choose_splits(const GemmDesc& g) {
-  const long tiles = ((g.M + BM - 1) / BM) * ((g.N + BN - 1) / BN) * g.batch;
+  const long blocks = ((g.M + 63) / 64) * ((g.N + 63) / 64) * g.batch;
   const long target = 152L * 2;
-  if (tiles >= target / 2) return 1;
-  long s = target / tiles;
-  const long kmax = (g.K + 4 * BK - 1) / (4 * BK);  // at least 4 k-slices each
+  if (blocks >= target / 2) return 1;
+  long s = target / blocks;
+  const long kmax = (g.K + 63) / 64;
   if (s > kmax) s = kmax;
-  if (s > 64) s = 64;
+  if (s > MAX_SPLITS) s = MAX_SPLITS;
   return s < 1 ? 1 : (int)s;
+}
+
+// CTAs that share the splits of a tile: doubled until the grid holds four
+// CTAs per SM or every CTA has one split
+int choose_ctas(const GemmDesc& g, int splits) {
+  const long tiles = ((g.M + TM - 1) / TM) * ((g.N + TN - 1) / TN) * g.batch;
+  int c = (splits + MAX_SPLITS / MAX_CTAS - 1) / (MAX_SPLITS / MAX_CTAS);
+  int n = 1;
+  while (n < c) n *= 2;   // part[] holds MAX_SPLITS / MAX_CTAS splits of a CTA
+  while (n < MAX_CTAS && 2 * n <= splits && tiles * n < 152L * 4) n *= 2;
+  return n;
 }
 
 template <typename T, int OPA, int OPB>
 cudaError_t run(const GemmP& p, int batch, cudaStream_t s, long* launches) {
-  dim3 grid((unsigned)((p.N + BN - 1) / BN), (unsigned)((p.M + BM - 1) / BM),
-            (unsigned)(batch * p.splits));
-  gemm_kernel<T, OPA, OPB><<<grid, 256, 0, s>>>(p);
+  const int ctas = (p.splits + p.per_cta - 1) / p.per_cta;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(((p.N + TN - 1) / TN) * ((p.M + TM - 1) / TM)),
+                     (unsigned)(batch * ctas));
+  cfg.blockDim = dim3(GT);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 1;
+  at[0].val.clusterDim.y = (unsigned)ctas;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = ctas > 1 ? 1 : 0;
   if (launches) ++*launches;
-  if (p.splits > 1) {
-    long n = p.M * p.N * batch;
-    long g = (n + 255) / 256;
-    if (g > 152 * 8) g = 152 * 8;
-    splitk_reduce<T><<<(unsigned)g, 256, 0, s>>>(p, batch);
-    if (launches) ++*launches;
-  }
-  return cudaGetLastError();
+  return cudaLaunchKernelEx(&cfg, gemm_kernel<T, OPA, OPB>, p);
 }
 
 template <typename T, int OPA>
@@ -382,9 +423,7 @@ __global__ void dot_final(const T* part, int nblk, T* out) {
 size_t gemm64_work_bytes(const GemmDesc& g) {
   const TsPlan t = ts_plan(g);
   if (t.use) return (size_t)t.gx * t.nout * (g.cx ? 16 : 8);
-  const int splits = choose_splits(g);
-  if (splits == 1) return 0;
-  return (size_t)splits * g.batch * g.M * g.N * (g.cx ? 16 : 8);
+  return 0;
 }
 
 cudaError_t gemm64(const GemmDesc& g, void* work, size_t work_bytes,
@@ -402,8 +441,8 @@ cudaError_t gemm64(const GemmDesc& g, void* work, size_t work_bytes,
   p.beta = make_double2(g.beta[0], g.beta[1]);
   p.lower_only = g.lower_only ? 1 : 0;
   p.splits = choose_splits(g);
-  if (p.splits > 1 && work_bytes < gemm64_work_bytes(g)) p.splits = 1;
-  p.work = work;
+  const int ctas = choose_ctas(g, p.splits);
+  p.per_cta = (p.splits + ctas - 1) / ctas;
   long kc = (g.K + p.splits - 1) / p.splits;
   kc = (kc + BK - 1) / BK * BK;
   p.kchunk = kc > 0 ? kc : BK;

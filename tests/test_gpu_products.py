@@ -1,0 +1,68 @@
+"""Corner x block products (ctm_corner_apply: the contractions of an enlarged
+corner, its absorption of A and conj(A), and the product with an N x k block)
+against a NumPy contraction of the same seeded tensors, at the sizes where the
+fp64 kernels can go wrong: one tile and less, ragged rows and columns, K
+splits that do not divide evenly among the CTAs of a cluster, and every
+geometry of the fused absorption.
+
+Every value is a chain of four fp64 sums of lengths chi, chi, D^2 and d D^2,
+then one of length N, so its error is at most (sum of the lengths + 5) eps
+times the same contraction of absolute values (each complex multiply-add
+counts as two real ones, hence the factor 2); the tolerance is that bound.
+"""
+import numpy as np
+import pytest
+
+import paper_2607_15158_gb300 as pkg
+
+pytestmark = pytest.mark.gpu
+
+
+def _normal(rng, shape, cplx):
+    x = rng.standard_normal(shape)
+    return x + 1j * rng.standard_normal(shape) if cplx else x
+
+
+def _corner(A, B, C, Ta, Tb):
+    x = np.einsum("pm,mnuv->pnuv", C, Ta)
+    x = np.einsum("tplw,pnuv->tlwnuv", Tb, x, optimize=True)
+    x = np.einsum("tlwnuv,sulde->twnvsde", x, A, optimize=True)
+    x = np.einsum("twnvsde,svwDE->tdDneE", x, B, optimize=True)
+    n = x.shape[0] * x.shape[1] * x.shape[2]
+    return x.reshape(n, n)
+
+
+@pytest.mark.parametrize("d,D,chi,p,cplx", [
+    (2, 2, 1, 5, False),     # N = k = 4: less than one tile
+    (2, 2, 8, 5, False),     # N = 32, k = 13
+    (2, 2, 9, 5, True),      # N = 36, k = 14
+    (1, 3, 10, 5, True),     # N = 90, d = 1
+    (2, 3, 27, 5, False),    # N = 243: four K splits
+    (2, 3, 33, 5, True),     # N = 297: five K splits on three CTAs
+    (3, 4, 17, 4, False),    # N = 272, d = 3, D = 4
+    (2, 4, 9, 2, True),      # D = 4 complex
+    (2, 5, 11, 5, False),    # N = 275, D = 5
+    (2, 5, 5, 5, True),
+    (2, 6, 7, 5, False),     # D = 6
+    (2, 6, 5, 1, True),
+    (2, 7, 4, 3, False),     # D = 7, 8: one pair per block
+    (2, 8, 3, 3, False),
+])
+@pytest.mark.parametrize("herm", [False, True])
+def test_corner_apply_fp64(d, D, chi, p, cplx, herm):
+    rng = np.random.default_rng(100 * D + chi)
+    A = _normal(rng, (d, D, D, D, D), cplx)
+    C = _normal(rng, (4, 1, chi, chi), cplx)
+    T = _normal(rng, (4, 1, chi, chi, D, D), cplx)
+    ctx = pkg.ctm_init(1, 1, [A], d, D, chi, cplx=cplx, opts=pkg.ctm_default_opts(p=p))
+    ctx.ctm_set_env(C, T)
+    Z = _normal(rng, (ctx.N, ctx.k), cplx)
+    out = ctx.ctm_corner_apply(0, 0, 0, 1, Z, herm=herm)
+    ctx.ctm_free()
+    Q = _corner(A, A.conj(), C[0, 0], T[0, 0], T[3, 0])
+    Qa = _corner(abs(A), abs(A), abs(C[0, 0]), abs(T[0, 0]), abs(T[3, 0]))
+    ref = (Q.conj().T if herm else Q) @ Z
+    bound = (Qa.T if herm else Qa) @ abs(Z)
+    n = 2 * chi + D * D + d * D * D + chi * D * D + 5
+    tol = (2 if cplx else 1) * n * np.finfo(float).eps
+    assert (np.abs(out - ref) <= tol * bound).all(), float((np.abs(out - ref) / bound).max())
