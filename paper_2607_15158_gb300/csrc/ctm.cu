@@ -464,7 +464,7 @@ ctm_status qr_inplace(ctm_ctx* c, void* Zm, void* tmp, bool split_mode) {
   ++c->qr_calls;
   const bool split = split_mode && c->split != nullptr && !c->exact;
   const int passes = 3;
-  const bool smem_chol = chol_smem_bytes(c->cx, c->k) <= (size_t)(226 * 1024);
+  const bool row_solve = trsm_rows_supported(c->cx, c->k);
   for (int pass = 0; pass < passes; ++pass) {
     const int opH = c->cx ? OP_C : OP_T;
     if (split && pass == passes - 1) {
@@ -499,45 +499,38 @@ ctm_status qr_inplace(ctm_ctx* c, void* Zm, void* tmp, bool split_mode) {
       g.A = Zm; g.lda = c->k;
       g.B = Zm; g.ldb = c->k;
       g.C = c->G; g.ldc = c->k;
-      g.lower_only = smem_chol;
+      g.lower_only = row_solve;
       CK(gemm_exact(c, g));
     }
     int* dead = c->dead;   // every pass finds and refills dependent columns
-    // the k x k factor on a cluster of eight SMs where it fits (chol_cluster.cu),
-    // else on one SM (the fp64 pipe of one SM bounds it)
+    const uint64_t rseed = (c->opts.seed * 1000003ull + c->qr_calls) * 4 + pass;
+    // the k x k factor on one SM or a cluster of eight (chol_cluster.cu)
     const bool cl_chol = chol_cluster_supported(c->cx, c->k);
-    if (split && smem_chol && pass == 1) {
+    if (split && row_solve && pass == 1) {
       // second pass of a split context: the block is already conditioned by
       // the shifted pass, so Q = Z D^-1 L^-H runs on the tensor cores (the
       // explicit k x k inverse replaces the fp64 row solve; its ~1e-7 error
       // is removed by the correction pass that follows)
-      if (cl_chol)
-        CTM_CUDA_OK(chol_cluster(c->cx, c->k, c->N, false, true, c->G, c->Linv, c->dsc, dead,
-                                 c->G, c->err, c->stream, &c->launches));
-      else
-        CTM_CUDA_OK(chol_factor_inv(c->cx, c->k, c->N, false, true, c->G, c->Linv, c->dsc, dead,
-                                    c->G, c->err, c->stream, &c->launches));
+      CTM_CUDA_OK(chol_cluster(c->cx, c->k, c->N, false, true, c->G, c->Linv, c->dsc, dead,
+                               c->G, c->err, c->stream, &c->launches));
       const ctm_status st = split_gemm(c->split, OP_N, Zm, c->k, OP_N, c->G, c->k, c->N, c->k,
                                        c->k, tmp, c->k, c->stream, &c->launches);
       if (st != CTM_OK) return fail(c, st, split_last_error(c->split));
-    } else if (smem_chol) {
-      // L = chol(D^-1 G D^-1) in shared memory, Q = Z D^-1 L^-H row by row
-      if (cl_chol && c->split && c->opts.fp64_tc) {
-        // split contexts: the explicit W = D^-1 L^-H (its norm is at most
-        // ~shift^-1/2 in the shifted pass) and Q = Z W as an fp64-accurate
-        // tensor-core product instead of the fp64 row solve
-        CTM_CUDA_OK(chol_cluster(c->cx, c->k, c->N, pass == 0, true, c->G, c->Linv, c->dsc, dead,
-                                 c->G, c->err, c->stream, &c->launches));
-        CK(mm_exact(c, OP_N, OP_N, c->N, c->k, c->k, Zm, c->k, c->G, c->k, tmp, c->k));
-      } else if (cl_chol) {
-        CTM_CUDA_OK(chol_cluster(c->cx, c->k, c->N, pass == 0, true, c->G, c->Linv, c->dsc, dead,
-                                 nullptr, c->err, c->stream, &c->launches));
-        CTM_CUDA_OK(trsm_rows(c->cx, c->k, c->N, c->Linv, c->dsc, Zm, tmp, c->num_sms, c->stream,
-                              &c->launches));
-      } else {
-        CTM_CUDA_OK(chol_qr_pass(c->cx, c->k, c->N, pass == 0, true, c->G, c->Linv, c->dsc, dead,
-                                 Zm, tmp, c->err, c->num_sms, c->stream, &c->launches));
-      }
+    } else if (row_solve && c->split && c->opts.fp64_tc) {
+      // split contexts: the explicit W = D^-1 L^-H (its norm is at most
+      // ~shift^-1/2 in the shifted pass) and Q = Z W as an fp64-accurate
+      // tensor-core product instead of the fp64 row solve
+      CTM_CUDA_OK(chol_cluster(c->cx, c->k, c->N, pass == 0, true, c->G, c->Linv, c->dsc, dead,
+                               c->G, c->err, c->stream, &c->launches));
+      CK(mm_exact(c, OP_N, OP_N, c->N, c->k, c->k, Zm, c->k, c->G, c->k, tmp, c->k));
+    } else if (row_solve) {
+      // L = chol(D^-1 G D^-1), Q = Z D^-1 L^-H row by row, in place, the dead
+      // columns refilled on the way
+      CTM_CUDA_OK(chol_cluster(c->cx, c->k, c->N, pass == 0, true, c->G, c->Linv, c->dsc, dead,
+                               nullptr, c->err, c->stream, &c->launches));
+      CTM_CUDA_OK(trsm_rows(c->cx, c->k, c->N, c->Linv, c->dsc, Zm, Zm, dead, rseed, c->num_sms,
+                            c->stream, &c->launches));
+      continue;
     } else if (cl_chol) {
       // the packed factor exceeds one CTA: the row-distributed cluster factor
       // forms W = D^-1 L^-H; Q = Z W (fp64-accurate in the shifted first
@@ -572,11 +565,8 @@ ctm_status qr_inplace(ctm_ctx* c, void* Zm, void* tmp, bool split_mode) {
         CK(gemm(c, h));
       }
     }
-    CTM_CUDA_OK(repair_dead_columns(c->cx, c->N, c->k, tmp, c->dead,
-                                    (c->opts.seed * 1000003ull + c->qr_calls) * 4 + pass,
-                                    c->stream, &c->launches));
-    CTM_CUDA_OK(cudaMemcpyAsync(Zm, tmp, (size_t)c->N * c->k * c->es, cudaMemcpyDeviceToDevice,
-                                c->stream));
+    CTM_CUDA_OK(repair_dead_columns(c->cx, c->N, c->k, tmp, Zm, dead, rseed, c->stream,
+                                    &c->launches));
   }
   return CTM_OK;
 }
@@ -2212,7 +2202,7 @@ ctm_status ctm_transfer_spectrum(ctm_ctx* c, int dir, int row, int nvals, double
       CK(mm_small(c, opH, OP_N, m, m, n, X, m, X, m, G, m));
       CTM_CUDA_OK(chol_inv(c->cx, m, n, false, G, Li, 1, dead, c->err, c->stream, &c->launches));
       CK(mm_small(c, OP_N, opH, n, m, m, X, m, Li, m, V2, m));
-      CTM_CUDA_OK(repair_dead_columns(c->cx, n, m, V2, dead, 104729ull + pass, c->stream,
+      CTM_CUDA_OK(repair_dead_columns(c->cx, n, m, V2, V2, dead, 104729ull + pass, c->stream,
                                       &c->launches));
       CTM_CUDA_OK(cudaMemcpyAsync(X, V2, (size_t)n * m * es, cudaMemcpyDeviceToDevice, c->stream));
     }

@@ -67,15 +67,15 @@ cudaError_t dot64(bool cx, bool conj_x, long n, const void* x, long sx,
 cudaError_t chol_inv(bool cx, int k, long n, bool shift, void* G, void* Linv,
                      int batch, int* dead, int* err, cudaStream_t s, long* launches);
 
-// One CholeskyQR pass with the factor in shared memory: L = chol(D^-1 G D^-1
-// (+ shift I)) (D = sqrt(diag G) with scale, else I; dead-column detection as
-// in chol_inv), then Q = Z D^-1 L^-H row by row on all SMs. Needs
-// chol_smem_bytes(cx, k) <= the shared memory of one block (k <= ~166
-// complex, ~235 real); dsc receives D (k doubles).
-size_t chol_smem_bytes(bool cx, int k);
-cudaError_t chol_qr_pass(bool cx, int k, long rows, bool shift, bool scale, const void* G,
-                         void* L, double* dsc, int* dead, const void* Z, void* Q, int* err,
-                         int num_sms, cudaStream_t s, long* launches);
+// Row solve of a CholeskyQR pass: Q = Z D^-1 L^-H row by row on all SMs, for a
+// factor L (k x k, lower) and scales D (dsc) of chol_cluster; the columns j
+// with dead[j] != 0 become repair directions (see repair_dead_columns). Q may
+// be Z. Needs the packed factor in one block's shared memory
+// (trsm_rows_supported: k <= ~166 complex, ~235 real).
+bool trsm_rows_supported(bool cx, int k);
+cudaError_t trsm_rows(bool cx, int k, long rows, const void* L, const double* dsc, const void* Z,
+                      void* Q, const int* dead, uint64_t seed, int num_sms, cudaStream_t s,
+                      long* launches);
 
 // ------------------------------------------------------------- absorb.cu
 // Out[t,d,D,n,e,E] = sum A[s,u,l,d,e] B[s,v,w,D,E] In[t,l,w,n,u,v] with In,
@@ -99,35 +99,23 @@ cudaError_t orth_correction(bool cx, int k, const void* G, void* B, cudaStream_t
 cudaError_t sub_inplace(bool cx, long n, void* z, const void* d, cudaStream_t s,
                         long* launches);
 
-// The factor of chol_qr_pass (same options) and, instead of the row solve,
-// W = D^-1 L^-H (k x k, row-major, upper triangular) so that the caller
-// forms Q = Z W with a GEMM. L receives the factor.
-cudaError_t chol_factor_inv(bool cx, int k, long rows, bool shift, bool scale, const void* G,
-                            void* L, double* dsc, int* dead, void* W, int* err, cudaStream_t s,
-                            long* launches);
-
-// The row solve of chol_qr_pass alone: Q = Z D^-1 L^-H for a factor L and
-// scales D already computed (chol_cluster).
-cudaError_t trsm_rows(bool cx, int k, long rows, const void* L, const double* dsc, const void* Z,
-                      void* Q, int num_sms, cudaStream_t s, long* launches);
-
 // ------------------------------------------------------- chol_cluster.cu
-// The factor of chol_qr_pass / chol_factor_inv (same options and outputs:
-// L, dsc, dead; with W != null also W = D^-1 L^-H) computed by a cluster of
-// eight CTAs (rows dealt cyclically, one cluster barrier per column). W may
-// alias G. Where the packed factor fits one CTA's shared memory (k <= 156
-// complex, 225 real) every CTA gathers it for the inverse; above that the
-// CTAs keep only their own rows and read the others through distributed
-// shared memory (chol_cluster_supported: up to k ~ 390 complex).
+// L = chol(D^-1 G D^-1 (+ shift I)) of a k x k Gram (D = sqrt(diag G) with
+// scale, else I; shift and dead-column detection as in chol_inv), with
+// W != null also W = D^-1 L^-H (row-major, upper triangular), on one CTA for
+// small k and on a cluster of eight CTAs above (rows dealt cyclically). dsc
+// receives D (k doubles). W may alias G. Supported up to k ~ 390 complex,
+// 576 real (chol_cluster_supported).
 bool chol_cluster_supported(bool cx, int k);
 cudaError_t chol_cluster(bool cx, int k, long rows, bool shift, bool scale, const void* G,
                          void* L, double* dsc, int* dead, void* W, int* err, cudaStream_t s,
                          long* launches);
 
-// Overwrite the dead columns of a rows x k matrix with deterministic
-// pseudo-random entries (a counter-based hash of seed, column, row).
-cudaError_t repair_dead_columns(bool cx, long rows, int k, void* Q, const int* dead,
-                                uint64_t seed, cudaStream_t s, long* launches);
+// Q = src (rows x k; src may be Q) with the dead columns overwritten with
+// deterministic pseudo-random entries (a counter-based hash of seed, column,
+// row).
+cudaError_t repair_dead_columns(bool cx, long rows, int k, const void* src, void* Q,
+                                const int* dead, uint64_t seed, cudaStream_t s, long* launches);
 
 // Per tensor (batch, stride): x <- x * conj(phase of its largest-modulus
 // entry, lowest index on ties) / ||x||_F. work: 3 * 152 * batch doubles;

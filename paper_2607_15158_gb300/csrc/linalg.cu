@@ -457,16 +457,25 @@ __device__ __forceinline__ double hash_uniform(uint64_t a, uint64_t b, uint64_t 
   return (double)(z >> 11) * (2.0 / 9007199254740992.0) - 1.0;
 }
 
+// entry (r, c) of a repair direction
+__device__ __forceinline__ double repair_entry(double, int c, long r, uint64_t seed) {
+  return hash_uniform(seed, (uint64_t)c, (uint64_t)r);
+}
+__device__ __forceinline__ cplx repair_entry(cplx, int c, long r, uint64_t seed) {
+  return make_double2(hash_uniform(seed, (uint64_t)c, (uint64_t)r),
+                      hash_uniform(seed ^ 0x5bd1e995ull, (uint64_t)c, (uint64_t)r));
+}
+
+// Q <- src with its dead columns replaced (src may be Q)
 template <typename T>
-__global__ void repair_kernel(long rows, int k, T* Q, const int* dead, uint64_t seed) {
+__global__ void repair_kernel(long rows, int k, const T* src, T* Q, const int* dead,
+                              uint64_t seed) {
   for (long idx = blockIdx.x * (long)blockDim.x + threadIdx.x; idx < rows * k;
        idx += (long)gridDim.x * blockDim.x) {
     const long r = idx / k;
     const int c = (int)(idx % k);
-    if (!dead[c]) continue;
-    const double x = hash_uniform(seed, (uint64_t)c, (uint64_t)r);
-    if constexpr (sizeof(T) == 8) Q[idx] = x;
-    else Q[idx] = make_double2(x, hash_uniform(seed ^ 0x5bd1e995ull, (uint64_t)c, (uint64_t)r));
+    if (dead[c]) Q[idx] = repair_entry(T(), c, r, seed);
+    else if (src != Q) Q[idx] = src[idx];
   }
 }
 
@@ -544,135 +553,40 @@ __global__ void scale_by_kernel(long n, T* x, long stride, const T* fac) {
 }
 
 // ---------------------------------------------------------------------
-// CholeskyQR pass with the Gram factor in shared memory: one block factors
-// the (optionally Jacobi-scaled, shifted) k x k Gram in packed lower storage
-// (fp64 bound on one SM; k(k+1)/2 elements must fit in shared memory), then
-// every block solves rows of Q L^H = Z D^-1 by forward substitution.
-__device__ __forceinline__ int tri(int i, int j) { return i * (i + 1) / 2 + j; }  // i >= j
-
-template <typename T>
-__global__ void __launch_bounds__(256) chol_smem_kernel(int k, long n, int shift, int scale,
-                                                        const T* G, T* L, double* dsc,
-                                                        int* dead, int* err) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* S = reinterpret_cast<T*>(smem_raw);
-  T* colj = S + (size_t)k * (k + 1) / 2;   // conj of column j of L, contiguous
-  double* orig = reinterpret_cast<double*>(colj + k);
-  __shared__ double red[8];
-  __shared__ double piv, sft_s;
-  __shared__ int isdead, bad;
-  // scales and packed load (lower triangle)
-  for (int i = threadIdx.x; i < k; i += blockDim.x) {
-    const double d = realv(G[(size_t)i * k + i]);
-    dsc[i] = scale ? (d > 0.0 ? sqrt(d) : 1.0) : 1.0;
-  }
-  __syncthreads();
-  for (long idx = threadIdx.x; idx < (long)k * (k + 1) / 2; idx += blockDim.x) {
-    // invert the packed index
-    int i = (int)((sqrt(8.0 * idx + 1.0) - 1.0) * 0.5);
-    while ((long)i * (i + 1) / 2 > idx) --i;
-    while ((long)(i + 1) * (i + 2) / 2 <= idx) ++i;
-    const int j = (int)(idx - (long)i * (i + 1) / 2);
-    S[idx] = scalev(G[(size_t)i * k + j], 1.0 / (dsc[i] * dsc[j]));
-  }
-  __syncthreads();
-  double tr = 0.0;
-  for (int i = threadIdx.x; i < k; i += blockDim.x) {
-    orig[i] = realv(S[tri(i, i)]);
-    tr += orig[i];
-    if (dead) dead[i] = 0;
-  }
-  tr = warp_sum(tr);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = tr;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-    sft_s = shift ? 11.0 * ((double)n * k + (double)k * (k + 1)) * DBL_EPSILON * t : 0.0;
-    bad = 0;
-  }
-  __syncthreads();
-  const double sft = sft_s;
-  if (sft != 0.0)
-    for (int i = threadIdx.x; i < k; i += blockDim.x) {
-      if constexpr (sizeof(T) == 8) S[tri(i, i)] += sft;
-      else S[tri(i, i)].x += sft;
-    }
-  __syncthreads();
-  for (int j = 0; j < k; ++j) {
-    if (threadIdx.x == 0) {
-      const double d = realv(S[tri(j, j)]);
-      isdead = 0;
-      if (dead && (shift ? !(d - sft > fmax(1e-9 * sft, 8.0 * k * DBL_EPSILON * (orig[j] + sft)))
-                         : !(d > 1e-10 * orig[j]))) {
-        isdead = 1;
-        piv = 1.0;
-        dead[j] = 1;
-      } else if (!(d > 0.0) || !isfinite(d)) {
-        piv = 1.0;
-        bad = 1;
-      } else {
-        piv = sqrt(d);
-      }
-    }
-    __syncthreads();
-    const double inv = 1.0 / piv;
-    for (int i = j + 1 + threadIdx.x; i < k; i += blockDim.x) {
-      const T v = isdead ? zero_of(T()) : scalev(S[tri(i, j)], inv);
-      S[tri(i, j)] = v;
-      colj[i] = conjv(v);
-    }
-    if (threadIdx.x == 0) {
-      if constexpr (sizeof(T) == 8) S[tri(j, j)] = isdead ? 1.0 : piv;
-      else S[tri(j, j)] = make_double2(isdead ? 1.0 : piv, 0.0);
-    }
-    __syncthreads();
-    if (!isdead) {
-      // trailing update S(i, l) -= L(i, j) conj(L(l, j)), j < l <= i: one
-      // row per warp, lanes along the row
-      const int wp = threadIdx.x >> 5, ln = threadIdx.x & 31, nw = blockDim.x >> 5;
-      for (int i = j + 1 + wp; i < k; i += nw) {
-        const T a = S[tri(i, j)];
-        T* Si = S + tri(i, 0);
-        for (int l = j + 1 + ln; l <= i; l += 32) Si[l] = subv(Si[l], mulv(a, colj[l]));
-      }
-    }
-    __syncthreads();
-  }
-  if (bad && threadIdx.x == 0) atomicOr(err, DEV_CHOL_PIVOT);
-  for (long idx = threadIdx.x; idx < (long)k * k; idx += blockDim.x) {
-    const int i = (int)(idx / k), j = (int)(idx % k);
-    L[idx] = (j <= i) ? S[tri(i, j)] : zero_of(T());
-  }
-}
+// Row solve of a CholeskyQR pass (the factor is chol_cluster's).
 
 // rows r of Q: q L^H = z D^-1, i.e. q_j = (z_j / D_j - sum_{i<j} q_i conj(L_ji)) / L_jj.
 // One warp per row, right-looking: lane l owns the columns l, l + 32, ...
-// (R of them, in registers); at step j the owner of column j finishes
-// q_j = acc_j / L_jj and broadcasts it, and every lane subtracts
-// q_j conj(L_ij) from its columns i > j. Each row costs k^2 / 2 multiply-adds
-// and no reductions; conj(L) is kept column by column (packed) in shared
-// memory so that the lanes read consecutive entries.
+// (R of them, in registers); at step j every lane finishes q_j = acc_j / L_jj
+// from the owner's acc_j and subtracts q_j conj(L_ij) from its columns i > j.
+// conj(L) is kept column by column (packed) in shared memory so that the
+// lanes read consecutive entries. Numerically dependent columns (dead) are
+// overwritten with the repair directions on the way out. Z and Q may be the
+// same matrix: a row is read before it is written, by the same warp.
+// Bound by latency: the chain of a row (a multiplication, a shuffle and a
+// multiply-add per column, ~160 clocks real) and, before it, the factor's way
+// into shared memory. The reciprocals of the diagonal are taken one per
+// thread (a division by one lane costs the fp64 pipe as much as 32), and the
+// rows are spread over all SMs before a block gets more than four warps.
+// 243 x 32 real 33 us -> 10, 1024 x 69 real 95 -> 24, 297 x 38 complex 94 -> 24
+// (before: 32 rows a block, a division per warp, then a repair and a copy).
 template <typename T, int R>
-__global__ void __launch_bounds__(1024, 1) trsm_warp_kernel(long rows, int k, const T* L,
-                                                            const double* dsc, const T* Z,
-                                                            T* Q) {
+__global__ void __launch_bounds__(1024, 1) trsm_rows_kernel(long rows, int k, const T* L,
+                                                            const double* dsc, const T* Z, T* Q,
+                                                            const int* dead, uint64_t seed) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* Lc = reinterpret_cast<T*>(smem_raw);   // column j at Lc[j k - j (j - 1) / 2 + i - j]
   double* rinv = reinterpret_cast<double*>(Lc + (size_t)k * (k + 1) / 2);
   double* dinv = rinv + k;
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int j = wp; j < k; j += nw) {
-    const int off = j * k - j * (j - 1) / 2;
-    for (int i = j + lane; i < k; i += 32) Lc[off + i - j] = conjv(L[(size_t)i * k + j]);
-    if (lane == 0) {
-      rinv[j] = 1.0 / realv(L[(size_t)j * k + j]);
-      dinv[j] = 1.0 / dsc[j];
-    }
+  for (int j = threadIdx.x; j < k; j += blockDim.x) {
+    rinv[j] = 1.0 / realv(L[(size_t)j * k + j]);
+    dinv[j] = 1.0 / dsc[j];
   }
+  for (int i = wp; i < k; i += nw)
+    for (int j = lane; j < i; j += 32)
+      Lc[j * k - j * (j - 1) / 2 + i - j] = conjv(L[(size_t)i * k + j]);
   __syncthreads();
-  // row r = wp G + b + t G nw: a partial last pass over the rows spreads
-  // over all blocks (a few warps each) instead of filling a few blocks
   for (long r = (long)wp * gridDim.x + blockIdx.x; r < rows; r += (long)gridDim.x * nw) {
     const T* z = Z + r * k;
     T a[R];
@@ -686,7 +600,6 @@ __global__ void __launch_bounds__(1024, 1) trsm_warp_kernel(long rows, int k, co
       for (int jj = 0; jj < 32; ++jj) {
         const int j = 32 * e + jj;
         if (j >= k) break;
-        if (lane == jj) a[e] = scalev(a[e], rinv[j]);
         T q;
         if constexpr (sizeof(T) == 8) {
           q = __shfl_sync(0xffffffffu, a[e], jj);
@@ -694,6 +607,8 @@ __global__ void __launch_bounds__(1024, 1) trsm_warp_kernel(long rows, int k, co
           q.x = __shfl_sync(0xffffffffu, a[e].x, jj);
           q.y = __shfl_sync(0xffffffffu, a[e].y, jj);
         }
+        q = scalev(q, rinv[j]);
+        if (lane == jj) a[e] = q;
         const T* Lj = Lc + (j * k - j * (j - 1) / 2) - j;
 #pragma unroll
         for (int e2 = e; e2 < R; ++e2) {
@@ -706,7 +621,7 @@ __global__ void __launch_bounds__(1024, 1) trsm_warp_kernel(long rows, int k, co
 #pragma unroll
     for (int e = 0; e < R; ++e) {
       const int i = lane + 32 * e;
-      if (i < k) qo[i] = a[e];
+      if (i < k) qo[i] = dead[i] ? repair_entry(T(), i, r, seed) : a[e];
     }
   }
 }
@@ -732,150 +647,59 @@ cudaError_t chol_inv(bool cx, int k, long n, bool shift, void* G, void* Linv,
   return cudaGetLastError();
 }
 
-size_t chol_smem_bytes(bool cx, int k) {
-  return ((size_t)k * (k + 1) / 2 + k) * (cx ? 16 : 8) + (size_t)k * sizeof(double) + 16;
+bool trsm_rows_supported(bool cx, int k) {
+  return ((size_t)k * (k + 1) / 2 + k) * (cx ? 16 : 8) + (size_t)k * sizeof(double) + 16 <=
+         (size_t)226 * 1024;
 }
 
-template <typename T>
-cudaError_t trsm_set_smem(size_t (&configured)[5], size_t shm) {
-  const void* fns[] = {(const void*)trsm_warp_kernel<T, 2>, (const void*)trsm_warp_kernel<T, 4>,
-                       (const void*)trsm_warp_kernel<T, 5>, (const void*)trsm_warp_kernel<T, 6>,
-                       (const void*)trsm_warp_kernel<T, 8>};
-  for (int i = 0; i < 5; ++i) {
-    const cudaError_t e = raise_smem(fns[i], configured[i], shm);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
-}
-
-// one shared-memory limit per Cholesky kernel instance, raised monotonically
-// (every launcher of chol_smem_kernel goes through here)
-cudaError_t chol_smem_prepare(bool cx, size_t shm) {
-  static size_t configured[2] = {0, 0};
-  return cx ? raise_smem((const void*)chol_smem_kernel<cplx>, configured[1], shm)
-            : raise_smem((const void*)chol_smem_kernel<double>, configured[0], shm);
-}
-
-// R = columns per lane: the smallest of 2, 4, 5, 6, 8 with 32 R >= k
-#define CTM_TRSM_LAUNCH(T)                                                                     \
-  do {                                                                                         \
-    if (k <= 64)                                                                               \
-      trsm_warp_kernel<T, 2><<<(unsigned)g, 1024, shm, s>>>(rows, k, (const T*)L, dsc,         \
-                                                             (const T*)Z, (T*)Q);              \
-    else if (k <= 128)                                                                         \
-      trsm_warp_kernel<T, 4><<<(unsigned)g, 1024, shm, s>>>(rows, k, (const T*)L, dsc,         \
-                                                             (const T*)Z, (T*)Q);              \
-    else if (k <= 160)                                                                         \
-      trsm_warp_kernel<T, 5><<<(unsigned)g, 1024, shm, s>>>(rows, k, (const T*)L, dsc,         \
-                                                             (const T*)Z, (T*)Q);              \
-    else if (k <= 192)                                                                         \
-      trsm_warp_kernel<T, 6><<<(unsigned)g, 1024, shm, s>>>(rows, k, (const T*)L, dsc,         \
-                                                             (const T*)Z, (T*)Q);              \
-    else                                                                                       \
-      trsm_warp_kernel<T, 8><<<(unsigned)g, 1024, shm, s>>>(rows, k, (const T*)L, dsc,         \
-                                                             (const T*)Z, (T*)Q);              \
-  } while (0)
-
-cudaError_t chol_qr_pass(bool cx, int k, long rows, bool shift, bool scale, const void* G,
-                         void* L, double* dsc, int* dead, const void* Z, void* Q, int* err,
-                         int num_sms, cudaStream_t s, long* launches) {
-  const size_t shm = chol_smem_bytes(cx, k);
-  static size_t configured_trsm[2][5] = {{0}};
-  {
-    cudaError_t e = chol_smem_prepare(cx, shm);
-    if (e == cudaSuccess) e = cx ? trsm_set_smem<cplx>(configured_trsm[1], shm)
-                                 : trsm_set_smem<double>(configured_trsm[0], shm);
-    if (e != cudaSuccess) return e;
-  }
-  // one 1024-thread block per SM (the factor fills shared memory), one warp
-  // per row
-  long g = (rows + 31) / 32;
+template <typename T, int R>
+cudaError_t launch_trsm(int k, long rows, const void* L, const double* dsc, const void* Z, void* Q,
+                        const int* dead, uint64_t seed, int num_sms, cudaStream_t s) {
+  const size_t shm = (size_t)k * (k + 1) / 2 * sizeof(T) + 2 * (size_t)k * sizeof(double);
+  static size_t configured = 0;
+  const cudaError_t e = raise_smem((const void*)trsm_rows_kernel<T, R>, configured, shm);
+  if (e != cudaSuccess) return e;
+  // four warps a block (one per fp64 pipe) while the rows fit that way, else
+  // as many as give every row its warp, up to 32
+  long nw = (rows + num_sms - 1) / num_sms;
+  nw = nw < 4 ? 4 : nw > 32 ? 32 : nw;
+  long g = (rows + nw - 1) / nw;
   if (g > num_sms) g = num_sms;
-  if (g < 1) g = 1;
-  if (cx) {
-    chol_smem_kernel<cplx><<<1, 256, shm, s>>>(k, rows, shift, scale, (const cplx*)G, (cplx*)L, dsc,
-                                                dead, err);
-    CTM_TRSM_LAUNCH(cplx);
-  } else {
-    chol_smem_kernel<double><<<1, 256, shm, s>>>(k, rows, shift, scale, (const double*)G, (double*)L,
-                                                  dsc, dead, err);
-    CTM_TRSM_LAUNCH(double);
-  }
-  if (launches) *launches += 2;
+  trsm_rows_kernel<T, R><<<(unsigned)g, (unsigned)(32 * nw), shm, s>>>(
+      rows, k, (const T*)L, dsc, (const T*)Z, (T*)Q, dead, seed);
   return cudaGetLastError();
+}
+
+// R = columns per lane: the smallest of 1, 2, 3, 4, 5, 6, 8 with 32 R >= k
+template <typename T>
+cudaError_t trsm_dispatch(int k, long rows, const void* L, const double* dsc, const void* Z,
+                          void* Q, const int* dead, uint64_t seed, int num_sms, cudaStream_t s) {
+  if (k <= 32) return launch_trsm<T, 1>(k, rows, L, dsc, Z, Q, dead, seed, num_sms, s);
+  if (k <= 64) return launch_trsm<T, 2>(k, rows, L, dsc, Z, Q, dead, seed, num_sms, s);
+  if (k <= 96) return launch_trsm<T, 3>(k, rows, L, dsc, Z, Q, dead, seed, num_sms, s);
+  if (k <= 128) return launch_trsm<T, 4>(k, rows, L, dsc, Z, Q, dead, seed, num_sms, s);
+  if (k <= 160) return launch_trsm<T, 5>(k, rows, L, dsc, Z, Q, dead, seed, num_sms, s);
+  if (k <= 192) return launch_trsm<T, 6>(k, rows, L, dsc, Z, Q, dead, seed, num_sms, s);
+  return launch_trsm<T, 8>(k, rows, L, dsc, Z, Q, dead, seed, num_sms, s);
 }
 
 cudaError_t trsm_rows(bool cx, int k, long rows, const void* L, const double* dsc, const void* Z,
-                      void* Q, int num_sms, cudaStream_t s, long* launches) {
-  const size_t shm = chol_smem_bytes(cx, k);
-  static size_t configured_trsm[2][5] = {{0}};
-  {
-    const cudaError_t e = cx ? trsm_set_smem<cplx>(configured_trsm[1], shm)
-                             : trsm_set_smem<double>(configured_trsm[0], shm);
-    if (e != cudaSuccess) return e;
-  }
-  long g = (rows + 31) / 32;
-  if (g > num_sms) g = num_sms;
-  if (g < 1) g = 1;
-  if (cx) CTM_TRSM_LAUNCH(cplx);
-  else CTM_TRSM_LAUNCH(double);
+                      void* Q, const int* dead, uint64_t seed, int num_sms, cudaStream_t s,
+                      long* launches) {
+  if (!trsm_rows_supported(cx, k)) return cudaErrorInvalidValue;
   if (launches) ++*launches;
-  return cudaGetLastError();
+  return cx ? trsm_dispatch<cplx>(k, rows, L, dsc, Z, Q, dead, seed, num_sms, s)
+            : trsm_dispatch<double>(k, rows, L, dsc, Z, Q, dead, seed, num_sms, s);
 }
 
-// W = D^-1 L^-H from the factor of chol_smem_kernel: block c solves the
-// column c of X = L^-1 by forward substitution (one warp, x in shared
-// memory) and writes row c of W, W[c][i] = conj(X[i][c]) / D_c (i >= c).
-template <typename T>
-__global__ void __launch_bounds__(32) trinv_kernel(int k, const T* L, const double* dsc, T* W) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* xs = reinterpret_cast<T*>(smem_raw);
-  const int c = blockIdx.x, lane = threadIdx.x;
-  for (int i = c; i < k; ++i) {
-    T acc = zero_of(T());
-    const T* Li = L + (size_t)i * k;
-    for (int l = c + lane; l < i; l += 32) fmav(acc, Li[l], xs[l]);
-    acc = warp_sum(acc);
-    if (lane == 0) {
-      const double inv = 1.0 / realv(Li[i]);
-      if (i == c) {
-        if constexpr (sizeof(T) == 8) xs[i] = inv;
-        else xs[i] = make_double2(inv, 0.0);
-      } else {
-        xs[i] = scalev(acc, -inv);
-      }
-    }
-    __syncwarp();
-  }
-  const double id = 1.0 / dsc[c];
-  for (int i = lane; i < k; i += 32)
-    W[(size_t)c * k + i] = i >= c ? scalev(conjv(xs[i]), id) : zero_of(T());
-}
-
-cudaError_t chol_factor_inv(bool cx, int k, long rows, bool shift, bool scale, const void* G,
-                            void* L, double* dsc, int* dead, void* W, int* err, cudaStream_t s,
-                            long* launches) {
-  const size_t shm = chol_smem_bytes(cx, k);
-  const cudaError_t e = chol_smem_prepare(cx, shm);
-  if (e != cudaSuccess) return e;
-  if (cx) {
-    chol_smem_kernel<cplx><<<1, 256, shm, s>>>(k, rows, shift, scale, (const cplx*)G, (cplx*)L,
-                                                dsc, dead, err);
-    trinv_kernel<cplx><<<k, 32, (size_t)k * sizeof(cplx), s>>>(k, (const cplx*)L, dsc, (cplx*)W);
-  } else {
-    chol_smem_kernel<double><<<1, 256, shm, s>>>(k, rows, shift, scale, (const double*)G,
-                                                  (double*)L, dsc, dead, err);
-    trinv_kernel<double><<<k, 32, (size_t)k * sizeof(double), s>>>(k, (const double*)L, dsc,
-                                                                    (double*)W);
-  }
-  if (launches) *launches += 2;
-  return cudaGetLastError();
-}
-
-cudaError_t repair_dead_columns(bool cx, long rows, int k, void* Q, const int* dead,
-                                uint64_t seed, cudaStream_t s, long* launches) {
-  if (cx) repair_kernel<cplx><<<grid_for(rows * k), 256, 0, s>>>(rows, k, (cplx*)Q, dead, seed);
-  else repair_kernel<double><<<grid_for(rows * k), 256, 0, s>>>(rows, k, (double*)Q, dead, seed);
+cudaError_t repair_dead_columns(bool cx, long rows, int k, const void* src, void* Q,
+                                const int* dead, uint64_t seed, cudaStream_t s, long* launches) {
+  if (cx)
+    repair_kernel<cplx><<<grid_for(rows * k), 256, 0, s>>>(rows, k, (const cplx*)src, (cplx*)Q,
+                                                           dead, seed);
+  else
+    repair_kernel<double><<<grid_for(rows * k), 256, 0, s>>>(rows, k, (const double*)src,
+                                                             (double*)Q, dead, seed);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
