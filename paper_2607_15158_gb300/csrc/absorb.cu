@@ -251,6 +251,145 @@ __global__ void __launch_bounds__(NG * GT * GT, ab_min_blocks<F, NG>())
   }
 }
 
+// The same contraction in fp64 (F = T), which the fp64 pipe bounds: a
+// multiply-add occupies a sub-partition for ~77 clocks however few lanes of
+// the warp take part, so no lane may idle and operand reads cost nothing
+// beside it. The outputs of NG pairs (t, n) are numbered through and dealt to
+// the warps 32 at a time, one output per lane and task, whatever D is; the
+// second product's outputs are numbered in the order of Out, so the results
+// go out from registers in runs of Dk Db. Register tiles of 3 x 3 on 12 x 12
+// threads, which compute 36 x 36 outputs whatever D is, took 605 us at real
+// D = 4, chi = 64 (150 here; 132 at the pipe's rate), 395 at complex D = 3,
+// chi = 33 (33 here), 75 at real D = 3, chi = 27 (11 here).
+constexpr int A64_THREADS = 256, A64_WARPS = A64_THREADS / 32;
+
+template <typename T, int MT>
+__global__ void __launch_bounds__(A64_THREADS)
+    absorb64_kernel(int chi, int Dk, int Db, int d, int ng, const T* __restrict__ In,
+                    const T* __restrict__ A, const T* __restrict__ B, T* __restrict__ Out) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int K1 = Dk * Dk, N1 = Db * Db, KN = K1 * N1, DD = Dk * Db;
+  T* As = reinterpret_cast<T*>(smem_raw);   // [d][(d,e)][(u,l)]
+  T* Bs = As + (size_t)d * K1 * K1;          // [d][(w,v)][(D,E)]
+  T* Xs = Bs + (size_t)d * N1 * N1;          // [pair][(u,l)][(w,v)]
+  T* Ys = Xs + (size_t)ng * KN;              // [pair][(d,e)][(w,v)]
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  for (int i = threadIdx.x; i < d * K1 * K1; i += A64_THREADS) {
+    // As[s][(d,e)][(u,l)] = A[s,u,l,d,e]
+    const int s = i / (K1 * K1), rem = i % (K1 * K1);
+    const int r = rem / K1, kk = rem % K1;
+    const int dd = r / Dk, e = r % Dk, u = kk / Dk, l = kk % Dk;
+    As[i] = A[(((size_t)(s * Dk + u) * Dk + l) * Dk + dd) * Dk + e];
+  }
+  for (int i = threadIdx.x; i < d * N1 * N1; i += A64_THREADS) {
+    // Bs[s][(w,v)][(D,E)] = B[s,v,w,D,E]
+    const int s = i / (N1 * N1), rem = i % (N1 * N1);
+    const int kk = rem / N1, c = rem % N1;
+    const int w = kk / Db, v = kk % Db, D = c / Db, E = c % Db;
+    Bs[i] = B[(((size_t)(s * Db + v) * Db + w) * Db + D) * Db + E];
+  }
+  const size_t row = (size_t)chi * DD;       // stride of the (first chi, Dk, Db) index
+  const long npairs = (long)chi * chi;
+  for (long p0 = (long)ng * blockIdx.x; p0 < npairs; p0 += (long)ng * gridDim.x) {
+    const int np = (int)min((long)ng, npairs - p0);
+    const int nout = np * KN;
+    for (int i = threadIdx.x; i < nout; i += A64_THREADS) {
+      // X[(u,l),(w,v)] = In[t,l,w,n,u,v]
+      const int pr = i / KN, ii = i % KN;
+      const long p = p0 + pr;
+      const int t = (int)(p / chi), n = (int)(p % chi);
+      const int lw = ii / DD, uv = ii % DD;
+      const int l = lw / Db, w = lw % Db, u = uv / Db, v = uv % Db;
+      Xs[(size_t)pr * KN + (u * Dk + l) * N1 + w * Db + v] =
+          In[((size_t)t * Dk + l) * Db * row + (size_t)w * row + (size_t)n * DD + uv];
+    }
+    T acc[MT];
+#pragma unroll
+    for (int m = 0; m < MT; ++m) acc[m] = zero_of(T());
+    for (int s = 0; s < d; ++s) {
+      __syncthreads();   // X loaded / previous Y consumed
+#pragma unroll
+      for (int m = 0; m < MT; ++m) {
+        const int t0 = 32 * (wp + A64_WARPS * m);
+        if (t0 >= nout) break;
+        const int o = min(t0 + lane, nout - 1);
+        const int pr = o / KN, r = o % KN / N1, c = o % N1;
+        const T* a = As + ((size_t)s * K1 + r) * K1;
+        const T* x = Xs + (size_t)pr * KN + c;
+        T y = zero_of(T());
+#pragma unroll 4
+        for (int kk = 0; kk < K1; ++kk) mac(y, a[kk], x[kk * N1]);
+        if (t0 + lane < nout) Ys[o] = y;
+      }
+      __syncthreads();
+#pragma unroll
+      for (int m = 0; m < MT; ++m) {
+        const int t0 = 32 * (wp + A64_WARPS * m);
+        if (t0 >= nout) break;
+        const int o = min(t0 + lane, nout - 1);
+        // output o = (pair, (d, D), (e, E)): row (d, e), column (D, E)
+        const int pr = o / KN, oo = o % KN, dD = oo / DD, eE = oo % DD;
+        const int r = dD / Db * Dk + eE / Db, c = dD % Db * Db + eE % Db;
+        const T* y = Ys + (size_t)pr * KN + r * N1;
+        const T* b = Bs + (size_t)s * N1 * N1 + c;
+#pragma unroll 4
+        for (int kk = 0; kk < N1; ++kk) mac(acc[m], y[kk], b[kk * N1]);
+      }
+    }
+#pragma unroll
+    for (int m = 0; m < MT; ++m) {
+      const int o = 32 * (wp + A64_WARPS * m) + lane;
+      if (o < nout) {
+        const int pr = o / KN, oo = o % KN, dD = oo / DD, eE = oo % DD;
+        const long p = p0 + pr;
+        const int t = (int)(p / chi), n = (int)(p % chi);
+        Out[((size_t)t * Dk * Db + dD) * row + (size_t)n * DD + eE] = acc[m];
+      }
+    }
+  }
+}
+
+size_t a64_smem(int Dk, int Db, int d, int ng, size_t tsize) {
+  const size_t K1 = (size_t)Dk * Dk, N1 = (size_t)Db * Db;
+  return ((size_t)d * K1 * K1 + (size_t)d * N1 * N1 + 2 * (size_t)ng * K1 * N1) * tsize;
+}
+
+template <typename T, int MT>
+cudaError_t launch_a64(int chi, int Dk, int Db, int d, int ng, const void* In, const void* A,
+                       const void* B, void* Out, int num_sms, cudaStream_t s) {
+  const size_t shm = a64_smem(Dk, Db, d, ng, sizeof(T));
+  static size_t configured = 0;
+  auto* fn = absorb64_kernel<T, MT>;
+  cudaError_t e = raise_smem((const void*)fn, configured, shm);
+  if (e != cudaSuccess) return e;
+  int per_sm = 0;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, A64_THREADS, shm);
+  if (e != cudaSuccess) return e;
+  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  const long tiles = ((long)chi * chi + ng - 1) / ng;
+  const long grid = std::min((long)num_sms * per_sm, tiles);
+  fn<<<(unsigned)grid, A64_THREADS, shm, s>>>(chi, Dk, Db, d, ng, static_cast<const T*>(In),
+                                              static_cast<const T*>(A), static_cast<const T*>(B),
+                                              static_cast<T*>(Out));
+  return cudaGetLastError();
+}
+
+// Pairs per block: as many as fill four tasks of every warp, while every SM
+// keeps two blocks' worth of them and they fit half its shared memory
+template <typename T>
+cudaError_t launch_absorb64(int chi, int Dk, int Db, int d, const void* In, const void* A,
+                            const void* B, void* Out, int num_sms, cudaStream_t s) {
+  const long kn = (long)Dk * Dk * Db * Db;
+  long ng = std::min(4L * A64_THREADS / kn, (long)chi * chi / (2L * num_sms));
+  ng = std::max(1L, ng);
+  while (ng > 1 && a64_smem(Dk, Db, d, (int)ng, sizeof(T)) > SMEM_MAX / 2) --ng;
+  const long tasks = (ng * kn + A64_THREADS - 1) / A64_THREADS;   // per warp
+  if (tasks <= 2) return launch_a64<T, 2>(chi, Dk, Db, d, (int)ng, In, A, B, Out, num_sms, s);
+  if (tasks <= 4) return launch_a64<T, 4>(chi, Dk, Db, d, (int)ng, In, A, B, Out, num_sms, s);
+  if (tasks <= 6) return launch_a64<T, 6>(chi, Dk, Db, d, (int)ng, In, A, B, Out, num_sms, s);
+  return launch_a64<T, 16>(chi, Dk, Db, d, (int)ng, In, A, B, Out, num_sms, s);
+}
+
 // shared memory of a geometry with ng groups: A and B, then X and Y per
 // group, then (staged) one raw input block per group
 size_t ab_smem(int Dk, int Db, int d, int ng, size_t fsize, size_t tsize, bool staged) {
@@ -262,11 +401,12 @@ size_t ab_smem(int Dk, int Db, int d, int ng, size_t fsize, size_t tsize, bool s
 
 // 0: no fused kernel; 3: 12 x 12 threads x 3 x 3 tiles, four groups with
 // staged input (fp32, D <= 6); 1: the same tiles, two groups; 2: 16 x 16
-// threads x 4 x 4 tiles, one group (D <= 8)
+// threads x 4 x 4 tiles, one group (D <= 8); 4: the fp64 kernel (D <= 8)
 int ab_geometry(int Dk, int Db, int d, size_t fsize, size_t tsize) {
   if (Dk < 1 || Db < 1 || d < 1) return 0;
   const int m = std::max(Dk * Dk, Db * Db);
-  if (m <= 36 && fsize < tsize && ab_smem(Dk, Db, d, 4, fsize, tsize, true) <= SMEM_MAX) return 3;
+  if (fsize == tsize) return m <= 64 && a64_smem(Dk, Db, d, 1, tsize) <= SMEM_MAX ? 4 : 0;
+  if (m <= 36 && ab_smem(Dk, Db, d, 4, fsize, tsize, true) <= SMEM_MAX) return 3;
   if (m <= 36 && ab_smem(Dk, Db, d, 2, fsize, tsize, false) <= SMEM_MAX) return 1;
   if (m <= 64 && ab_smem(Dk, Db, d, 1, fsize, tsize, false) <= SMEM_MAX) return 2;
   return 0;
@@ -296,18 +436,20 @@ cudaError_t launch_ab(int chi, int Dk, int Db, int d, const void* In, const void
 template <typename T, typename F>
 cudaError_t launch_geom(int geom, int chi, int Dk, int Db, int d, const void* In, const void* A,
                         const void* B, void* Out, int num_sms, cudaStream_t s) {
-  const bool sq = Dk == Db;
-  if constexpr (sizeof(F) < sizeof(T)) {
+  if constexpr (sizeof(F) == sizeof(T)) {
+    return launch_absorb64<T>(chi, Dk, Db, d, In, A, B, Out, num_sms, s);
+  } else {
+    const bool sq = Dk == Db;
     if (geom == 3 && sq && Dk == 6)
       return launch_ab<T, F, 12, 3, 4, true, 6>(chi, Dk, Db, d, In, A, B, Out, num_sms, s);
     if (geom == 3)
       return launch_ab<T, F, 12, 3, 4, true, 0>(chi, Dk, Db, d, In, A, B, Out, num_sms, s);
     if (geom == 2 && sq && Dk == 8)
       return launch_ab<T, F, 16, 4, 1, false, 8>(chi, Dk, Db, d, In, A, B, Out, num_sms, s);
+    if (geom == 1)
+      return launch_ab<T, F, 12, 3, 2, false, 0>(chi, Dk, Db, d, In, A, B, Out, num_sms, s);
+    return launch_ab<T, F, 16, 4, 1, false, 0>(chi, Dk, Db, d, In, A, B, Out, num_sms, s);
   }
-  if (geom == 1)
-    return launch_ab<T, F, 12, 3, 2, false, 0>(chi, Dk, Db, d, In, A, B, Out, num_sms, s);
-  return launch_ab<T, F, 16, 4, 1, false, 0>(chi, Dk, Db, d, In, A, B, Out, num_sms, s);
 }
 
 size_t elem_size(bool cx, bool fp32) { return (cx ? 2 : 1) * (fp32 ? 4 : 8); }
