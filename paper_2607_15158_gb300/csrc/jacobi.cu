@@ -110,8 +110,8 @@ __device__ __forceinline__ void stcg<double>(double* p, double v) { __stcg(p, v)
 template <>
 __device__ __forceinline__ void stcg<cplx>(cplx* p, cplx v) { __stcg(p, v); }
 
-__device__ __forceinline__ void st_release(unsigned* p, unsigned v) {
-  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+__device__ __forceinline__ void st_relaxed(unsigned* p, unsigned v) {
+  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
 // the warp waits until columns p and q (q < 0: none) have been through
@@ -257,41 +257,35 @@ __global__ void __launch_bounds__(JT) jacobi_coop(JacobiArgs a) {
             if (lane + 32 * e < k) fmacv(ga, xr[e], yr[e]);
           ga = warp_sum(ga);
           const double al = __ldcg(nsq + p), be = __ldcg(nsq + q);
-          // the rotation's scalars on lane 0 only, then broadcast: every
-          // fp64 instruction a whole warp executes costs the SM's narrow fp64
-          // pipe its full width
-          double gm = 0.0, tt = 0.0, c = 1.0, s = 0.0, ex = 0.0, ey = 0.0;
-          int rot = 0;
-          if (lane == 0) {
-            gm = sqrt(absq(ga));
-            const double nrm = sqrt(al) * sqrt(be);
-            // rotate when |gamma| > tol sqrt(alpha beta)
-            rot = gm > tol * nrm && gm != 0.0;
-            if (rot) {
+          // the rotation's scalars: every fp64 instruction costs the SM's
+          // narrow fp64 pipe the same for one lane as for 32 and the chain of
+          // square roots and divisions is what a round waits for, so the
+          // independent ones (the three roots; zeta, 1 / |gamma| and the
+          // ratio) are taken side by side in lanes 0, 1 and 2
+          double v = lane == 0 ? absq(ga) : lane == 1 ? al : be;
+          v = sqrt(v);
+          const double gm = __shfl_sync(0xffffffffu, v, 0);
+          const double nrm = __shfl_sync(0xffffffffu, v, 1) * __shfl_sync(0xffffffffu, v, 2);
+          // rotate when |gamma| > tol sqrt(alpha beta)
+          if (gm > tol * nrm && gm != 0.0) {
+            v = (lane == 0 ? be - al : lane == 1 ? 1.0 : gm) /
+                (lane == 0 ? 2.0 * gm : lane == 1 ? gm : nrm);
+            if (lane == 2)
               atomicMax(offb, (unsigned long long)__double_as_longlong(
-                                  nrm > 0.0 ? fmin(gm / nrm, 1.0) : 1.0));   // this sweep rotated
-              const double zeta = (be - al) / (2.0 * gm);
-              tt = copysign(1.0, zeta) / (fabs(zeta) + hypot(1.0, zeta));
-              c = 1.0 / hypot(1.0, tt);
-              s = c * tt;
-              // conj(gamma) / |gamma|
-              const double ig = 1.0 / gm;
-              if constexpr (sizeof(T) == 8) {
-                ex = ga * ig;
-              } else {
-                ex = ga.x * ig;
-                ey = -ga.y * ig;
-              }
+                                  nrm > 0.0 ? fmin(v, 1.0) : 1.0));   // this sweep rotated
+            const double zeta = __shfl_sync(0xffffffffu, v, 0);
+            const double ig = __shfl_sync(0xffffffffu, v, 1);
+            const double tt = copysign(1.0, zeta) / (fabs(zeta) + hypot(1.0, zeta));
+            const double c = 1.0 / hypot(1.0, tt);
+            const double s = c * tt;
+            // conj(gamma) / |gamma|
+            double ex = 0.0, ey = 0.0;
+            if constexpr (sizeof(T) == 8) {
+              ex = ga * ig;
+            } else {
+              ex = ga.x * ig;
+              ey = -ga.y * ig;
             }
-          }
-          rot = __shfl_sync(0xffffffffu, rot, 0);
-          if (rot) {
-            gm = __shfl_sync(0xffffffffu, gm, 0);
-            tt = __shfl_sync(0xffffffffu, tt, 0);
-            c = __shfl_sync(0xffffffffu, c, 0);
-            s = __shfl_sync(0xffffffffu, s, 0);
-            ex = __shfl_sync(0xffffffffu, ex, 0);
-            if constexpr (sizeof(T) == 16) ey = __shfl_sync(0xffffffffu, ey, 0);
             T eph;
             if constexpr (sizeof(T) == 8) eph = ex;
             else eph = make_double2(ex, ey);
@@ -328,12 +322,14 @@ __global__ void __launch_bounds__(JT) jacobi_coop(JacobiArgs a) {
             }
           }
         }
-        // publish: columns p and q have been through round rg
+        // publish: columns p and q have been through round rg (one fence, then
+        // relaxed stores: the release pattern; a releasing store would fence
+        // again for each)
         __syncwarp();
         if (lane == 0 && !dead) {
           __threadfence();
-          st_release(ver + p, rg + 1u);
-          if (real) st_release(ver + q, rg + 1u);
+          st_relaxed(ver + p, rg + 1u);
+          if (real) st_relaxed(ver + q, rg + 1u);
         }
       }
     }

@@ -10,13 +10,17 @@
 // cluster of two CTAs: CTA 0 holds A in shared memory and computes and
 // applies the rotations of each round; it writes their parameters into the
 // shared memory of CTA 1 (distributed shared memory), which holds V and
-// applies them one round behind. One cluster barrier separates the rounds.
+// applies them one batch of rounds behind. The rounds of a CTA are separated
+// by its own barrier (21 to 77 clocks by its size), batches of up to eight by
+// a cluster barrier (400 clocks); a CTA has eight threads per column pair and
+// no more, since its barrier grows with the threads.
 // The result V0 is accurate to the fp32 threshold; the caller makes it
 // unitary in fp64 and runs the fp64 sweeps on A V0, whose columns are then
 // orthogonal to ~1e-6 and converge in a few sweeps (quadratic convergence of
 // the cyclic method).
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <cfloat>
 
 #include "common.cuh"
@@ -28,11 +32,13 @@ namespace {
 
 namespace cg = cooperative_groups;
 
-constexpr int J32T = 1024;   // threads per CTA (32 warps)
-constexpr int J32G = J32T / 8;   // 8-lane groups per CTA (one column pair each)
+constexpr int J32T = 1024;   // most threads per CTA (32 warps)
+constexpr int J32G = J32T / 8;   // most 8-lane groups per CTA (one column pair each)
+constexpr int J32B = 8;          // most rounds per batch
 
 struct J32Args {
   int k, max_sweeps;
+  int rounds;       // rounds per batch
   const void* A;    // fp64 k x k row-major per matrix (stride strideA elements)
   long strideA;
   void* V0;         // fp64 k x k row-major per matrix (output)
@@ -99,7 +105,7 @@ __device__ __forceinline__ void apply_round(typename F32<CX>::T* M, const float4
                                             int kk, int m, int npairs, int t, int gi, int l8) {
   typedef F32<CX> E;
   typedef typename E::T T;
-  for (int pr = gi; pr < npairs; pr += J32G) {
+  for (int pr = gi; pr < npairs; pr += blockDim.x / 8) {
     int p = player32(pr, t, m), q = player32(kk - 1 - pr, t, m);
     if (p > q) {
       const int tmp = p;
@@ -134,7 +140,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(J32T, 1)
   extern __shared__ __align__(16) unsigned char smem[];
   T* M = reinterpret_cast<T*>(smem);   // A (rank 0) or V (rank 1), column c at M[c k]
   const size_t mbytes = ((size_t)k * k * sizeof(T) + 15) & ~(size_t)15;
-  float4* prm = reinterpret_cast<float4*>(smem + mbytes);   // [2][npairs] (c, s, e)
+  float4* prm = reinterpret_cast<float4*>(smem + mbytes);   // [2][rounds][npairs] (c, s, e)
   __shared__ int rotated, stop;
   __shared__ unsigned long long amax;   // bits of max |a_ij| (non-negative doubles order as integers)
   const int lane = threadIdx.x & 31;
@@ -155,7 +161,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(J32T, 1)
     // the entries in range
     double mx = 0.0;
     const double* Ad = static_cast<const double*>(Ab);
-    for (long idx = threadIdx.x; idx < (long)k * k * (CX ? 2 : 1); idx += J32T)
+    for (long idx = threadIdx.x; idx < (long)k * k * (CX ? 2 : 1); idx += blockDim.x)
       mx = fmax(mx, fabs(Ad[idx]));
     for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     if (lane == 0 && mx > 0.0 && isfinite(mx))
@@ -163,12 +169,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(J32T, 1)
     __syncthreads();
     const double mxa = __longlong_as_double((long long)amax);
     const double sc = mxa > 0.0 ? ldexp(1.0, -ilogb(mxa)) : 1.0;
-    for (long idx = threadIdx.x; idx < (long)k * k; idx += J32T) {
+    for (long idx = threadIdx.x; idx < (long)k * k; idx += blockDim.x) {
       const int r = (int)(idx / k), c = (int)(idx % k);
       M[(size_t)c * k + r] = E::load64s(Ab, idx, sc);
     }
   } else {
-    for (long idx = threadIdx.x; idx < (long)k * k; idx += J32T) {
+    for (long idx = threadIdx.x; idx < (long)k * k; idx += blockDim.x) {
       const int r = (int)(idx / k), c = (int)(idx % k);
       M[(size_t)c * k + r] = r == c ? E::one() : E::zero();
     }
@@ -180,62 +186,77 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(J32T, 1)
   // of a length-k dot product
   const float tol = fmaxf(1e-6f, 2.f * sqrtf((float)k) * FLT_EPSILON);
   int sweep = 0;
-  long g = 0;   // rounds done (all sweeps)
+  int par = 0;             // parity of the current batch
+  int bt0 = 0, bn = 0;     // CTA 1: first round and size of the batch to apply
+  // CTA 1: V <- V J for the previous batch's rounds (a barrier after each)
+  auto apply_batch = [&]() {
+    for (int i = 0; i < bn; ++i) {
+      apply_round<CX>(M, prm + (size_t)((par ^ 1) * a.rounds + i) * npairs, k, kk, m, npairs,
+                      bt0 + i, gi, l8);
+      __syncthreads();
+    }
+  };
   for (; sweep < a.max_sweeps; ++sweep) {
-    for (int t = 0; t < m; ++t, ++g) {
+    for (int t0 = 0; t0 < m; t0 += a.rounds) {
+      const int n = min(a.rounds, m - t0);
       if (rank == 0) {
-        for (int pr = gi; pr < npairs; pr += J32G) {
-          int p = player32(pr, t, m), q = player32(kk - 1 - pr, t, m);
-          if (p > q) {
-            const int tmp = p;
-            p = q;
-            q = tmp;
-          }
-          float4 rp = make_float4(1.f, 0.f, 1.f, 0.f);   // identity
-          if (q < k) {
-            T* x = M + (size_t)p * k;
-            T* y = M + (size_t)q * k;
-            // exact squared norms and the overlap of the pair, every round
-            float2 ga = make_float2(0.f, 0.f);
-            float al = 0.f, be = 0.f;
-            #pragma unroll 4
-            for (int r = l8; r < k; r += 8) {
-              const T xv = x[r], yv = y[r];
-              al += E::nrm2(xv);
-              be += E::nrm2(yv);
-              E::dotc(ga, xv, yv);
+        for (int i = 0; i < n; ++i) {
+          const int t = t0 + i;
+          for (int pr = gi; pr < npairs; pr += blockDim.x / 8) {
+            int p = player32(pr, t, m), q = player32(kk - 1 - pr, t, m);
+            if (p > q) {
+              const int tmp = p;
+              p = q;
+              q = tmp;
             }
-#pragma unroll
-            for (int o = 4; o > 0; o >>= 1) {
-              al += __shfl_xor_sync(m8, al, o);
-              be += __shfl_xor_sync(m8, be, o);
-              ga.x += __shfl_xor_sync(m8, ga.x, o);
-              if (CX) ga.y += __shfl_xor_sync(m8, ga.y, o);
-            }
-            const float gm = sqrtf(ga.x * ga.x + ga.y * ga.y);
-            if (gm > tol * sqrtf(al) * sqrtf(be) && gm > 0.f) {
-              const float zeta = (be - al) / (2.f * gm);
-              const float tt = copysignf(1.f, zeta) / (fabsf(zeta) + sqrtf(1.f + zeta * zeta));
-              const float c = 1.f / sqrtf(1.f + tt * tt), s = c * tt;
-              const float2 e = make_float2(ga.x / gm, -ga.y / gm);   // conj(gamma) / |gamma|
+            float4 rp = make_float4(1.f, 0.f, 1.f, 0.f);   // identity
+            if (q < k) {
+              T* x = M + (size_t)p * k;
+              T* y = M + (size_t)q * k;
+              // exact squared norms and the overlap of the pair, every round
+              float2 ga = make_float2(0.f, 0.f);
+              float al = 0.f, be = 0.f;
               #pragma unroll 4
               for (int r = l8; r < k; r += 8) {
-                T xv = x[r], yv = y[r];
-                E::rot(xv, yv, c, s, e);
-                x[r] = xv;
-                y[r] = yv;
+                const T xv = x[r], yv = y[r];
+                al += E::nrm2(xv);
+                be += E::nrm2(yv);
+                E::dotc(ga, xv, yv);
               }
-              rp = make_float4(c, s, e.x, e.y);
-              if (l8 == 0) rotated = 1;
+#pragma unroll
+              for (int o = 4; o > 0; o >>= 1) {
+                al += __shfl_xor_sync(m8, al, o);
+                be += __shfl_xor_sync(m8, be, o);
+                ga.x += __shfl_xor_sync(m8, ga.x, o);
+                if (CX) ga.y += __shfl_xor_sync(m8, ga.y, o);
+              }
+              const float gm = sqrtf(ga.x * ga.x + ga.y * ga.y);
+              if (gm > tol * sqrtf(al) * sqrtf(be) && gm > 0.f) {
+                const float zeta = (be - al) / (2.f * gm);
+                const float tt = copysignf(1.f, zeta) / (fabsf(zeta) + sqrtf(1.f + zeta * zeta));
+                const float c = 1.f / sqrtf(1.f + tt * tt), s = c * tt;
+                const float2 e = make_float2(ga.x / gm, -ga.y / gm);   // conj(gamma) / |gamma|
+                #pragma unroll 4
+                for (int r = l8; r < k; r += 8) {
+                  T xv = x[r], yv = y[r];
+                  E::rot(xv, yv, c, s, e);
+                  x[r] = xv;
+                  y[r] = yv;
+                }
+                rp = make_float4(c, s, e.x, e.y);
+                if (l8 == 0) rotated = 1;
+              }
             }
+            if (l8 == 0) prm1[(size_t)(par * a.rounds + i) * npairs + pr] = rp;
           }
-          if (l8 == 0) prm1[(g & 1) * npairs + pr] = rp;
+          __syncthreads();
         }
-      } else if (g > 0) {
-        // V <- V J for the rotations of the previous round
-        const long g1 = g - 1;
-        apply_round<CX>(M, prm + (g1 & 1) * npairs, k, kk, m, npairs, (int)(g1 % m), gi, l8);
+      } else {
+        apply_batch();
       }
+      bt0 = t0;
+      bn = n;
+      par ^= 1;
       cl.sync();
     }
     // a sweep without rotations ends the iteration (decided by CTA 0)
@@ -252,12 +273,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(J32T, 1)
     }
   }
   if (rank == 1) {
-    if (g > 0) {
-      const long g1 = g - 1;
-      apply_round<CX>(M, prm + (g1 & 1) * npairs, k, kk, m, npairs, (int)(g1 % m), gi, l8);
-    }
+    apply_batch();
     __syncthreads();
-    for (long idx = threadIdx.x; idx < (long)k * k; idx += J32T) {
+    for (long idx = threadIdx.x; idx < (long)k * k; idx += blockDim.x) {
       const int r = (int)(idx / k), c = (int)(idx % k);
       E::store64(a.V0, (size_t)b * k * k + idx, M[(size_t)c * k + r]);
     }
@@ -267,21 +285,24 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(J32T, 1)
   cl.sync();
 }
 
-size_t j32_smem(bool cx, int k) {
+size_t j32_smem(bool cx, int k, int rounds) {
   const int npairs = (k + (k & 1)) / 2;
-  return (((size_t)k * k * (cx ? 8 : 4) + 15) & ~(size_t)15) + 2 * (size_t)npairs * 16;
+  return (((size_t)k * k * (cx ? 8 : 4) + 15) & ~(size_t)15) + 2 * (size_t)rounds * npairs * 16;
 }
 
 }  // namespace
 
 bool jacobi32_supported(bool cx, int k) {
-  return k >= 2 && (k + 1) / 2 <= J32G && j32_smem(cx, k) <= (size_t)227 * 1024;
+  return k >= 2 && (k + 1) / 2 <= J32G && j32_smem(cx, k, 1) <= (size_t)227 * 1024;
 }
 
 cudaError_t jacobi32_presolve(bool cx, int k, const void* A, long strideA, void* V0, int batch,
                               int max_sweeps, int* sweeps, cudaStream_t s, long* launches) {
   if (!jacobi32_supported(cx, k) || batch < 1) return cudaErrorInvalidValue;
-  const size_t shm = j32_smem(cx, k);
+  int rounds = J32B;   // as many rounds per batch as the parameters' room allows
+  while (rounds > 1 && j32_smem(cx, k, rounds) > (size_t)227 * 1024) --rounds;
+  const size_t shm = j32_smem(cx, k, rounds);
+  const int threads = std::max(128, ((k + 1) / 2 * 8 + 31) / 32 * 32);
   static size_t configured[2] = {0, 0};
   const void* fn = cx ? (const void*)jacobi32_kernel<true> : (const void*)jacobi32_kernel<false>;
   cudaError_t e = raise_smem(fn, configured[cx ? 1 : 0], shm);
@@ -289,12 +310,13 @@ cudaError_t jacobi32_presolve(bool cx, int k, const void* A, long strideA, void*
   J32Args a;
   a.k = k;
   a.max_sweeps = max_sweeps;
+  a.rounds = rounds;
   a.A = A;
   a.strideA = strideA;
   a.V0 = V0;
   a.sweeps = sweeps;
-  if (cx) jacobi32_kernel<true><<<2 * batch, J32T, shm, s>>>(a);
-  else jacobi32_kernel<false><<<2 * batch, J32T, shm, s>>>(a);
+  if (cx) jacobi32_kernel<true><<<2 * batch, threads, shm, s>>>(a);
+  else jacobi32_kernel<false><<<2 * batch, threads, shm, s>>>(a);
   if (launches) ++*launches;
   return cudaGetLastError();
 }
