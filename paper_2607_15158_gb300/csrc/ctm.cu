@@ -123,6 +123,7 @@ ctm_status dalloc(ctm_ctx* c, void** p, size_t bytes) {
       if (g_fail_alloc_after.compare_exchange_weak(left, left - 1)) {
         if (left == 0) {
           *p = nullptr;
+          c->alloc_injected = true;
           return fail(c, CTM_ENOMEM, "device allocation failed (injected by ctm_debug_fail_alloc)");
         }
         break;
@@ -166,10 +167,8 @@ void* BRAp(ctm_ctx* c, int rot, int site) { return at(c->bra[rot & 3], (size_t)s
 void* fC(ctm_ctx* c, int r, int i, int x, int y) { return Cp(c, frame_label(r, i), frame_site(c, r, x, y)); }
 void* fT(ctm_ctx* c, int r, int i, int x, int y) { return Tp(c, frame_label(r, i), frame_site(c, r, x, y)); }
 
-// Point the per-cut workspace fields of c at lane i (see ctm_ctx::Lane).
-void use_lane(ctm_ctx* c, int i) {
-  if (c->lanes.empty() || i == c->cur_lane) return;
-  const ctm_ctx::Lane& L = c->lanes[i];
+// Point the per-cut workspace fields of c at a lane (see ctm_ctx::Lane).
+void point_at(ctm_ctx* c, const ctm_ctx::Lane& L) {
   c->stream = L.stream;
   for (int q = 0; q < 4; ++q) c->Q[q] = L.Q[q];
   c->pipe[0] = L.pipe[0];
@@ -189,8 +188,48 @@ void use_lane(ctm_ctx* c, int i) {
   c->Vs = L.Vs;
   c->Us = L.Us;
   c->ph = L.ph;
+}
+void use_lane(ctm_ctx* c, int i) {
+  if (c->lanes.empty() || i == c->cur_lane) return;
+  point_at(c, c->lanes[i]);
   c->cur_lane = i;
 }
+void use_helper(ctm_ctx* c, int i) {
+  point_at(c, c->helpers[i]);
+  c->cur_lane = -1 - i;
+}
+
+// The W half of a cut beside its X half: from a fork on, w() points c at the
+// helper of the cut's lane and x() back at the lane; join() makes the lane wait
+// for the helper. Without a helper all of it runs on the lane.
+struct Halves {
+  ctm_ctx* c;
+  int lane;
+  bool on;
+  Halves(ctm_ctx* c_, bool want) : c(c_), lane(c_->cur_lane), on(want && !c_->helpers.empty()) {}
+  ctm_status fork() {
+    if (!on) return CTM_OK;
+    const ctm_ctx::Lane &L = c->lanes[lane], &H = c->helpers[lane];
+    if (H.split) split_borrow_corners(H.split, L.split);
+    CTM_CUDA_OK(cudaEventRecord(L.ev, L.stream));
+    CTM_CUDA_OK(cudaStreamWaitEvent(H.stream, L.ev, 0));
+    return CTM_OK;
+  }
+  ctm_status join() {
+    if (!on) return CTM_OK;
+    const ctm_ctx::Lane &L = c->lanes[lane], &H = c->helpers[lane];
+    CTM_CUDA_OK(cudaEventRecord(H.ev, H.stream));
+    CTM_CUDA_OK(cudaStreamWaitEvent(L.stream, H.ev, 0));
+    use_lane(c, lane);
+    return CTM_OK;
+  }
+  void x() {
+    if (on) use_lane(c, lane);
+  }
+  void w() {
+    if (on) use_helper(c, lane);
+  }
+};
 
 // returns c to lane 0 when a move leaves early
 struct LaneReset {
@@ -616,9 +655,14 @@ ctm_status si_rho(ctm_ctx* c, int r, int cut, int y) {
                                 cudaMemcpyDeviceToDevice, c->stream));
     ready = 0;
   }
+  // the coupled update alternates between X and W: nothing runs side by side
+  Halves half(c, !c->opts.si_coupled);
+  CK(half.fork());
   if (!ready) {
     CK(qr_inplace(c, X, Z[0], false));
+    half.w();
     CK(qr_inplace(c, W, Z[0], false));
+    half.x();
     ready = 1;
   }
   const int rc = r * c->S + cut;
@@ -668,6 +712,7 @@ ctm_status si_rho(ctm_ctx* c, int r, int cut, int y) {
     CK(apply_corner(c, Q[1], true, Z[0], X));
     CK(qr_inplace(c, X, Z[0], split_qr));
     // W <- qr(M qr(M^H W))
+    half.w();
     CK(apply_corner(c, Q[2], true, W, Z[0]));
     CK(apply_corner(c, Q[3], true, Z[0], Z[1]));
     CK(apply_corner(c, Q[0], true, Z[1], Z[0]));
@@ -678,6 +723,7 @@ ctm_status si_rho(ctm_ctx* c, int r, int cut, int y) {
     CK(apply_corner(c, Q[3], false, Z[2], Z[0]));
     CK(apply_corner(c, Q[2], false, Z[0], W));
     CK(qr_inplace(c, W, Z[0], split_qr));
+    half.x();
   }
   if (track && rounds > 0) {
     // overlap of the bases before and after the update, for the principal
@@ -691,8 +737,10 @@ ctm_status si_rho(ctm_ctx* c, int r, int cut, int y) {
   void* ZL = at(c->ZL, y * Nk, c);
   CK(apply_corner(c, Q[1], false, X, Z[0]));
   CK(apply_corner(c, Q[0], false, Z[0], ZR));
+  half.w();
   CK(apply_corner(c, Q[2], true, W, Z[0]));
   CK(apply_corner(c, Q[3], true, Z[0], ZL));
+  CK(half.join());
   const int k = c->k;
   const int opH = c->cx ? OP_C : OP_T;
   PhaseScope ps(c, PH_SMALL);
@@ -782,19 +830,19 @@ ctm_status si_finish(ctm_ctx* c, int r, int cut, int y, void* Pl, void* PrH) {
     CTM_CUDA_OK(scale_columns_conj(c->cx, k, k, k, u, c->ph, c->stream, &c->launches));
     CTM_CUDA_OK(scale_columns_conj(c->cx, k, k, k, v, c->ph, c->stream, &c->launches));
   }
-  // recycled bases X v, W u: the next update re-orthonormalises them, so in
-  // split contexts they run on the tensor cores
-  if (c->split && !c->exact) {
-    ctm_status st = split_gemm(c->split, OP_N, X, k, OP_N, v, k, (int)c->N, k, k, c->Xn, k,
-                               c->stream, &c->launches);
-    if (st == CTM_OK)
-      st = split_gemm(c->split, OP_N, W, k, OP_N, u, k, (int)c->N, k, k, c->Wn, k, c->stream,
-                      &c->launches);
-    if (st != CTM_OK) return fail(c, st, split_last_error(c->split));
-  } else {
-    CK(mm_small(c, OP_N, OP_N, c->N, k, k, X, k, v, k, c->Xn, k));
-    CK(mm_small(c, OP_N, OP_N, c->N, k, k, W, k, u, k, c->Wn, k));
-  }
+  Halves half(c, true);
+  CK(half.fork());
+  // recycled bases X v, W u (the next update re-orthonormalises them, so in
+  // split contexts they run on the tensor cores) and the projectors
+  auto recycled = [&](void* X0, const void* r0, void* out) -> ctm_status {
+    if (c->split && !c->exact) {
+      const ctm_status st = split_gemm(c->split, OP_N, X0, k, OP_N, r0, k, (int)c->N, k, k, out, k,
+                                       c->stream, &c->launches);
+      return st == CTM_OK ? CTM_OK : fail(c, st, split_last_error(c->split));
+    }
+    return mm_small(c, OP_N, OP_N, c->N, k, k, X0, k, r0, k, out, k);
+  };
+  CK(recycled(X, v, c->Xn));
   if (c->opts.recycle_sin2 > 0.0) {
     // mean sin^2 of the principal angles between the leading chi-subspaces
     // of the bases before (X_old) and after (X_upd v) this move:
@@ -810,12 +858,15 @@ ctm_status si_finish(ctm_ctx* c, int r, int cut, int y, void* Pl, void* PrH) {
   }
   CTM_CUDA_OK(scale_by_inv_sqrt(c->cx, k, chi, v, sv, c->opts.svd_rel_cutoff, c->Vs,
                                 c->stream, &c->launches));
+  CK(mm_exact(c, OP_N, OP_N, c->N, chi, k, ZR, k, c->Vs, chi, Pl, chi));
+  CTM_CUDA_OK(cudaMemcpyAsync(X, c->Xn, Nk * c->es, cudaMemcpyDeviceToDevice, c->stream));
+  half.w();
+  CK(recycled(W, u, c->Wn));
   CTM_CUDA_OK(scale_by_inv_sqrt(c->cx, k, chi, u, sv, c->opts.svd_rel_cutoff, c->Us,
                                 c->stream, &c->launches));
-  CK(mm_exact(c, OP_N, OP_N, c->N, chi, k, ZR, k, c->Vs, chi, Pl, chi));
   CK(mm_exact(c, OP_N, OP_N, c->N, chi, k, ZL, k, c->Us, chi, PrH, chi));
-  CTM_CUDA_OK(cudaMemcpyAsync(X, c->Xn, Nk * c->es, cudaMemcpyDeviceToDevice, c->stream));
   CTM_CUDA_OK(cudaMemcpyAsync(W, c->Wn, Nk * c->es, cudaMemcpyDeviceToDevice, c->stream));
+  CK(half.join());
   return CTM_OK;
 }
 
@@ -1215,6 +1266,57 @@ ctm_status update_recycling(ctm_ctx* c) {
   return CTM_OK;
 }
 
+void destroy_helpers(ctm_ctx* c) {
+  for (auto& H : c->helpers) {
+    if (H.split) split_destroy(H.split);
+    if (H.ev) cudaEventDestroy(H.ev);
+    if (H.stream) cudaStreamDestroy(H.stream);
+  }
+  c->helpers.clear();
+}
+
+// scratch of a helper: the partial sums of a tall-skinny fp64 product
+size_t helper_scratch(size_t N) { return N >= 4096 ? (size_t)16 << 20 : (size_t)64 << 10; }
+
+// Helpers of the lanes that run cuts. A context runs without them, one half of
+// a cut after the other, when the device has no room for them.
+ctm_status create_helpers(ctm_ctx* c) {
+  const size_t N = c->N, k = c->k, chi = c->chi, es = c->es, mark = c->allocs.size();
+  const int nl = (int)c->lanes.size();
+  c->helpers.resize(nl);
+  ctm_status st = CTM_OK;
+  for (int l = nl > 1 ? 1 : 0; l < nl && st == CTM_OK; ++l) {
+    ctm_ctx::Lane& H = c->helpers[l];
+    for (int q = 0; q < 4; ++q) H.Q[q] = c->lanes[l].Q[q];
+    if (cudaStreamCreateWithFlags(&H.stream, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&H.ev, cudaEventDisableTiming) != cudaSuccess)
+      return fail(c, CTM_ECUDA, "helper stream creation failed");
+    H.scratch_bytes = helper_scratch(N);
+    auto al = [&](auto& p, size_t bytes) {
+      if (st == CTM_OK) st = dalloc(c, (void**)&p, bytes);
+    };
+    al(H.scratch, H.scratch_bytes);
+    for (int q = 0; q < 3; ++q) al(H.Z[q], N * k * es);
+    al(H.G, k * k * es);
+    al(H.Linv, k * k * es);
+    al(H.dsc, k * sizeof(double));
+    al(H.dead, k * sizeof(int));
+    al(H.chol_work, chol_coop_work_bytes((int)k, 1));
+    al(H.Wn, N * k * es);
+    al(H.Us, k * chi * es);
+    if (st == CTM_OK && c->opts.prec != CTM_PREC_FP64 &&
+        split_create(&H.split, c->cx, c->opts.prec == CTM_PREC_SPLIT_TF32, (int)N, (int)k, c->err,
+                     H.stream) != CTM_OK)
+      return fail(c, CTM_ECUDA, "split-precision setup failed");
+  }
+  if (st != CTM_ENOMEM || c->alloc_injected) return st;
+  for (size_t i = mark; i < c->allocs.size(); ++i) cudaFree(c->allocs[i]);
+  c->allocs.resize(mark);
+  destroy_helpers(c);
+  c->msg.clear();
+  return CTM_OK;
+}
+
 ctm_status create(ctm_ctx** out, int Lx, int Ly, int d, int Dk, int Db, int chi, bool cx,
                   const ctm_opts* opts, const void* const* kets, const void* const* bras,
                   bool classical) {
@@ -1467,6 +1569,9 @@ ctm_status create(ctm_ctx** out, int Lx, int Ly, int d, int Dk, int Db, int chi,
       }
     }
   }
+  if (c->opts.method == CTM_PROJ_SI && !c->opts.si_coupled &&
+      (st = create_helpers(c)) != CTM_OK)
+    return bail(st);
   if (c->opts.method == CTM_PROJ_SVD) {
     st = svd_create(&c->svd, cx, (int)N, chi);
     if (st != CTM_OK) {
@@ -1740,7 +1845,17 @@ static size_t footprint_bytes(int Lx, int Ly, int d, int Dk, int Db, int chi, bo
       lane += 10 * N * Kp * sb + split_partial_splits(N, cx) * N * ((cx ? 2 : 1) * k + 160) * 4;
     }
     lane += oz_refine;
-    b += (size_t)(lanes_for(Lx, Ly) - 1) * lane;
+    const int nl = lanes_for(Lx, Ly);
+    b += (size_t)(nl - 1) * lane;
+    if (!o->si_coupled) {
+      // helpers of the lanes that run cuts: blocks, QR work, split state
+      size_t help = helper_scratch(N) + 4 * N * k * es + 2 * k * k * es + k * chi * es + 12 * k +
+                    chol_coop_work_bytes((int)k, 1) + ((size_t)1 << 20);
+      if (o->prec != CTM_PREC_FP64)
+        help += split_partial_splits(N, cx) * N * ((cx ? 2 : 1) * k + 160) * 4 + 40 * N * k * es;
+      if (refine) help += 4 * NN * es;
+      b += (size_t)std::max(1, nl - 1) * help;
+    }
   }
   return b + b / 20 + ((size_t)64 << 20);
 }
@@ -2313,6 +2428,16 @@ ctm_status ctm_last_timing(const ctm_ctx* c, double* ms, long* launches) {
   return CTM_OK;
 }
 
+// split-precision states of the lanes and helpers
+static std::vector<SplitCtx*> split_states(const ctm_ctx* c) {
+  std::vector<SplitCtx*> v;
+  if (c->lanes.empty()) v.push_back(c->split);
+  for (const auto& L : c->lanes) v.push_back(L.split);
+  for (const auto& H : c->helpers)
+    if (H.split) v.push_back(H.split);
+  return v;
+}
+
 ctm_status ctm_profile_enable(ctm_ctx* c, int on) {
   if (!c) return CTM_EINVAL;
   Guard gd(c);
@@ -2326,8 +2451,7 @@ ctm_status ctm_profile_enable(ctm_ctx* c, int on) {
   c->pev_used = 0;
   for (double& v : c->phase_ms) v = 0.0;
   if (!c->split) return CTM_OK;
-  for (size_t l = 0; l < std::max<size_t>(1, c->lanes.size()); ++l) {
-    SplitCtx* sp = c->lanes.empty() ? c->split : c->lanes[l].split;
+  for (SplitCtx* sp : split_states(c)) {
     const ctm_status st = split_profile(sp, on ? 1 : 0, nullptr, nullptr, nullptr, nullptr);
     if (st != CTM_OK) return fail(c, st, split_last_error(sp));
   }
@@ -2341,8 +2465,7 @@ ctm_status ctm_profile_read(ctm_ctx* c, double* ms, long* launches, double* flop
   Guard gd(c);
   double tms = 0, tfl = 0, tby = 0;
   long tl = 0;
-  for (size_t l = 0; l < std::max<size_t>(1, c->lanes.size()); ++l) {
-    SplitCtx* sp = c->lanes.empty() ? c->split : c->lanes[l].split;
+  for (SplitCtx* sp : split_states(c)) {
     double m = 0, f = 0, b = 0;
     long n = 0;
     const ctm_status st = split_profile(sp, -1, &m, &n, &f, &b);
@@ -2370,7 +2493,10 @@ void ctm_free(ctm_ctx* c) {
   grad_destroy(c);
   for (auto& L : c->lanes)
     if (L.stream) cudaStreamSynchronize(L.stream);
+  for (auto& H : c->helpers)
+    if (H.stream) cudaStreamSynchronize(H.stream);
   if (c->stream) cudaStreamSynchronize(c->stream);
+  destroy_helpers(c);
   for (auto& e : c->pev) cudaEventDestroy(e);
   if (c->stream) cudaStreamSynchronize(c->stream);
   if (c->split) split_destroy(c->split);

@@ -152,7 +152,13 @@ struct ctm_ctx {
     void* ph = nullptr;
   };
   std::vector<Lane> lanes;   // lane 0 = the context's own buffers and stream
-  int cur_lane = 0;
+  int cur_lane = 0;          // -1 - i: the helper of lane i
+  // helper of a lane that runs cuts: the W half of a cut's subspace iteration
+  // and projector step (independent of the X half but for the corners) on its
+  // own stream, with the lane's corners and its own blocks and QR work. Empty
+  // when the device had no room for them: then both halves run on the lane.
+  std::vector<Lane> helpers; // one per lane (those of lanes without cuts unused)
+  bool alloc_injected = false;   // the last allocation failure was injected
   // standard truncated-SVD projectors (CTM_PROJ_SVD)
   SvdCtx* svd = nullptr;
   void* svdM = nullptr;      // N x N
@@ -208,6 +214,7 @@ void* Tp(ctm_ctx* c, int label, int site);
 void* KETp(ctm_ctx* c, int rot, int site);
 void* BRAp(ctm_ctx* c, int rot, int site);
 void use_lane(ctm_ctx* c, int i);
+void use_helper(ctm_ctx* c, int i);
 void* scratch_alloc(ctm_ctx* c, size_t bytes);
 // out = contraction of A and B given as an einsum spec (no batch or traced
 // labels): at most one permute per operand, one GEMM, one permute of out

@@ -1030,6 +1030,7 @@ struct SplitCtx {
   void* corner_src[4] = {nullptr};
   void* cslices[4][2] = {{nullptr}};
   int corner_Kp = 0;
+  bool borrowed = false;    // cslices belong to another context
   // generic operand buffers (grown on demand)
   void* abuf = nullptr;
   size_t abuf_bytes = 0;
@@ -1273,7 +1274,7 @@ ctm_status split_profile(SplitCtx* sc, int on, double* ms, long* launches, doubl
 void split_destroy(SplitCtx* sc) {
   if (!sc) return;
   for (auto& e : sc->ev) cudaEventDestroy(e);
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < 4 && !sc->borrowed; ++i)
     for (int o = 0; o < 2; ++o)
       if (sc->cslices[i][o]) cudaFree(sc->cslices[i][o]);
   if (sc->abuf) cudaFree(sc->abuf);
@@ -1307,6 +1308,15 @@ ctm_status split_prepare_corners(SplitCtx* sc, void* const* Q, int N, unsigned m
     }
   }
   return CTM_OK;
+}
+
+void split_borrow_corners(SplitCtx* sc, const SplitCtx* src) {
+  sc->borrowed = true;
+  sc->corner_Kp = src->corner_Kp;
+  for (int i = 0; i < 4; ++i) {
+    sc->corner_src[i] = src->corner_src[i];
+    for (int o = 0; o < 2; ++o) sc->cslices[i][o] = src->cslices[i][o];
+  }
 }
 
 ctm_status split_apply(SplitCtx* sc, const void* Q, bool herm, const void* Zin, void* Zout, int N,

@@ -24,6 +24,10 @@ void split_destroy(SplitCtx* sc);
 ctm_status split_prepare_corners(SplitCtx* sc, void* const* Q, int N, unsigned mask,
                                  cudaStream_t s, long* launches);
 
+// Let sc apply the corners that src has prepared (and will prepare again): the
+// slices stay src's, and the caller orders their use.
+void split_borrow_corners(SplitCtx* sc, const SplitCtx* src);
+
 // Zout = op(Q) Zin for one of the prepared corners (identified by pointer),
 // Zin, Zout fp64 N x k row-major.
 ctm_status split_apply(SplitCtx* sc, const void* Q, bool herm, const void* Zin, void* Zout,
