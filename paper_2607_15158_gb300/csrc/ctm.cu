@@ -1124,6 +1124,13 @@ ctm_status move_impl(ctm_ctx* c, int r) {
 ctm_status corner_spectra(ctm_ctx* c, double* out) {
   PhaseScope ps(c, PH_SPECTRA);
   // unnormalised singular values of all 4 S corners, [label][site][chi]
+  if (jacobi_vals_supported(c->cx, c->chi)) {
+    // (the fp32 pre-solve of the other path has a budget of 40 sweeps of its own)
+    CTM_CUDA_OK(jacobi_vals(c->cx, c->chi, c->C, (long)elems_C(c), out, 4 * (int)c->S,
+                            c->opts.svd_max_sweeps + (c->opts.svd_presolve ? 40 : 0), c->err,
+                            c->stream, &c->launches));
+    return CTM_OK;
+  }
   const void* A = c->C;
   long sA = (long)elems_C(c);
   if (use_presolve(c, c->chi)) {
@@ -2054,9 +2061,13 @@ ctm_status ctm_spectrum(ctm_ctx* c, int x, int y, int label, double* s_out) {
   if (!valid_site(c, x, y) || label < 1 || label > 4) return fail(c, CTM_EINVAL, "bad site or label");
   Guard gd(c);
   const int site = y * c->Lx + x;
-  CTM_CUDA_OK(jacobi_svd_coop(c->cx, c->chi, Cp(c, label - 1, site), 0, c->sv, nullptr,
-                              nullptr, false, c->jw, 1, c->opts.svd_max_sweeps, c->err, c->num_sms, c->stream,
-                              &c->launches));
+  if (jacobi_vals_supported(c->cx, c->chi))
+    CTM_CUDA_OK(jacobi_vals(c->cx, c->chi, Cp(c, label - 1, site), 0, c->sv, 1,
+                            c->opts.svd_max_sweeps, c->err, c->stream, &c->launches));
+  else
+    CTM_CUDA_OK(jacobi_svd_coop(c->cx, c->chi, Cp(c, label - 1, site), 0, c->sv, nullptr, nullptr,
+                                false, c->jw, 1, c->opts.svd_max_sweeps, c->err, c->num_sms,
+                                c->stream, &c->launches));
   CTM_CUDA_OK(normalize(false, c->chi, c->sv, 0, 1, c->dscal, true, c->scratch, c->stream, &c->launches));
   CTM_CUDA_OK(cudaMemcpyAsync(s_out, c->sv, c->chi * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   CK(check_err(c));

@@ -155,6 +155,14 @@ cudaError_t jacobi32_presolve(bool cx, int k, const void* A, long strideA, void*
                               int max_sweeps, int* sweeps, cudaStream_t s, long* launches);
 size_t jacobi_coop_work_bytes(bool cx, int k, int batch);
 
+// ---------------------------------------------------------- jacobi_vals.cu
+// Singular values (descending) of a batch of k x k matrices (row- or
+// column-major alike, stride strideA elements), without vectors and without
+// workspace. Supported up to k = 128 real, 96 complex.
+bool jacobi_vals_supported(bool cx, int k);
+cudaError_t jacobi_vals(bool cx, int k, const void* A, long strideA, double* s, int batch,
+                        int max_sweeps, int* err, cudaStream_t s_, long* launches);
+
 // chol_inv on a cooperative grid (blocked, jacobi.cu); with scale the Gram
 // is first scaled to unit diagonal (D^-1 G D^-1) and Linv returns
 // L_s^-1 D^-1, so that Z Linv^H is still the orthonormalised block. work:

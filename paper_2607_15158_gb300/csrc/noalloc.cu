@@ -82,8 +82,12 @@ extern "C" ctm_status ctm_svdvals_noalloc(const void* A, int k, ctm_dtype dtype,
   void* jw = b + kHeaderBytes;                   // Jacobi work area
   if (cudaMemsetAsync(err, 0, sizeof(int), st) != cudaSuccess)
     return nfail(CTM_ECUDA, "clearing the error word failed");
-  if (ctm::jacobi_svd_coop(cx, k, A, 0, s, nullptr, nullptr, false, jw, 1, 80, err, sms, st,
-                           nullptr) != cudaSuccess) {
+  const cudaError_t e =
+      ctm::jacobi_vals_supported(cx, k)
+          ? ctm::jacobi_vals(cx, k, A, 0, s, 1, 80, err, st, nullptr)
+          : ctm::jacobi_svd_coop(cx, k, A, 0, s, nullptr, nullptr, false, jw, 1, 80, err, sms, st,
+                                 nullptr);
+  if (e != cudaSuccess) {
     cudaGetLastError();
     return nfail(CTM_ECUDA, "launch of the Jacobi kernel failed");
   }
