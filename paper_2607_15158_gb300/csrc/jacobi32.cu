@@ -230,12 +230,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(J32T, 1)
                 ga.x += __shfl_xor_sync(m8, ga.x, o);
                 if (CX) ga.y += __shfl_xor_sync(m8, ga.y, o);
               }
-              const float gm = sqrtf(ga.x * ga.x + ga.y * ga.y);
-              if (gm > tol * sqrtf(al) * sqrtf(be) && gm > 0.f) {
-                const float zeta = (be - al) / (2.f * gm);
+              // the three roots, then zeta and the phase's two divisions, side by
+              // side in lanes 0, 1 and 2 of the group
+              const float g2 = ga.x * ga.x + ga.y * ga.y;
+              float w = sqrtf(l8 == 0 ? g2 : l8 == 1 ? al : be);
+              const float gm = __shfl_sync(m8, w, 0, 8);
+              const float sa = __shfl_sync(m8, w, 1, 8), sb = __shfl_sync(m8, w, 2, 8);
+              if (gm > tol * sa * sb && gm > 0.f) {
+                w = (l8 == 0 ? be - al : l8 == 1 ? ga.x : -ga.y) / (l8 == 0 ? 2.f * gm : gm);
+                const float zeta = __shfl_sync(m8, w, 0, 8);
+                const float2 e = make_float2(__shfl_sync(m8, w, 1, 8), __shfl_sync(m8, w, 2, 8));
                 const float tt = copysignf(1.f, zeta) / (fabsf(zeta) + sqrtf(1.f + zeta * zeta));
                 const float c = 1.f / sqrtf(1.f + tt * tt), s = c * tt;
-                const float2 e = make_float2(ga.x / gm, -ga.y / gm);   // conj(gamma) / |gamma|
                 #pragma unroll 4
                 for (int r = l8; r < k; r += 8) {
                   T xv = x[r], yv = y[r];
