@@ -542,7 +542,11 @@ ctm_status qr_inplace(ctm_ctx* c, void* Zm, void* tmp, bool split_mode) {
       CK(gemm_exact(c, g));
     }
     int* dead = c->dead;   // every pass finds and refills dependent columns
-    const uint64_t rseed = (c->opts.seed * 1000003ull + c->qr_calls) * 4 + pass;
+    // a recorded move counts its QRs from its start (ctm_ctx::MoveGraph)
+    RepairSeed rseed;
+    rseed.base = c->recording_move ? c->qr_base : nullptr;
+    rseed.add = c->opts.seed * 1000003ull + c->qr_calls - (c->recording_move ? c->qr_start : 0);
+    rseed.pass = pass;
     // the k x k factor on one SM or a cluster of eight (chol_cluster.cu)
     const bool cl_chol = chol_cluster_supported(c->cx, c->k);
     if (split && row_solve && pass == 1) {
@@ -1121,6 +1125,107 @@ ctm_status move_impl(ctm_ctx* c, int r) {
   return CTM_OK;
 }
 
+// split-precision states of the lanes and helpers
+std::vector<SplitCtx*> split_states(const ctm_ctx* c) {
+  std::vector<SplitCtx*> v;
+  for (const auto& L : c->lanes)
+    if (L.split) v.push_back(L.split);
+  for (const auto& H : c->helpers)
+    if (H.split) v.push_back(H.split);
+  return v;
+}
+
+void drop_graph(ctm_ctx::MoveGraph& g) {
+  if (g.exec) cudaGraphExecDestroy(g.exec);
+  g.exec = nullptr;
+}
+
+// A move in direction r, replayed from its graph where that pays: a kernel
+// starts 2.1 us after the one before it on its stream, 0.6 us inside a graph,
+// and the host needs 2.1 us a launch, which bounds cells with several lanes.
+// Per iteration, direct and replayed: 1x1 real D = 2 chi = 8 4.43 ms and 3.53,
+// 3x3 complex D = 2 chi = 9 12.1 and 8.6, 1x1 D = 3 chi = 27 7.8 and 6.9,
+// exact-digit 2x2 complex D = 4 chi = 64 (N = 1024) 92.8 and 85.8, 3x3 D = 4
+// chi = 64 194.8 and 193.2, split 3x3 complex D = 6 chi = 144 (N = 5184) the same:
+// the line lies where nothing is left to gain. A direction is recorded after
+// it has run once directly with the same buffers (so that all have their
+// size), past its warm-up, and only where the host decides nothing from move
+// to move (no recycling policy, no recording for gradients, no profiling).
+constexpr int GRAPH_MAX_N = 2048;
+ctm_status run_move(ctm_ctx* c, int r) {
+  bool ok = !c->graphs_off && c->opts.method == CTM_PROJ_SI && c->N <= GRAPH_MAX_N && !c->prof &&
+            !grad_recording(c) && c->moves_done[r] >= c->opts.warmup_iters &&
+            !(c->opts.recycle_sin2 > 0.0);
+  for (int i = 0; ok && i < c->S; ++i) ok = c->rf_ready[r * c->S + i] != 0;
+  if (!ok) return move_impl(c, r);
+  auto key_now = [&]() {
+    long k = 0;
+    for (SplitCtx* sp : split_states(c)) k += split_generation(sp);
+    return k;
+  };
+  ctm_ctx::MoveGraph& g = c->graphs[r][c->exact ? 1 : 0];
+  if (g.exec && g.key != key_now()) drop_graph(g);
+  if (!g.exec && g.ran != key_now()) {
+    const ctm_status st = move_impl(c, r);
+    g.ran = key_now();
+    return st;
+  }
+  const uint64_t qr0 = c->qr_calls;
+  if (g.exec) {
+    // what move_impl does on the host
+    c->spectra_fresh = false;
+    const bool updates = c->opts.si_rounds > 0;
+    for (int i = 0; i < c->S; ++i) {
+      c->si_rounds_used[r * c->S + i] = updates;
+      if (updates) ++c->si_updates[r * c->S + i];
+    }
+    (updates ? c->n_updates : c->n_skipped) += c->S;
+    c->qr_calls += g.qrs;
+    c->launches += g.launches;
+    c->moves_done[r] += 1;
+    c->last_dir = r;
+  } else {
+    const long l0 = c->launches, up0 = c->n_updates, sk0 = c->n_skipped;
+    const std::vector<int> su0 = c->si_updates;
+    const int last0 = c->last_dir, moves0 = c->moves_done[r];
+    const std::string msg0 = c->msg;
+    cudaGraph_t graph = nullptr;
+    ctm_status st = CTM_ECUDA;
+    if (cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+      c->recording_move = true;
+      c->qr_start = qr0;
+      st = move_impl(c, r);
+      c->recording_move = false;
+      if (cudaStreamEndCapture(c->stream, &graph) != cudaSuccess) st = CTM_ECUDA;
+    }
+    if (st == CTM_OK && cudaGraphInstantiate(&g.exec, graph, 0) != cudaSuccess) {
+      g.exec = nullptr;
+      st = CTM_ECUDA;
+    }
+    if (graph) cudaGraphDestroy(graph);
+    if (st != CTM_OK) {
+      // nothing has run: back to the state before, and directly from now on
+      cudaGetLastError();
+      c->graphs_off = true;
+      c->msg = msg0;
+      c->last_dir = last0;
+      c->moves_done[r] = moves0;
+      c->qr_calls = qr0;
+      c->launches = l0;
+      c->n_updates = up0;
+      c->n_skipped = sk0;
+      c->si_updates = su0;
+      return move_impl(c, r);
+    }
+    g.key = key_now();
+    g.launches = c->launches - l0;
+    g.qrs = c->qr_calls - qr0;
+  }
+  CTM_CUDA_OK(set_u64(c->qr_base, qr0, c->stream, &c->launches));
+  CTM_CUDA_OK(cudaGraphLaunch(g.exec, c->stream));
+  return CTM_OK;
+}
+
 ctm_status corner_spectra(ctm_ctx* c, double* out) {
   PhaseScope ps(c, PH_SPECTRA);
   // unnormalised singular values of all 4 S corners, [label][site][chi]
@@ -1444,6 +1549,7 @@ ctm_status create(ctm_ctx** out, int Lx, int Ly, int d, int Dk, int Db, int chi,
   AL(c->imp[0], nk * es);
   AL(c->imp[1], nk * es);
   AL(c->err, sizeof(int));
+  AL(c->qr_base, sizeof(uint64_t));
   AL(c->dead, k * sizeof(int));
   AL(c->chol_work, chol_coop_work_bytes((int)k, 1));
   AL(c->dsc, k * sizeof(double));
@@ -1999,7 +2105,7 @@ ctm_status ctm_move(ctm_ctx* c, ctm_dir dir) {
   ExactScope xs(c, exact_always(c));
   const long l0 = c->launches;
   CTM_CUDA_OK(cudaEventRecord(c->ev0, c->stream));
-  CK(move_impl(c, (int)dir));
+  CK(run_move(c, (int)dir));
   CTM_CUDA_OK(cudaEventRecord(c->ev1, c->stream));
   CK(check_err(c));
   CK(update_recycling(c));
@@ -2031,7 +2137,7 @@ ctm_status ctm_converge(ctm_ctx* c, double tol, int max_iter, int* iters_out, do
   int it = 0;
   while (it < max_iter) {
     if (c->split && c->opts.split_refine > 0.0 && delta < c->opts.split_refine) c->exact = true;
-    for (int r = 0; r < 4; ++r) CK(move_impl(c, r));
+    for (int r = 0; r < 4; ++r) CK(run_move(c, r));
     ++it;
     CK(corner_spectra(c, c->spec_new));
     CTM_CUDA_OK(spectra_delta(c->chi, 4 * c->S, c->spec_new, c->spec_old, c->dscal + 1, c->stream, &c->launches));
@@ -2328,7 +2434,10 @@ ctm_status ctm_transfer_spectrum(ctm_ctx* c, int dir, int row, int nvals, double
       CK(mm_small(c, opH, OP_N, m, m, n, X, m, X, m, G, m));
       CTM_CUDA_OK(chol_inv(c->cx, m, n, false, G, Li, 1, dead, c->err, c->stream, &c->launches));
       CK(mm_small(c, OP_N, opH, n, m, m, X, m, Li, m, V2, m));
-      CTM_CUDA_OK(repair_dead_columns(c->cx, n, m, V2, V2, dead, 104729ull + pass, c->stream,
+      RepairSeed rseed;   // 104729 + pass
+      rseed.add = (104729ull + pass) / 4;
+      rseed.pass = (int)((104729ull + pass) % 4);
+      CTM_CUDA_OK(repair_dead_columns(c->cx, n, m, V2, V2, dead, rseed, c->stream,
                                       &c->launches));
       CTM_CUDA_OK(cudaMemcpyAsync(X, V2, (size_t)n * m * es, cudaMemcpyDeviceToDevice, c->stream));
     }
@@ -2439,16 +2548,6 @@ ctm_status ctm_last_timing(const ctm_ctx* c, double* ms, long* launches) {
   return CTM_OK;
 }
 
-// split-precision states of the lanes and helpers
-static std::vector<SplitCtx*> split_states(const ctm_ctx* c) {
-  std::vector<SplitCtx*> v;
-  if (c->lanes.empty()) v.push_back(c->split);
-  for (const auto& L : c->lanes) v.push_back(L.split);
-  for (const auto& H : c->helpers)
-    if (H.split) v.push_back(H.split);
-  return v;
-}
-
 ctm_status ctm_profile_enable(ctm_ctx* c, int on) {
   if (!c) return CTM_EINVAL;
   Guard gd(c);
@@ -2507,6 +2606,8 @@ void ctm_free(ctm_ctx* c) {
   for (auto& H : c->helpers)
     if (H.stream) cudaStreamSynchronize(H.stream);
   if (c->stream) cudaStreamSynchronize(c->stream);
+  for (auto& d : c->graphs)
+    for (auto& g : d) drop_graph(g);
   destroy_helpers(c);
   for (auto& e : c->pev) cudaEventDestroy(e);
   if (c->stream) cudaStreamSynchronize(c->stream);

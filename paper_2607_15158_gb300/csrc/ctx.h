@@ -107,6 +107,23 @@ struct ctm_ctx {
   double* dsc = nullptr;       // column scales of the Jacobi-scaled Gram
   void* fac = nullptr;         // per-tensor normalisation factors
   uint64_t qr_calls = 0;       // counter of the repair directions
+  // Moves of small cells, whose kernels are as short as their launches, are
+  // recorded as CUDA graphs once their direction is past its warm-up, and
+  // replayed (run_move). A graph holds while the buffers that its kernels
+  // were given stay (key: the growth of the split buffers); the QR counter
+  // reaches its kernels through qr_base.
+  struct MoveGraph {
+    cudaGraphExec_t exec = nullptr;
+    long key = -1;        // of the graph
+    long ran = -1;        // key under which a move of this direction last ran directly
+    long launches = 0;
+    uint64_t qrs = 0;
+  };
+  MoveGraph graphs[4][2];      // per direction; [1]: with exact-digit products
+  bool graphs_off = false;     // recording failed once: every move runs directly
+  bool recording_move = false;
+  uint64_t qr_start = 0;       // qr_calls at the start of the recorded move
+  uint64_t* qr_base = nullptr; // device copy of qr_calls at the start of a replay
   // recycling policy (opts.recycle_sin2): per direction and cut, the number of
   // subspace-iteration updates made and whether the next move only recycles
   std::vector<int> si_updates;
@@ -227,5 +244,6 @@ ctm_status check_err(ctm_ctx* c);
 // recorded moves (grad.cu): called at the start of every move while recording
 ctm_status grad_checkpoint(ctm_ctx* c, int r);
 void grad_destroy(ctm_ctx* c);
+bool grad_recording(const ctm_ctx* c);
 
 }  // namespace ctmi

@@ -903,6 +903,8 @@ ctm_status seed(Tape& T, void* v, size_t n, const double* src) {
 
 }  // namespace
 
+bool grad_recording(const ctm_ctx* c) { return c->grad && c->grad->recording; }
+
 ctm_status grad_checkpoint(ctm_ctx* c, int r) {
   if (!c->grad || !c->grad->recording) return CTM_OK;
   Checkpoint cp;

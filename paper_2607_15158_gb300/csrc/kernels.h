@@ -55,6 +55,20 @@ cudaError_t dot64(bool cx, bool conj_x, long n, const void* x, long sx,
                   const void* y, long sy, void* out, int batch, void* work,
                   size_t work_bytes, cudaStream_t s, long* launches);
 
+// Seed of the repair directions of one CholeskyQR pass: 4 (add + *base) + pass
+// (base may be null). Kernels of a replayed move read the number of earlier
+// QRs from device memory, since their arguments stay those of the recording.
+struct RepairSeed {
+  const uint64_t* base = nullptr;
+  uint64_t add = 0;
+  int pass = 0;
+#ifdef __CUDACC__
+  __device__ uint64_t value() const { return (add + (base ? *base : 0ull)) * 4ull + pass; }
+#endif
+};
+// *p = v
+cudaError_t set_u64(uint64_t* p, uint64_t v, cudaStream_t s, long* launches);
+
 // ------------------------------------------------------------- linalg.cu
 // Lower Cholesky factor of G (+ shift I) and its inverse, one block per
 // matrix: G is k x k (ld k), overwritten by L; Linv receives L^-1. With
@@ -74,7 +88,7 @@ cudaError_t chol_inv(bool cx, int k, long n, bool shift, void* G, void* Linv,
 // (trsm_rows_supported: k <= ~166 complex, ~235 real).
 bool trsm_rows_supported(bool cx, int k);
 cudaError_t trsm_rows(bool cx, int k, long rows, const void* L, const double* dsc, const void* Z,
-                      void* Q, const int* dead, uint64_t seed, int num_sms, cudaStream_t s,
+                      void* Q, const int* dead, RepairSeed seed, int num_sms, cudaStream_t s,
                       long* launches);
 
 // ------------------------------------------------------------- absorb.cu
@@ -115,7 +129,7 @@ cudaError_t chol_cluster(bool cx, int k, long rows, bool shift, bool scale, cons
 // deterministic pseudo-random entries (a counter-based hash of seed, column,
 // row).
 cudaError_t repair_dead_columns(bool cx, long rows, int k, const void* src, void* Q,
-                                const int* dead, uint64_t seed, cudaStream_t s, long* launches);
+                                const int* dead, RepairSeed seed, cudaStream_t s, long* launches);
 
 // Per tensor (batch, stride): x <- x * conj(phase of its largest-modulus
 // entry, lowest index on ties) / ||x||_F. work: 3 * 152 * batch doubles;

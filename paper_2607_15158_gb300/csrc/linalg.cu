@@ -469,7 +469,8 @@ __device__ __forceinline__ cplx repair_entry(cplx, int c, long r, uint64_t seed)
 // Q <- src with its dead columns replaced (src may be Q)
 template <typename T>
 __global__ void repair_kernel(long rows, int k, const T* src, T* Q, const int* dead,
-                              uint64_t seed) {
+                              RepairSeed rs) {
+  const uint64_t seed = rs.value();
   for (long idx = blockIdx.x * (long)blockDim.x + threadIdx.x; idx < rows * k;
        idx += (long)gridDim.x * blockDim.x) {
     const long r = idx / k;
@@ -573,8 +574,9 @@ __global__ void scale_by_kernel(long n, T* x, long stride, const T* fac) {
 template <typename T, int R>
 __global__ void __launch_bounds__(1024, 1) trsm_rows_kernel(long rows, int k, const T* L,
                                                             const double* dsc, const T* Z, T* Q,
-                                                            const int* dead, uint64_t seed) {
+                                                            const int* dead, RepairSeed rs) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  const uint64_t seed = rs.value();
   T* Lc = reinterpret_cast<T*>(smem_raw);   // column j at Lc[j k - j (j - 1) / 2 + i - j]
   double* rinv = reinterpret_cast<double*>(Lc + (size_t)k * (k + 1) / 2);
   double* dinv = rinv + k;
@@ -654,7 +656,7 @@ bool trsm_rows_supported(bool cx, int k) {
 
 template <typename T, int R>
 cudaError_t launch_trsm(int k, long rows, const void* L, const double* dsc, const void* Z, void* Q,
-                        const int* dead, uint64_t seed, int num_sms, cudaStream_t s) {
+                        const int* dead, RepairSeed seed, int num_sms, cudaStream_t s) {
   const size_t shm = (size_t)k * (k + 1) / 2 * sizeof(T) + 2 * (size_t)k * sizeof(double);
   static size_t configured = 0;
   const cudaError_t e = raise_smem((const void*)trsm_rows_kernel<T, R>, configured, shm);
@@ -673,7 +675,7 @@ cudaError_t launch_trsm(int k, long rows, const void* L, const double* dsc, cons
 // R = columns per lane: the smallest of 1, 2, 3, 4, 5, 6, 8 with 32 R >= k
 template <typename T>
 cudaError_t trsm_dispatch(int k, long rows, const void* L, const double* dsc, const void* Z,
-                          void* Q, const int* dead, uint64_t seed, int num_sms, cudaStream_t s) {
+                          void* Q, const int* dead, RepairSeed seed, int num_sms, cudaStream_t s) {
   if (k <= 32) return launch_trsm<T, 1>(k, rows, L, dsc, Z, Q, dead, seed, num_sms, s);
   if (k <= 64) return launch_trsm<T, 2>(k, rows, L, dsc, Z, Q, dead, seed, num_sms, s);
   if (k <= 96) return launch_trsm<T, 3>(k, rows, L, dsc, Z, Q, dead, seed, num_sms, s);
@@ -684,7 +686,7 @@ cudaError_t trsm_dispatch(int k, long rows, const void* L, const double* dsc, co
 }
 
 cudaError_t trsm_rows(bool cx, int k, long rows, const void* L, const double* dsc, const void* Z,
-                      void* Q, const int* dead, uint64_t seed, int num_sms, cudaStream_t s,
+                      void* Q, const int* dead, RepairSeed seed, int num_sms, cudaStream_t s,
                       long* launches) {
   if (!trsm_rows_supported(cx, k)) return cudaErrorInvalidValue;
   if (launches) ++*launches;
@@ -693,7 +695,7 @@ cudaError_t trsm_rows(bool cx, int k, long rows, const void* L, const double* ds
 }
 
 cudaError_t repair_dead_columns(bool cx, long rows, int k, const void* src, void* Q,
-                                const int* dead, uint64_t seed, cudaStream_t s, long* launches) {
+                                const int* dead, RepairSeed seed, cudaStream_t s, long* launches) {
   if (cx)
     repair_kernel<cplx><<<grid_for(rows * k), 256, 0, s>>>(rows, k, (const cplx*)src, (cplx*)Q,
                                                            dead, seed);
@@ -891,6 +893,14 @@ __global__ void small_eig_kernel(int m, const T* H, double* ev, int* status) {
 }
 
 }  // namespace
+
+__global__ void set_u64_kernel(uint64_t* p, uint64_t v) { *p = v; }
+
+cudaError_t set_u64(uint64_t* p, uint64_t v, cudaStream_t s, long* launches) {
+  set_u64_kernel<<<1, 1, 0, s>>>(p, v);
+  if (launches) ++*launches;
+  return cudaGetLastError();
+}
 
 cudaError_t hash_fill(long n, uint64_t seed, double* x, cudaStream_t s, long* launches) {
   long b = (n + 255) / 256;

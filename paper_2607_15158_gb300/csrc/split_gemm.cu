@@ -1048,6 +1048,7 @@ struct SplitCtx {
   void* oz_part = nullptr;
   size_t oz_part_bytes = 0;
   long oz_launches = 0;
+  long generation = 0;      // buffers allocated or replaced
   int* err = nullptr;       // device error flag of the owning context
   // per-launch CUDA events around the tensor-core kernel (profiling)
   bool prof = false;
@@ -1074,6 +1075,7 @@ ctm_status grow(SplitCtx* sc, void** p, size_t* have, size_t need) {
     return sfail(sc, CTM_ENOMEM, "split-precision buffer allocation failed");
   }
   *have = need;
+  ++sc->generation;
   return CTM_OK;
 }
 
@@ -1301,6 +1303,7 @@ ctm_status split_prepare_corners(SplitCtx* sc, void* const* Q, int N, unsigned m
           cudaGetLastError();
           return sfail(sc, CTM_ENOMEM, "corner slice allocation failed");
         }
+        ++sc->generation;
       }
       const int op = o == 0 ? OP_N : (sc->cx ? OP_C : OP_T);
       ctm_status st = prep_a(sc, Q[i], N, op, N, N, Kp, sc->cslices[i][o], s, launches);
@@ -1438,6 +1441,8 @@ size_t split_partial_splits(size_t N, bool cx) {
   const size_t kb = ((cx ? 2 : 1) * N + BK - 1) / BK;
   return std::max<size_t>(32, (kb + KB_SPLIT_MAX - 1) / KB_SPLIT_MAX);
 }
+
+long split_generation(const SplitCtx* sc) { return sc->generation; }
 
 const char* split_last_error(const SplitCtx* sc) {
   return sc ? sc->msg.c_str() : "split precision not initialised";

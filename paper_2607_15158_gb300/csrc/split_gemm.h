@@ -60,6 +60,9 @@ ctm_status split_profile(SplitCtx* sc, int on, double* ms, long* launches, doubl
 // for complex) uses: each partial covers a bounded number of K blocks.
 size_t split_partial_splits(size_t N, bool cx);
 
+// Number of times a buffer of the state was allocated or replaced.
+long split_generation(const SplitCtx* sc);
+
 const char* split_last_error(const SplitCtx* sc);
 
 }  // namespace ctm
