@@ -1766,11 +1766,12 @@ ctm_status two_site(ctm_ctx* c, int r, int x, int y, void* K1, void* K2, void* o
          tn(K1, {d, Dk, Dk, Dk, Dk}), false, tn(c->pipe[0], {chi, Db, chi, Db, d, Dk, Dk})));
   CK(ein(c, "kLcUsxm,tULXM->kcsxmtXM", tn(c->pipe[0], {chi, Db, chi, Db, d, Dk, Dk}), false,
          tn(B1, {d, Db, Db, Db, Db}), false, tn(c->pipe[1], {chi, chi, d, Dk, Dk, d, Db, Db})));
-  CK(ein(c, "kcsxmtXM,jk->jcsxmtXM", tn(c->pipe[1], {chi, chi, d, Dk, Dk, d, Db, Db}), false,
-         C_(3, x), false, tn(c->pipe[0], {chi, chi, d, Dk, Dk, d, Db, Db})));
+  // the corner below joins the edge below first (chi^3 D^2), so the patch's
+  // chi^2 d^2 D^4 elements meet one product instead of two
   Tn L = tn(Lbuf, {chi, chi, d, Dk, d, Db});
-  CK(ein(c, "jcsxmtXM,ijxX->icsmtM", tn(c->pipe[0], {chi, chi, d, Dk, Dk, d, Db, Db}), false,
-         T_(2, x), false, L));
+  CK(ein(c, "ijxX,jk->ikxX", T_(2, x), false, C_(3, x), false, tn(c->pipe[0], {chi, chi, Dk, Db})));
+  CK(ein(c, "kcsxmtXM,ikxX->icsmtM", tn(c->pipe[1], {chi, chi, d, Dk, Dk, d, Db, Db}), false,
+         tn(c->pipe[0], {chi, chi, Dk, Db}), false, L));
   // right half R[c, i, q, m, v, M]
   CK(ein(c, "ceoO,ef->cfoO", T_(0, x + 1), false, C_(1, x + 1), false,
          tn(c->pipe[0], {chi, chi, Dk, Db})));
@@ -1780,11 +1781,11 @@ ctm_status two_site(ctm_ctx* c, int r, int x, int y, void* K1, void* K2, void* o
          tn(K2, {d, Dk, Dk, Dk, Dk}), false, tn(c->pipe[0], {chi, chi, Db, Db, d, Dk, Dk})));
   CK(ein(c, "cgORqmw,vOMWR->cgqmwvMW", tn(c->pipe[0], {chi, chi, Db, Db, d, Dk, Dk}), false,
          tn(B2, {d, Db, Db, Db, Db}), false, tn(c->pipe[1], {chi, chi, d, Dk, Dk, d, Db, Db})));
-  CK(ein(c, "cgqmwvMW,gh->chqmwvMW", tn(c->pipe[1], {chi, chi, d, Dk, Dk, d, Db, Db}), false,
-         C_(2, x + 1), false, tn(c->pipe[0], {chi, chi, d, Dk, Dk, d, Db, Db})));
   Tn R = tn(Rbuf, {chi, chi, d, Dk, d, Db});
-  CK(ein(c, "chqmwvMW,hiwW->ciqmvM", tn(c->pipe[0], {chi, chi, d, Dk, Dk, d, Db, Db}), false,
-         T_(2, x + 1), false, R));
+  CK(ein(c, "gh,hiwW->giwW", C_(2, x + 1), false, T_(2, x + 1), false,
+         tn(c->pipe[0], {chi, chi, Dk, Db})));
+  CK(ein(c, "cgqmwvMW,giwW->ciqmvM", tn(c->pipe[1], {chi, chi, d, Dk, Dk, d, Db, Db}), false,
+         tn(c->pipe[0], {chi, chi, Dk, Db}), false, R));
   CK(ein(c, "icsmtM,ciqmvM->sqtv", L, false, R, false, tn(out, {d, d, d, d})));
   c->scratch_off = mark;
   return CTM_OK;
