@@ -18,7 +18,8 @@
 // pair's input staged by cp.async in fp32, else two groups; GT = 16, TL = 4,
 // one group for <= 64 (D <= 8). D = 6 and D = 8 also have compile-time
 // variants. Arithmetic in F: fp32 (split-precision contexts, ~1e-7 relative
-// like the bf16x3 products) or fp64.
+// like the bf16x3 products) or fp64. Square bonds of 4 to 6 with many pairs in
+// fp32, and all of fp64, have kernels of their own below.
 #include <algorithm>
 
 #include "common.cuh"
@@ -251,6 +252,214 @@ __global__ void __launch_bounds__(NG * GT * GT, ab_min_blocks<F, NG>())
   }
 }
 
+// fp32 arithmetic for square bonds DK = 4, 5, 6 and many pairs, the steps of a
+// pair overlapped: four warps copy and convert the next input blocks into the
+// second of two X buffers while the others multiply, and the results go from
+// the registers to Out. In absorb_ab_kernel all warps of a block convert,
+// multiply and write in turn, and whatever D is compute 36 x 36 outputs.
+// The multiplying warps form two halves, each with its own named barriers, so
+// that one half's waits fall into the other's work. A pair's DK^2 x DK^2
+// outputs are TR x TC register tiles of RG x CG threads in a SLOT of lanes;
+// larger tiles than 3 x 3 keep the shared-memory reads (2 (TR + TC) wavefronts
+// a warp and k, complex) under the fp32 pipes' TR TC clocks. Measured for
+// complex data, d = 2: D = 4, chi = 80 162 us -> 42, D = 5, chi = 58 142 -> 72,
+// D = 6, chi = 144 915 -> 866 (the pipes' rate: 384; tiles of 6 x 4 with packed
+// multiply-adds, 3 x 3, 3 x 6 and 4 x 4 took 900 to 1010).
+template <int DK> struct AP;
+template <> struct AP<6> {
+  static constexpr int TR = 4, TC = 6, RG = 9, CG = 6, SLOT = 64, PH = 2, HW = 4, UNROLL = 1;
+};
+template <> struct AP<5> {
+  static constexpr int TR = 5, TC = 5, RG = 5, CG = 5, SLOT = 32, PH = 6, HW = 6, UNROLL = 4;
+};
+template <> struct AP<4> {
+  static constexpr int TR = 4, TC = 4, RG = 4, CG = 4, SLOT = 16, PH = 12, HW = 6, UNROLL = 1;
+};
+constexpr int AP_LOAD = 128;   // threads that copy and convert
+
+template <int DK, typename F>
+struct APL {   // shared layout, in elements of F
+  // an odd row length spreads a column of A or Y over the banks
+  static constexpr int K1 = DK * DK, LD = K1 | 1, NP = 2 * AP<DK>::PH;
+  static constexpr int PAD4 = DK == 4 ? 8 : 0;   // two pairs a warp: other banks
+  static constexpr int A_S = (K1 * LD + 3) / 4 * 4, B_S = K1 * K1;
+  static constexpr int X_P = (K1 * K1 + 3) / 4 * 4 + PAD4, Y_P = (K1 * LD + 3) / 4 * 4 + PAD4;
+  static constexpr int THREADS = 64 * AP<DK>::HW + AP_LOAD;
+  static constexpr size_t bytes(int d) {
+    return ((size_t)d * (A_S + (B_S + 3) / 4 * 4) + (size_t)NP * (2 * X_P + Y_P)) * sizeof(F);
+  }
+};
+
+__device__ __forceinline__ void nb_sync(int id, int n) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+__device__ __forceinline__ void nb_arrive(int id, int n) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+// fp32 -> fp64, on the integer pipe but for subnormal values
+__device__ __forceinline__ double wide(float a) {
+  return (__float_as_uint(a) & 0x7f800000u) != 0u ? f64_of(a) : (double)a;
+}
+__device__ __forceinline__ cplx wide(float2 a) { return make_double2(wide(a.x), wide(a.y)); }
+
+// v += left (rows ti + RG a, LD apart) times right (columns tj + CG c)
+template <typename F, int DK>
+__device__ __forceinline__ void tile_multiply(F (&v)[AP<DK>::TR][AP<DK>::TC], const F* left,
+                                              const F* right, int ti, int tj) {
+  using P = AP<DK>;
+  constexpr int K1 = DK * DK, LD = APL<DK, F>::LD, UNROLL = P::UNROLL;
+  left += ti * LD;
+  right += tj;
+#pragma unroll UNROLL
+  for (int kk = 0; kk < K1; ++kk) {
+    F xa[P::TR], xb[P::TC];
+#pragma unroll
+    for (int a = 0; a < P::TR; ++a) xa[a] = left[P::RG * a * LD + kk];
+#pragma unroll
+    for (int c = 0; c < P::TC; ++c) xb[c] = right[kk * K1 + P::CG * c];
+#pragma unroll
+    for (int a = 0; a < P::TR; ++a)
+#pragma unroll
+      for (int c = 0; c < P::TC; ++c) mac(v[a][c], xa[a], xb[c]);
+  }
+}
+template <typename F, int DK>
+__device__ __forceinline__ void tile_zero(F (&v)[AP<DK>::TR][AP<DK>::TC]) {
+#pragma unroll
+  for (int a = 0; a < AP<DK>::TR; ++a)
+#pragma unroll
+    for (int c = 0; c < AP<DK>::TC; ++c) v[a][c] = fz<F>();
+}
+template <typename F, int DK, typename Fn>
+__device__ __forceinline__ void tile_each(F (&v)[AP<DK>::TR][AP<DK>::TC], int ti, int tj, Fn&& fn) {
+  using P = AP<DK>;
+#pragma unroll
+  for (int a = 0; a < P::TR; ++a)
+#pragma unroll
+    for (int c = 0; c < P::TC; ++c) fn(ti + P::RG * a, tj + P::CG * c, v[a][c]);
+}
+
+template <typename T, typename F, int DK>
+__global__ void __launch_bounds__(APL<DK, F>::THREADS, 1)
+    absorb_pipe_kernel(int chi, int d, const T* __restrict__ In, const T* __restrict__ A,
+                       const T* __restrict__ B, T* __restrict__ Out) {
+  using L = APL<DK, F>;
+  using P = AP<DK>;
+  constexpr int K1 = L::K1, KN = K1 * K1, LD = L::LD, PH = P::PH;
+  constexpr int HT = 32 * P::HW, NB = HT + AP_LOAD;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  F* Bs = reinterpret_cast<F*>(smem_raw);   // [d][(w,v)][(D,E)]
+  constexpr int BS = (L::B_S + 3) / 4 * 4;
+  F* As = Bs + (size_t)d * BS;               // [d][(d,e)][(u,l)], rows of LD
+  F* Ys = As + (size_t)d * L::A_S;           // [pair][(d,e)][(w,v)], rows of LD
+  F* Xs = Ys + L::NP * L::Y_P;               // [buffer][pair][(u,l)][(w,v)]
+  for (int i = threadIdx.x; i < d * KN; i += L::THREADS) {
+    // As[s][(d,e)][(u,l)] = A[s,u,l,d,e]; Bs[s][(w,v)][(D,E)] = B[s,v,w,D,E]
+    const int s = i / KN, rem = i % KN, x = rem / K1, y = rem % K1;
+    As[s * L::A_S + y * LD + x] = cvt(A[i], F());
+    Bs[s * BS + ((x % DK) * DK + x / DK) * K1 + y] = cvt(B[i], F());
+  }
+  __syncthreads();
+  const size_t row = (size_t)chi * K1;       // stride of the (first chi, Dk, Db) index
+  const long npairs = (long)chi * chi, step = (long)L::NP * gridDim.x;
+  const long first = (long)L::NP * blockIdx.x;
+  const int nsteps = first < npairs ? (int)((npairs - first + step - 1) / step) : 0;
+  // barriers: X buffer b of half h filled 1 + 4 h + b, free again 3 + 4 h + b; Y of pair q 9 + q
+  if (threadIdx.x >= 2 * HT) {
+    const int lt = threadIdx.x - 2 * HT;
+    for (int i = 0; i < nsteps; ++i) {
+      const int b = i & 1;
+#pragma unroll 1
+      for (int h = 0; h < 2; ++h) {
+        if (i >= 2) nb_sync(3 + 4 * h + b, NB);
+        const long p0 = first + i * step + h * PH;
+#pragma unroll 1
+        for (int q = 0; q < PH; ++q) {
+          const long p = p0 + q;
+          if (p >= npairs) break;
+          const int t = (int)(p / chi), n = (int)(p % chi);
+          const T* src = In + (size_t)t * K1 * row + (size_t)n * K1;
+          F* X = Xs + (size_t)(b * L::NP + h * PH + q) * L::X_P;
+          constexpr int U = (KN + AP_LOAD - 1) / AP_LOAD;   // all loads in flight at once
+          T v[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const int e = lt + u * AP_LOAD;
+            if (e < KN) v[u] = __ldcs(src + (size_t)(e / K1) * row + e % K1);
+          }
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            // X[(u,l),(w,v)] = In[t,l,w,n,u,v]
+            const int e = lt + u * AP_LOAD, lw = e / K1, uv = e % K1;
+            if (e < KN)
+              X[(uv / DK * DK + lw / DK) * K1 + lw % DK * DK + uv % DK] = cvt(v[u], F());
+          }
+        }
+        nb_arrive(1 + 4 * h + b, NB);
+      }
+    }
+    return;
+  }
+  const int h = threadIdx.x / HT, ht = threadIdx.x % HT;
+  const int q = ht / P::SLOT, lt = ht % P::SLOT, ti = lt / P::CG, tj = lt % P::CG;
+  F* Y = Ys + (size_t)(h * PH + q) * L::Y_P;
+  auto team_sync = [&] {
+    if constexpr (P::SLOT > 32) nb_sync(9 + h * PH + q, P::SLOT); else __syncwarp();
+  };
+  for (int i = 0; i < nsteps; ++i) {
+    const int b = i & 1;
+    const long p = first + i * step + h * PH + q;
+    const bool live = lt < P::RG * P::CG && p < npairs;
+    const F* X = Xs + (size_t)(b * L::NP + h * PH + q) * L::X_P;
+    F acc[P::TR][P::TC];
+    tile_zero<F, DK>(acc);
+    nb_sync(1 + 4 * h + b, NB);
+    for (int s = 0; s < d; ++s) {
+      F y[P::TR][P::TC];
+      tile_zero<F, DK>(y);
+      if (live) tile_multiply<F, DK>(y, As + s * L::A_S, X, ti, tj);
+      team_sync();   // the previous Y is consumed
+      if (live) tile_each<F, DK>(y, ti, tj, [&](int r, int c, F v) { Y[r * LD + c] = v; });
+      if (s == d - 1 && i + 2 < nsteps) nb_arrive(3 + 4 * h + b, NB);   // X is free
+      team_sync();
+      if (live) tile_multiply<F, DK>(acc, Y, Bs + s * BS, ti, tj);
+    }
+    if (live) {
+      // Out[t,d,D,n,e,E]: the threads of a tile row write runs of (e, E)
+      const int t = (int)(p / chi), n = (int)(p % chi);
+      T* dst = Out + (size_t)t * K1 * row + (size_t)n * K1;
+      tile_each<F, DK>(acc, ti, tj, [&](int r, int c, F v) {
+        dst[(size_t)(r / DK * DK + c / DK) * row + r % DK * DK + c % DK] = wide(v);
+      });
+    }
+  }
+}
+
+template <typename T, typename F, int DK>
+cudaError_t launch_pipe(int chi, int d, const void* In, const void* A, const void* B, void* Out,
+                        int num_sms, cudaStream_t s) {
+  using L = APL<DK, F>;
+  static size_t configured = 0;
+  auto* fn = absorb_pipe_kernel<T, F, DK>;
+  cudaError_t e = raise_smem((const void*)fn, configured, L::bytes(d));
+  if (e != cudaSuccess) return e;
+  const long tiles = ((long)chi * chi + L::NP - 1) / L::NP;
+  fn<<<(unsigned)std::min((long)num_sms, tiles), L::THREADS, L::bytes(d), s>>>(
+      chi, d, static_cast<const T*>(In), static_cast<const T*>(A), static_cast<const T*>(B),
+      static_cast<T*>(Out));
+  return cudaGetLastError();
+}
+
+// more pairs than absorb_ab_kernel's grid of four a block takes at once: up to
+// there that kernel's time is one block's, 19 to 33 us against 27 to 42 here
+// (complex, D = 4 to 6, chi <= 24); above it was never faster (chi = 28: 34, 51
+// and 60 us against 27, 43 and 60)
+template <int DK, typename F>
+bool use_pipe(int chi, int Dk, int Db, int d, int num_sms) {
+  return Dk == DK && Db == DK && APL<DK, F>::bytes(d) <= SMEM_MAX &&
+         (long)chi * chi > 4L * num_sms;
+}
+
 // The same contraction in fp64 (F = T), which the fp64 pipe bounds: a
 // multiply-add occupies a sub-partition for ~77 clocks however few lanes of
 // the warp take part, so no lane may idle and operand reads cost nothing
@@ -440,6 +649,12 @@ cudaError_t launch_geom(int geom, int chi, int Dk, int Db, int d, const void* In
     return launch_absorb64<T>(chi, Dk, Db, d, In, A, B, Out, num_sms, s);
   } else {
     const bool sq = Dk == Db;
+    if (use_pipe<4, F>(chi, Dk, Db, d, num_sms))
+      return launch_pipe<T, F, 4>(chi, d, In, A, B, Out, num_sms, s);
+    if (use_pipe<5, F>(chi, Dk, Db, d, num_sms))
+      return launch_pipe<T, F, 5>(chi, d, In, A, B, Out, num_sms, s);
+    if (use_pipe<6, F>(chi, Dk, Db, d, num_sms))
+      return launch_pipe<T, F, 6>(chi, d, In, A, B, Out, num_sms, s);
     if (geom == 3 && sq && Dk == 6)
       return launch_ab<T, F, 12, 3, 4, true, 6>(chi, Dk, Db, d, In, A, B, Out, num_sms, s);
     if (geom == 3)

@@ -66,3 +66,40 @@ def test_corner_apply_fp64(d, D, chi, p, cplx, herm):
     n = 2 * chi + D * D + d * D * D + chi * D * D + 5
     tol = (2 if cplx else 1) * n * np.finfo(float).eps
     assert (np.abs(out - ref) <= tol * bound).all(), float((np.abs(out - ref) / bound).max())
+
+
+# The split-precision corner product over more than 608 (t, n) pairs, at square
+# bonds D = 4, 5, 6: the fp32 absorption whose warps copy and multiply side by
+# side, with a last group of pairs that is not full and blocks that run one and
+# several steps. Each of the three slice products sums at most 8 K blocks of four
+# matrix instructions in fp32 and keeps values to a few units of 2^-24 (38 in
+# all); the absorption is two fp32 sums of D^2 and d D^2 complex terms between
+# three roundings. The tolerance is the sum of these times 2^-24 times the
+# contraction of absolute values.
+@pytest.mark.parametrize("d,D,chi,cplx", [
+    (2, 4, 25, True),     # 24 pairs a block: fewer blocks than SMs, the last with one pair
+    (3, 4, 62, False),    # a second step for some blocks
+    (2, 5, 25, True),     # 12 pairs a block
+    (1, 5, 45, False),
+    (2, 6, 25, True),     # 4 pairs a block, two steps
+    (2, 6, 37, False),    # 1369 pairs: three steps, both X buffers filled again
+])
+def test_corner_apply_split(d, D, chi, cplx):
+    rng = np.random.default_rng(10 * D + chi)
+    A = _normal(rng, (d, D, D, D, D), cplx)
+    C = _normal(rng, (4, 1, chi, chi), cplx)
+    T = _normal(rng, (4, 1, chi, chi, D, D), cplx)
+    opts = pkg.ctm_default_opts(p=5, precision=pkg.CTM_PREC_SPLIT_BF16)
+    ctx = pkg.ctm_init(1, 1, [A], d, D, chi, cplx=cplx, opts=opts)
+    ctx.ctm_set_env(C, T)
+    Z = _normal(rng, (ctx.N, ctx.k), cplx)
+    out = ctx.ctm_corner_apply(0, 0, 0, 1, Z)
+    ctx.ctm_free()
+    a = (A, np.conj(A), C[0, 0], T[0, 0], T[3, 0])
+    ref = _corner(*a) @ Z
+    bound = _corner(*map(np.abs, a)) @ np.abs(Z)
+    if cplx:
+        bound = 4 * bound
+    tol = (3 * 38 + 2 * D * D + 2 * d * D * D + 3) * 2.0 ** -24
+    assert np.isfinite(out).all()
+    assert np.max(np.abs(out - ref) / bound) < tol
