@@ -24,8 +24,8 @@
 //
 // Kernel: one CTA = 128 output rows x BNc (<= 160) output columns; A and B
 // slices are K-major, staged by TMA in 64-element (128-byte, 128B-swizzled)
-// K blocks through a two-stage mbarrier pipeline; one thread issues the
-// tcgen05.mma instructions, four warps drain the accumulator with
+// K blocks through an mbarrier pipeline; one thread issues the
+// tcgen05.mma instructions, eight warps drain the accumulator with
 // tcgen05.ld. Every mbarrier wait is bounded (2 s of %globaltimer), after
 // which the CTA records DEV_MBAR_TIMEOUT, skips its work, frees its tensor
 // memory and returns.
@@ -49,7 +49,9 @@ namespace {
 constexpr int BM = 128;          // rows per CTA (tcgen05 M)
 constexpr int BK = 64;           // bf16 K elements per stage (128 bytes)
 constexpr int KROW = 128;        // bytes of one staged K row (either format)
-constexpr int STAGES = 2;
+constexpr int STAGES = 2;        // of the exact-digit kernel
+constexpr int MAX_STAGES = 4;    // of the slice kernel: as many as shared memory holds
+constexpr size_t STAGE_SMEM = 225 * 1024;   // shared memory for stages
 constexpr int MAX_BNC = 160;     // columns per CTA
 constexpr int A_SLICE_BYTES = BM * KROW;     // 16 KB
 constexpr uint64_t WAIT_NS = 2000000000ull;  // bound of every mbarrier wait
@@ -169,34 +171,63 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// 16 columns from each of two accumulators
+__device__ __forceinline__ void tmem_ld16x2(uint32_t ta, uint32_t tb, uint32_t (&r)[16],
+                                            uint32_t (&q)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%32];\n"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%33];\n"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+        "=r"(q[0]), "=r"(q[1]), "=r"(q[2]), "=r"(q[3]), "=r"(q[4]), "=r"(q[5]), "=r"(q[6]), "=r"(q[7]), "=r"(q[8]), "=r"(q[9]), "=r"(q[10]), "=r"(q[11]), "=r"(q[12]), "=r"(q[13]), "=r"(q[14]), "=r"(q[15])
+      : "r"(ta), "r"(tb)
+      : "memory");
+}
+
 struct MmaParams {
   int M;          // output rows
   int Np;         // padded output columns (row length of the partials)
   int BNc;        // columns per CTA, multiple of 16, <= MAX_BNC
   int kb_total;   // K blocks of 64
   int kb_split;   // K blocks per split
+  int mt, nchunks, nks;   // work items: row tiles x column chunks x splits
+  int stages;     // staged K blocks, 2 .. MAX_STAGES
   float* part;    // [nks][M][Np] fp32 partial sums
   int* err;
 };
 
+// A persistent grid: CTA b takes the work items b, b + gridDim.x, ..., each one
+// partial sum of a 128 x BNc tile. What bounds it is the operand stream from L2
+// (6 slices of a K block, 84 KB at BNc = 96 and 108 KB at 160, feed 1150 and
+// 1920 clocks of MMA), so the stream never stops: the producer runs on into the
+// next item while the epilogue is at the last one, and the epilogue moves the
+// accumulators to registers first, frees them for the next item's MMAs and only
+// then stores. With one item per CTA, its start (barriers, tensor memory, the
+// first loads) and its epilogue stood between the loads: a 5184 x 10368 corner
+// times 298 columns took 193 us, now 144 (87 at the tensor rate), 2880 x 5760
+// 63 us, now 50; a launch with one item per CTA is as before (15 us).
+// Items are numbered with the chunk fastest, so that the tiles of A that the
+// chunks share, and the splits of B that all row tiles share, are read together.
+// Warp 0 loads, warp 1 issues, warps 2 to 9 drain (two per 32 lanes of tensor
+// memory, alternate 16-column groups).
+constexpr int MMA_THREADS = 320, MMA_EPI = 8, MMA_GROUPS = MAX_BNC / 32;
+
 template <typename F>
-__global__ void __launch_bounds__(128, 1)
+__global__ void __launch_bounds__(MMA_THREADS, 1)
     split_mma_kernel(const __grid_constant__ CUtensorMap tmA,
                      const __grid_constant__ CUtensorMap tmB, MmaParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  const int BNc = p.BNc;
+  const int BNc = p.BNc, nst = p.stages;
   const uint32_t b_slice_bytes = (uint32_t)BNc * KROW;
   const uint32_t stage_bytes = F::NS * A_SLICE_BYTES + F::NS * b_slice_bytes;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STAGES * stage_bytes);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 1);
-  const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + STAGES),
-                 done = smem_u32(bars + 2 * STAGES);
+  __shared__ uint64_t bars[2 * MAX_STAGES + 2];
+  __shared__ uint32_t tmem_slot;
+  const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + MAX_STAGES),
+                 done = smem_u32(bars + 2 * MAX_STAGES),
+                 drained = smem_u32(bars + 2 * MAX_STAGES + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m_tile = blockIdx.x, chunk = blockIdx.y, ks = blockIdx.z;
-  const int kb0 = ks * p.kb_split;
-  const int nkb = min(p.kb_split, p.kb_total - kb0);
   // two accumulators of BNc columns each: [0, acc1) for s0 t0, [acc1, ..)
   // for the five smaller slice products
   uint32_t acc1 = 32;
@@ -204,17 +235,18 @@ __global__ void __launch_bounds__(128, 1)
   const uint32_t ncols = 2 * acc1;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) {
+    for (int s = 0; s < nst; ++s) {
       mbar_init(full0 + 8 * s, 1);
       mbar_init(empty0 + 8 * s, 1);
     }
     mbar_init(done, 1);
+    mbar_init(drained, MMA_EPI);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                     smem_u32(tmem_slot)),
+                     smem_u32(&tmem_slot)),
                  "r"(ncols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -222,90 +254,137 @@ __global__ void __launch_bounds__(128, 1)
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = *tmem_slot;
-  __shared__ int failed;
-  if (threadIdx.x == 0) failed = 0;
-  __syncthreads();
+  const uint32_t tmem = tmem_slot;
+  const int items = p.mt * p.nchunks * p.nks;
+  auto kblocks = [&](int item) {
+    const int kb0 = item / (p.mt * p.nchunks) * p.kb_split;
+    return min(p.kb_split, p.kb_total - kb0);
+  };
 
-  if (nkb > 0 && warp == 0 && lane == 0) {
-    // TMA producer
-    for (int kb = 0; kb < nkb; ++kb) {
-      const int s = kb % STAGES;
-      if (kb >= STAGES && !mbar_wait(empty0 + 8 * s, ((kb / STAGES) - 1) & 1, p.err)) {
-        failed = 1;
-        break;
-      }
-      const uint32_t full = full0 + 8 * s;
-      mbar_expect_tx(full, stage_bytes);
-      uint8_t* st = smem + s * stage_bytes;
-      const int kx = (kb0 + kb) * F::KE;
-      for (int sl = 0; sl < F::NS; ++sl)
-        tma_load_3d(smem_u32(st + sl * A_SLICE_BYTES), &tmA, kx, m_tile * BM, sl, full);
-      for (int sl = 0; sl < F::NS; ++sl)
-        tma_load_3d(smem_u32(st + F::NS * A_SLICE_BYTES + sl * b_slice_bytes), &tmB, kx,
-                    chunk * BNc, sl, full);
-    }
-  } else if (nkb > 0 && warp == 1 && lane == 0) {
-    // MMA issuer: NP slice products per K block, four 32-byte K steps each
-    const uint32_t idesc = F::EB == 2 ? idesc_bf16(BM, BNc) : idesc_tf32(BM, BNc);
-    const int pa[6] = {0, 0, 1, 0, 1, 2};
-    const int pb[6] = {0, 1, 0, 2, 1, 0};
-    bool ok = true;
-    for (int kb = 0; kb < nkb; ++kb) {
-      const int s = kb % STAGES;
-      if (!mbar_wait(full0 + 8 * s, (kb / STAGES) & 1, p.err)) {
-        ok = false;
-        failed = 1;
-        break;
-      }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t st = smem_u32(smem + s * stage_bytes);
-      for (int pr = 0; pr < F::NP; ++pr) {
-        const uint32_t a0 = st + pa[pr] * A_SLICE_BYTES;
-        const uint32_t b0 = st + F::NS * A_SLICE_BYTES + pb[pr] * b_slice_bytes;
-        const uint32_t d = pr == 0 ? tmem : tmem + acc1;
-        const bool first = kb == 0 && (pr == 0 || pr == 1);
-        for (int kk = 0; kk < KROW / 32; ++kk) {
-          if (F::EB == 2)
-            mma_bf16(d, smem_desc(a0 + kk * 32), smem_desc(b0 + kk * 32), idesc,
-                     (first && kk == 0) ? 0u : 1u);
-          else
-            mma_tf32(d, smem_desc(a0 + kk * 32), smem_desc(b0 + kk * 32), idesc,
-                     (first && kk == 0) ? 0u : 1u);
+  if (warp == 0) {
+    if (lane == 0) {
+      // TMA producer
+      int s = 0, lap = 0;   // the stage, and how often it has been filled
+      bool ok = true;
+      for (int item = blockIdx.x; item < items && ok; item += gridDim.x) {
+        const int chunk = item % p.nchunks, m_tile = item / p.nchunks % p.mt;
+        const int kb0 = item / (p.mt * p.nchunks) * p.kb_split, nkb = kblocks(item);
+        for (int kb = 0; kb < nkb; ++kb) {
+          if (lap > 0 && !mbar_wait(empty0 + 8 * s, (lap - 1) & 1, p.err)) {
+            ok = false;
+            break;
+          }
+          const uint32_t full = full0 + 8 * s;
+          mbar_expect_tx(full, stage_bytes);
+          uint8_t* st = smem + s * stage_bytes;
+          const int kx = (kb0 + kb) * F::KE;
+          for (int sl = 0; sl < F::NS; ++sl)
+            tma_load_3d(smem_u32(st + sl * A_SLICE_BYTES), &tmA, kx, m_tile * BM, sl, full);
+          for (int sl = 0; sl < F::NS; ++sl)
+            tma_load_3d(smem_u32(st + F::NS * A_SLICE_BYTES + sl * b_slice_bytes), &tmB, kx,
+                        chunk * BNc, sl, full);
+          if (++s == nst) s = 0, ++lap;
         }
       }
-      mma_commit(empty0 + 8 * s);
+      // a CTA that gave up does not end before its copies have landed
+      for (int i = 0; !ok && i < nst; ++i) {
+        const int fills = lap + (i < s ? 1 : 0);
+        if (fills > 0) mbar_wait(full0 + 8 * i, (fills - 1) & 1, p.err);
+      }
     }
-    if (ok) mma_commit(done);
-  }
-  // epilogue: all four warps, TMEM lanes 32w .. 32w+31 = rows of this warp
-  __syncwarp();
-  bool have = nkb > 0;
-  if (have && !mbar_wait(done, 0, p.err)) have = false;
-  __syncthreads();
-  if (failed) have = false;
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (have) {
-    const int row = m_tile * BM + warp * 32 + lane;
-    float* out = p.part + ((size_t)ks * p.M + row) * p.Np + (size_t)chunk * BNc;
-    for (int c0 = 0; c0 < BNc; c0 += 16) {
-      uint32_t r[16], q[16];
-      tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, r);
-      tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + acc1 + (uint32_t)c0, q);
-      if (row < p.M) {
-        // 64 contiguous bytes of this thread's row (Np, BNc and c0 are
-        // multiples of 16 floats, so the row segment is 64-byte aligned);
+  } else if (warp == 1) {
+    if (lane == 0) {
+      // MMA issuer: NP slice products per K block, four 32-byte K steps each
+      const uint32_t idesc = F::EB == 2 ? idesc_bf16(BM, BNc) : idesc_tf32(BM, BNc);
+      const int pa[6] = {0, 0, 1, 0, 1, 2};
+      const int pb[6] = {0, 1, 0, 2, 1, 0};
+      int s = 0, lap = 0, u = 0;
+      bool ok = true;
+      for (int item = blockIdx.x; item < items && ok; item += gridDim.x, ++u) {
+        if (u > 0 && !mbar_wait(drained, (u - 1) & 1, p.err)) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const int nkb = kblocks(item);
+        for (int kb = 0; kb < nkb; ++kb) {
+          if (!mbar_wait(full0 + 8 * s, lap & 1, p.err)) {
+            ok = false;
+            break;
+          }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint32_t st = smem_u32(smem + s * stage_bytes);
+          for (int pr = 0; pr < F::NP; ++pr) {
+            const uint32_t a0 = st + pa[pr] * A_SLICE_BYTES;
+            const uint32_t b0 = st + F::NS * A_SLICE_BYTES + pb[pr] * b_slice_bytes;
+            const uint32_t d = pr == 0 ? tmem : tmem + acc1;
+            const bool first = kb == 0 && (pr == 0 || pr == 1);
+            for (int kk = 0; kk < KROW / 32; ++kk) {
+              if (F::EB == 2)
+                mma_bf16(d, smem_desc(a0 + kk * 32), smem_desc(b0 + kk * 32), idesc,
+                         (first && kk == 0) ? 0u : 1u);
+              else
+                mma_tf32(d, smem_desc(a0 + kk * 32), smem_desc(b0 + kk * 32), idesc,
+                         (first && kk == 0) ? 0u : 1u);
+            }
+          }
+          mma_commit(empty0 + 8 * s);
+          if (++s == nst) s = 0, ++lap;
+        }
+        if (ok) mma_commit(done);
+      }
+    }
+  } else {
+    // epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31, rows of the tile
+    const int quarter = warp & 3, half = (warp - 2) >> 2;
+    const uint32_t lanes = tmem + ((uint32_t)(quarter * 32) << 16);
+    int u = 0;
+    for (int item = blockIdx.x; item < items; item += gridDim.x, ++u) {
+      if (!mbar_wait(done, u & 1, p.err)) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const int chunk = item % p.nchunks, m_tile = item / p.nchunks % p.mt;
+      const int ks = item / (p.mt * p.nchunks);
+      const int row = m_tile * BM + quarter * 32 + lane;
+      // 64 contiguous bytes of this thread's row per group (Np, BNc and c0 are
+      // multiples of 16 floats, so the row segment is 64-byte aligned)
+      float* out = p.part + ((size_t)ks * p.M + row) * p.Np + (size_t)chunk * BNc;
+      auto load = [&](int c0, float (&v)[16]) {
+        uint32_t r[16], q[16];
+        tmem_ld16x2(lanes + (uint32_t)c0, lanes + acc1 + (uint32_t)c0, r, q);
         // one rounded addition joins the two accumulators
-        float v[16];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] = __fadd_rn(__uint_as_float(r[i]), __uint_as_float(q[i]));
+        for (int i = 0; i < 16; ++i)
+          v[i] = __fadd_rn(__uint_as_float(r[i]), __uint_as_float(q[i]));
+      };
+      auto store = [&](int c0, const float (&v)[16]) {
         float4* o4 = reinterpret_cast<float4*>(out + c0);
 #pragma unroll
         for (int i = 0; i < 4; ++i)
           o4[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+      };
+      if (item + (int)gridDim.x >= items) {
+        // nothing waits for the accumulators: a short loop (the one below, unrolled,
+        // costs a launch of one item per CTA 1 us of instruction fetches)
+#pragma unroll 1
+        for (int c0 = half * 16; c0 < BNc; c0 += 32) {
+          float v[16];
+          load(c0, v);
+          if (row < p.M) store(c0, v);
+        }
+        break;
+      }
+      float v[MMA_GROUPS][16];
+#pragma unroll
+      for (int g = 0; g < MMA_GROUPS; ++g)
+        if ((2 * g + half) * 16 < BNc) load((2 * g + half) * 16, v[g]);
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(drained) : "memory");
+      if (row < p.M) {
+#pragma unroll
+        for (int g = 0; g < MMA_GROUPS; ++g)
+          if ((2 * g + half) * 16 < BNc) store((2 * g + half) * 16, v[g]);
       }
     }
   }
+  __syncwarp();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0)
@@ -1139,17 +1218,21 @@ ctm_status run_mma(SplitCtx* sc, const void* As, const void* Bs, int M, int Kp,
   p.BNc = BNc;
   p.kb_total = kb_total;
   p.kb_split = kb_split;
+  p.mt = mt;
+  p.nchunks = nchunks;
+  p.nks = nks;
   p.part = sc->part;
   p.err = sc->err;
   const int ns = ns_of(sc);
-  const size_t smem = 1024 + (size_t)STAGES * (ns * A_SLICE_BYTES + ns * (size_t)BNc * KROW) +
-                      (2 * STAGES + 1) * 8 + 16;
+  const size_t stage = ns * A_SLICE_BYTES + ns * (size_t)BNc * KROW;
+  p.stages = (int)std::min<size_t>(MAX_STAGES, STAGE_SMEM / stage);
+  const size_t smem = 1024 + p.stages * stage;
   static size_t configured_bf16 = 0, configured_tf32 = 0;
   const void* kfn = sc->tf32 ? (const void*)split_mma_kernel<FmtTF32>
                              : (const void*)split_mma_kernel<FmtBF16>;
   if (raise_smem(kfn, sc->tf32 ? configured_tf32 : configured_bf16, smem) != cudaSuccess)
     return sfail(sc, CTM_ECUDA, "cannot reserve shared memory for the tensor-core kernel");
-  dim3 grid(mt, nchunks, nks);
+  const unsigned grid = (unsigned)std::min<long>(152, (long)mt * nchunks * nks);
   if (sc->prof && sc->ev_used + 2 > sc->ev.size()) {
     // every launch of the profiled region is timed: the event pool grows
     const size_t old = sc->ev.size();
@@ -1162,8 +1245,8 @@ ctm_status run_mma(SplitCtx* sc, const void* As, const void* Bs, int M, int Kp,
   }
   const bool timed = sc->prof && sc->ev_used + 2 <= sc->ev.size();
   if (timed) cudaEventRecord(sc->ev[sc->ev_used], s);
-  if (sc->tf32) split_mma_kernel<FmtTF32><<<grid, 128, smem, s>>>(ta, tb, p);
-  else split_mma_kernel<FmtBF16><<<grid, 128, smem, s>>>(ta, tb, p);
+  if (sc->tf32) split_mma_kernel<FmtTF32><<<grid, MMA_THREADS, smem, s>>>(ta, tb, p);
+  else split_mma_kernel<FmtBF16><<<grid, MMA_THREADS, smem, s>>>(ta, tb, p);
   if (timed) {
     cudaEventRecord(sc->ev[sc->ev_used + 1], s);
     sc->ev_used += 2;

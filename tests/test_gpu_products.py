@@ -73,33 +73,36 @@ def test_corner_apply_fp64(d, D, chi, p, cplx, herm):
 # side, with a last group of pairs that is not full and blocks that run one and
 # several steps. Each of the three slice products sums at most 8 K blocks of four
 # matrix instructions in fp32 and keeps values to a few units of 2^-24 (38 in
-# all); the absorption is two fp32 sums of D^2 and d D^2 complex terms between
-# three roundings. The tolerance is the sum of these times 2^-24 times the
-# contraction of absolute values.
-@pytest.mark.parametrize("d,D,chi,cplx", [
-    (2, 4, 25, True),     # 24 pairs a block: fewer blocks than SMs, the last with one pair
-    (3, 4, 62, False),    # a second step for some blocks
-    (2, 5, 25, True),     # 12 pairs a block
-    (1, 5, 45, False),
-    (2, 6, 25, True),     # 4 pairs a block, two steps
-    (2, 6, 37, False),    # 1369 pairs: three steps, both X buffers filled again
+# all; tf32: 64 instructions and 12 units, 80 in all); the absorption is two fp32
+# sums of D^2 and d D^2 complex terms between three roundings. The tolerance is
+# the sum of these times 2^-24 times the contraction of absolute values.
+@pytest.mark.parametrize("d,D,chi,p,prec,cplx", [
+    (2, 4, 25, 5, "BF16", True),     # 24 pairs a block: fewer blocks than SMs, the last with one pair
+    (3, 4, 62, 5, "BF16", False),    # a second step for some blocks
+    (2, 5, 25, 5, "BF16", True),     # 12 pairs a block
+    (1, 5, 45, 5, "BF16", False),
+    (2, 6, 25, 5, "BF16", True),     # 4 pairs a block, two steps
+    (2, 6, 37, 5, "BF16", False),    # 1369 pairs: three steps, both X buffers filled again
+    (1, 6, 25, 600, "BF16", True),    # 625 columns: more slice products than CTAs
+    (1, 6, 26, 600, "TF32", False),
+    (1, 5, 25, 3, "TF32", True),      # N = 625: odd, the slices' second half misaligned
 ])
-def test_corner_apply_split(d, D, chi, cplx):
+@pytest.mark.parametrize("herm", [False, True])
+def test_corner_apply_split(d, D, chi, p, prec, cplx, herm):
     rng = np.random.default_rng(10 * D + chi)
     A = _normal(rng, (d, D, D, D, D), cplx)
     C = _normal(rng, (4, 1, chi, chi), cplx)
     T = _normal(rng, (4, 1, chi, chi, D, D), cplx)
-    opts = pkg.ctm_default_opts(p=5, precision=pkg.CTM_PREC_SPLIT_BF16)
+    opts = pkg.ctm_default_opts(p=p, precision=getattr(pkg, "CTM_PREC_SPLIT_" + prec))
     ctx = pkg.ctm_init(1, 1, [A], d, D, chi, cplx=cplx, opts=opts)
     ctx.ctm_set_env(C, T)
     Z = _normal(rng, (ctx.N, ctx.k), cplx)
-    out = ctx.ctm_corner_apply(0, 0, 0, 1, Z)
+    out = ctx.ctm_corner_apply(0, 0, 0, 1, Z, herm=herm)
     ctx.ctm_free()
     a = (A, np.conj(A), C[0, 0], T[0, 0], T[3, 0])
-    ref = _corner(*a) @ Z
-    bound = _corner(*map(np.abs, a)) @ np.abs(Z)
-    if cplx:
-        bound = 4 * bound
-    tol = (3 * 38 + 2 * D * D + 2 * d * D * D + 3) * 2.0 ** -24
+    Q, Qa = _corner(*a), _corner(*map(np.abs, a))
+    ref = (Q.conj().T if herm else Q) @ Z
+    bound = (4 if cplx else 1) * (Qa.T if herm else Qa) @ np.abs(Z)
+    tol = (3 * (38 if prec == "BF16" else 80) + 2 * D * D + 2 * d * D * D + 3) * 2.0 ** -24
     assert np.isfinite(out).all()
     assert np.max(np.abs(out - ref) / bound) < tol
