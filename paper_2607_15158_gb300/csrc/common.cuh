@@ -21,6 +21,13 @@ typedef double2 cplx;
 __host__ __device__ __forceinline__ float f32_of(double x) {
 #ifdef __CUDA_ARCH__
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  // results in the normal range: the low nine exponent bits and the 23 kept
+  // bits are one funnel shift, rebiasing is one addition modulo 2^32
+  if ((hi & 0x7fffffffu) - 0x38100000u < 0x47f00000u - 0x38100000u) {
+    unsigned u = __funnelshift_l(lo, hi, 3);
+    u += (lo << 3) + (u & 1u) > 0x80000000u ? 0x40000001u : 0x40000000u;
+    return __uint_as_float((u & 0x7fffffffu) | (hi & 0x80000000u));
+  }
 #else
   uint64_t b;
   memcpy(&b, &x, 8);

@@ -1024,7 +1024,7 @@ ctm_status move_impl(ctm_ctx* c, int r) {
       }
       if (c->split && !c->exact) {
         PhaseScope ps(c, PH_SLICE);
-        const ctm_status st = split_prepare_corners(c->split, c->Q, c->N, pre ? 0x9u : 0xFu,
+        const ctm_status st = split_prepare_corners(c->split, c->Q, c->N, pre ? 0x9u : 0xFu, 3u,
                                                     c->stream, &c->launches);
         if (st != CTM_OK) return fail(c, st, split_last_error(c->split));
       }
@@ -1051,7 +1051,7 @@ ctm_status move_impl(ctm_ctx* c, int r) {
           if (c->split && !c->exact) {
             PhaseScope ps(c, PH_SLICE);
             const ctm_status st =
-                split_prepare_corners(c->split, c->Q, c->N, 0x6u, c->stream, &c->launches);
+                split_prepare_corners(c->split, c->Q, c->N, 0x6u, 3u, c->stream, &c->launches);
             if (st != CTM_OK) return fail(c, st, split_last_error(c->split));
           }
           prefetched[y] = 1;
@@ -2370,8 +2370,8 @@ ctm_status ctm_corner_apply(ctm_ctx* c, ctm_dir dir, int x, int y, int i, int he
   const size_t Nk = (size_t)c->N * c->k;
   CK(enlarged_corner(c, r, i - 1, x, y, c->Q[i - 1]));
   if (c->split) {
-    const ctm_status st = split_prepare_corners(c->split, c->Q, c->N, 1u << (i - 1), c->stream,
-                                                &c->launches);
+    const ctm_status st = split_prepare_corners(c->split, c->Q, c->N, 1u << (i - 1),
+                                                herm ? 2u : 1u, c->stream, &c->launches);
     if (st != CTM_OK) return fail(c, st, split_last_error(c->split));
   }
   CTM_CUDA_OK(cudaMemcpyAsync(c->Z[0], Z_in, Nk * c->es, cudaMemcpyHostToDevice, c->stream));

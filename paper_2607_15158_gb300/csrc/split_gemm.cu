@@ -36,6 +36,7 @@
 #include <cstdio>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
@@ -449,59 +450,143 @@ __device__ __forceinline__ void put_digits(__nv_bfloat16* out, long slice, long 
 }
 
 // A slices: out[s][m][kr], kr < K: Re op(A)(m, kr); K <= kr < 2K: Im
-// (complex); zero up to Kp. A 32 x 32 shared tile of op(A) is read along A's
-// contiguous axis (rows for op N / R, columns for op T / C) and each element
-// is read once and written to both halves.
-template <typename T, typename F>
-__global__ void prep_a_kernel(const T* A, long lda, int op, int M, int K, int Kp,
-                              typename SliceT<F>::T* out) {
+// (complex); zero up to Kp. The stored matrix (R x C, row-major) is read once, in
+// PA x PA blocks, and each element sliced once; "direct" takes rows m = r and
+// kr = c (op N and, conjugated, R), "trans" rows m = c and kr = r (op T and C),
+// and both may be asked for. DRAM bounds it (16 bytes read and 12 written per
+// complex element and orientation), so eight
+// loads of a thread are in flight and the slices leave in eight bytes a lane. Both
+// orientations of a complex 5184 x 5184 corner: 235 us (153 at the copy rate;
+// two readings in 32 x 32 blocks with two-byte stores 310), one: 169 (156); at
+// 2880 x 2880 72 (102), one 53.
+struct PrepOut {
+  void* out;   // null: not wanted
+  int cj;      // conjugate
+};
+constexpr int PA_THREADS = 256;
+
+// one slice of a value: the parts (re, im) side by side, so that both are rounded
+// to bf16 by one instruction and stored by one
+template <typename S, int PARTS>
+struct alignas(sizeof(S) * PARTS) Cell { S p[PARTS]; };
+
+__device__ __forceinline__ void cells_of(FmtBF16, cplx x, Cell<__nv_bfloat16, 2>* v) {
+  float re = f32_of(x.x), im = f32_of(x.y);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const __nv_bfloat162 s = __floats2bfloat162_rn(re, im);
+    v[i].p[0] = s.x;
+    v[i].p[1] = s.y;
+    re -= __low2float(s);
+    im -= __high2float(s);
+  }
+}
+__device__ __forceinline__ void cells_of(FmtBF16, double x, Cell<__nv_bfloat16, 1>* v) {
+  __nv_bfloat16 s[3];
+  slices_of(FmtBF16(), x, s);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) v[i].p[0] = s[i];
+}
+__device__ __forceinline__ void cells_of(FmtTF32, cplx x, Cell<float, 2>* v) {
+  float a[2], b[2];
+  slices_of(FmtTF32(), x.x, a);
+  slices_of(FmtTF32(), x.y, b);
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    v[i].p[0] = a[i];
+    v[i].p[1] = b[i];
+  }
+}
+__device__ __forceinline__ void cells_of(FmtTF32, double x, Cell<float, 1>* v) {
+  float s[2];
+  slices_of(FmtTF32(), x, s);
+#pragma unroll
+  for (int i = 0; i < 2; ++i) v[i].p[0] = s[i];
+}
+
+template <typename T, typename F, int PA>
+constexpr size_t prep_a_smem() {
+  return (size_t)F::NS * PA * (PA + 1) * (sizeof(T) / 8) * sizeof(typename SliceT<F>::T);
+}
+
+template <typename T, typename F, int PA>
+__global__ void __launch_bounds__(PA_THREADS)
+    prep_a_kernel(const T* __restrict__ A, long lda, int R, int C, int KpD, int KpT, PrepOut direct,
+                  PrepOut trans) {
   using S = typename SliceT<F>::T;
-  __shared__ T tile[32][33];
-  constexpr bool cx = sizeof(T) == 16;
-  const int Kr = cx ? 2 * K : K;
-  const long slice = (long)M * Kp;
-  const int tiles_k = (K + 31) / 32, tiles_m = (M + 31) / 32;
-  const bool trans = (op == OP_T || op == OP_C);
-  const bool cj = (op == OP_C || op == OP_R);
-  for (int t = blockIdx.x; t < tiles_k * tiles_m; t += gridDim.x) {
-    const int k0 = (t % tiles_k) * 32, m0 = (t / tiles_k) * 32;
-    // tile[m - m0][kk - k0] = op(A)(m, kk) before conjugation
-    for (int yy = threadIdx.y; yy < 32; yy += 8) {
-      if (!trans) {
-        const int m = m0 + yy, kk = k0 + threadIdx.x;
-        tile[yy][threadIdx.x] = (m < M && kk < K) ? A[(long)m * lda + kk] : zero_of(T());
-      } else {
-        const int kk = k0 + yy, m = m0 + threadIdx.x;
-        tile[threadIdx.x][yy] = (m < M && kk < K) ? A[(long)kk * lda + m] : zero_of(T());
+  constexpr int PARTS = sizeof(T) / 8, W = 8 / sizeof(S), PA_LD = PA + 1;
+  using CellT = Cell<S, PARTS>;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  CellT* tile = reinterpret_cast<CellT*>(smem_raw);   // [slice][PA][PA_LD]
+  const int tc = (C + PA - 1) / PA, tr = (R + PA - 1) / PA;
+  for (int t = blockIdx.x; t < tc * tr; t += gridDim.x) {
+    const int c0 = (t % tc) * PA, r0 = (t / tc) * PA;
+    constexpr int STEP = PA_THREADS / PA, U = PA / STEP < 8 ? PA / STEP : 8;
+    const int lc = threadIdx.x % PA, lr = threadIdx.x / PA;
+#pragma unroll 1
+    for (int b = 0; b < PA; b += U * STEP) {
+      T v[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int r = r0 + lr + b + u * STEP, c = c0 + lc;
+        v[u] = r < R && c < C ? __ldcs(A + (long)r * lda + c) : zero_of(T());
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        CellT sv[F::NS];
+        cells_of(F(), v[u], sv);
+#pragma unroll
+        for (int i = 0; i < F::NS; ++i) tile[(i * PA + lr + b + u * STEP) * PA_LD + lc] = sv[i];
       }
     }
     __syncthreads();
-    for (int yy = threadIdx.y; yy < 32; yy += 8) {
-      const int m = m0 + yy, kk = k0 + threadIdx.x;
-      if (m < M && kk < K) {
-        const T v = tile[yy][threadIdx.x];
-        S sv[3];
-        if constexpr (cx) {
-          slices_of(F(), v.x, sv);
-          put_slices<F>(out, slice, (long)m * Kp + kk, sv, false);
-          slices_of(F(), v.y, sv);
-          put_slices<F>(out, slice, (long)m * Kp + K + kk, sv, cj);
-        } else {
-          slices_of(F(), v, sv);
-          put_slices<F>(out, slice, (long)m * Kp + kk, sv, false);
+    // rows of the output, eight bytes a lane and part: W slice values
+    auto write = [&](const PrepOut& w, auto tr_, int m0, int M, int k0, int K, int Kp) {
+      S* out = static_cast<S*>(w.out);
+      const long slice = (long)M * Kp;
+      constexpr int LPR = PA / W;   // lanes a row
+      const int k = threadIdx.x % LPR * W, kc = k0 + k;
+      const bool whole = kc + W <= K, cj = w.cj != 0, even = K % W == 0;
+#pragma unroll 2
+      for (int i = threadIdx.x / LPR; i < F::NS * PA; i += PA_THREADS / LPR) {
+        const int sl = i / PA, m = i % PA;
+        const CellT* src = tile + sl * PA * PA_LD;
+        CellT e[W];
+#pragma unroll
+        for (int x = 0; x < W; ++x)
+          e[x] = decltype(tr_)::value ? src[(k + x) * PA_LD + m] : src[m * PA_LD + k + x];
+        if (m0 + m < M) {
+          S* dst = out + sl * slice + (long)(m0 + m) * Kp + kc;
+#pragma unroll
+          for (int q = 0; q < PARTS; ++q, dst += K) {
+            __align__(8) S o[W];
+#pragma unroll
+            for (int x = 0; x < W; ++x) o[x] = q == 1 && cj ? negv(e[x].p[q]) : e[x].p[q];
+            if (whole && (q == 0 || even)) {
+              *reinterpret_cast<uint2*>(dst) = *reinterpret_cast<const uint2*>(o);
+            } else {
+#pragma unroll
+              for (int x = 0; x < W; ++x)
+                if (kc + x < K) dst[x] = o[x];
+            }
+          }
         }
       }
-    }
+    };
+    if (direct.out) write(direct, std::false_type(), r0, R, c0, C, KpD);
+    if (trans.out) write(trans, std::true_type(), c0, C, r0, R, KpT);
     __syncthreads();
   }
-  // padding columns kr >= Kr
-  const S z = zero_slice<S>();
-  const S zz[3] = {z, z, z};
-  const int pc = Kp - Kr;
-  const long tid = (long)blockIdx.x * blockDim.x * blockDim.y + threadIdx.y * blockDim.x + threadIdx.x;
-  const long nth = (long)gridDim.x * blockDim.x * blockDim.y;
-  for (long idx = tid; idx < (long)M * pc; idx += nth)
-    put_slices<F>(out, slice, (idx / pc) * Kp + Kr + idx % pc, zz, false);
+  // padding columns
+  const long tid = (long)blockIdx.x * blockDim.x + threadIdx.x, nth = (long)gridDim.x * blockDim.x;
+  auto pad = [&](const PrepOut& w, int M, int K, int Kp) {
+    S* out = static_cast<S*>(w.out);
+    const int Kr = PARTS * K, pc = Kp - Kr;
+    for (long idx = tid; idx < (long)F::NS * M * pc; idx += nth)
+      out[idx / pc * Kp + Kr + idx % pc] = zero_slice<S>();
+  };
+  if (direct.out) pad(direct, R, C, KpD);
+  if (trans.out) pad(trans, C, R, KpT);
 }
 
 // B slices (K-major rows = output real columns): out[s][j][kr] = B_emb[kr][j]
@@ -584,9 +669,9 @@ __device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float x) {
 // rounding of its low part, ~2^-48 relative.
 template <typename T>
 __global__ void reduce_kernel(const float* part, int nks, int M, int N, int Np, T* C, long ldc) {
-  for (long idx = blockIdx.x * (long)blockDim.x + threadIdx.x; idx < (long)M * N;
-       idx += (long)gridDim.x * blockDim.x) {
-    const int m = (int)(idx / N), j = (int)(idx % N);
+  for (unsigned idx = blockIdx.x * blockDim.x + threadIdx.x; idx < (unsigned)M * (unsigned)N;
+       idx += gridDim.x * blockDim.x) {
+    const unsigned m = idx / (unsigned)N, j = idx % (unsigned)N;
     const float* row = part + (size_t)m * Np + j;
     const size_t sstep = (size_t)M * Np;
     float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
@@ -1272,21 +1357,50 @@ ctm_status run_mma(SplitCtx* sc, const void* As, const void* Bs, int M, int Kp,
   return CTM_OK;
 }
 
+template <typename T, typename F, int PA>
+cudaError_t launch_prep_a_tiles(const void* A, long lda, int R, int C, int KpD, int KpT, PrepOut direct,
+                          PrepOut trans, cudaStream_t s) {
+  static size_t configured = 0;
+  constexpr size_t smem = prep_a_smem<T, F, PA>();
+  cudaError_t e = raise_smem((const void*)prep_a_kernel<T, F, PA>, configured, smem);
+  if (e != cudaSuccess) return e;
+  const long tiles = (long)((R + PA - 1) / PA) * ((C + PA - 1) / PA);
+  const unsigned g = (unsigned)std::max<long>(1, std::min<long>(tiles, 152L * 16));
+  prep_a_kernel<T, F, PA><<<g, PA_THREADS, smem, s>>>(static_cast<const T*>(A), lda, R, C, KpD, KpT,
+                                                      direct, trans);
+  return cudaGetLastError();
+}
+
+// blocks of 64 x 64, or of 32 x 32 where those would leave SMs without a block (an
+// edge of 41 x 1025: 17 blocks of 64)
+template <typename T, typename F>
+cudaError_t launch_prep_a(const void* A, long lda, int R, int C, int KpD, int KpT, PrepOut direct,
+                          PrepOut trans, cudaStream_t s) {
+  if ((long)((R + 63) / 64) * ((C + 63) / 64) < 152)
+    return launch_prep_a_tiles<T, F, 32>(A, lda, R, C, KpD, KpT, direct, trans, s);
+  return launch_prep_a_tiles<T, F, 64>(A, lda, R, C, KpD, KpT, direct, trans, s);
+}
+
+// slices of the stored R x C matrix A in either orientation
+ctm_status prep_a_both(SplitCtx* sc, const void* A, long lda, int R, int C, int KpD, int KpT,
+                       PrepOut direct, PrepOut trans, cudaStream_t s, long* launches) {
+  cudaError_t e;
+  if (sc->tf32)
+    e = sc->cx ? launch_prep_a<cplx, FmtTF32>(A, lda, R, C, KpD, KpT, direct, trans, s)
+               : launch_prep_a<double, FmtTF32>(A, lda, R, C, KpD, KpT, direct, trans, s);
+  else
+    e = sc->cx ? launch_prep_a<cplx, FmtBF16>(A, lda, R, C, KpD, KpT, direct, trans, s)
+               : launch_prep_a<double, FmtBF16>(A, lda, R, C, KpD, KpT, direct, trans, s);
+  if (launches) ++*launches;
+  return e == cudaSuccess ? CTM_OK : sfail(sc, CTM_ECUDA, "slice launch failed");
+}
+
 ctm_status prep_a(SplitCtx* sc, const void* A, long lda, int op, int M, int K, int Kp,
                   void* out, cudaStream_t s, long* launches) {
-  const long tiles = (long)((K + 31) / 32) * ((M + 31) / 32);
-  const unsigned g = (unsigned)std::max<long>(1, std::min<long>(tiles, 152L * 16));
-  const dim3 b(32, 8);
-  if (sc->tf32) {
-    if (sc->cx) prep_a_kernel<cplx, FmtTF32><<<g, b, 0, s>>>((const cplx*)A, lda, op, M, K, Kp, (float*)out);
-    else prep_a_kernel<double, FmtTF32><<<g, b, 0, s>>>((const double*)A, lda, op, M, K, Kp, (float*)out);
-  } else {
-    __nv_bfloat16* o = static_cast<__nv_bfloat16*>(out);
-    if (sc->cx) prep_a_kernel<cplx, FmtBF16><<<g, b, 0, s>>>((const cplx*)A, lda, op, M, K, Kp, o);
-    else prep_a_kernel<double, FmtBF16><<<g, b, 0, s>>>((const double*)A, lda, op, M, K, Kp, o);
-  }
-  if (launches) ++*launches;
-  return cudaGetLastError() == cudaSuccess ? CTM_OK : sfail(sc, CTM_ECUDA, "slice launch failed");
+  const PrepOut none{nullptr, 0}, o{out, op == OP_C || op == OP_R};
+  if (op == OP_T || op == OP_C)
+    return prep_a_both(sc, A, lda, K, M, Kp, Kp, none, o, s, launches);
+  return prep_a_both(sc, A, lda, M, K, Kp, Kp, o, none, s, launches);
 }
 
 ctm_status prep_b(SplitCtx* sc, const void* B, long ldb, int op, int K, int N, int Kp, int Np,
@@ -1373,25 +1487,26 @@ void split_destroy(SplitCtx* sc) {
 }
 
 ctm_status split_prepare_corners(SplitCtx* sc, void* const* Q, int N, unsigned mask,
-                                 cudaStream_t s, long* launches) {
+                                 unsigned ops, cudaStream_t s, long* launches) {
   const int Kr = sc->cx ? 2 * N : N;
   const int Kp = pad_to(Kr, ke_of(sc));
   sc->corner_Kp = Kp;
   for (int i = 0; i < 4; ++i) {
     if (!(mask >> i & 1u)) continue;
     sc->corner_src[i] = Q[i];
-    for (int o = 0; o < 2; ++o) {
-      if (!sc->cslices[i][o]) {
+    for (int o = 0; o < 2; ++o)
+      if ((ops >> o & 1u) && !sc->cslices[i][o]) {
         if (cudaMalloc(&sc->cslices[i][o], (size_t)ns_of(sc) * N * Kp * eb_of(sc)) != cudaSuccess) {
           cudaGetLastError();
           return sfail(sc, CTM_ENOMEM, "corner slice allocation failed");
         }
         ++sc->generation;
       }
-      const int op = o == 0 ? OP_N : (sc->cx ? OP_C : OP_T);
-      ctm_status st = prep_a(sc, Q[i], N, op, N, N, Kp, sc->cslices[i][o], s, launches);
-      if (st != CTM_OK) return st;
-    }
+    // both orientations from one reading
+    const PrepOut direct{ops & 1u ? sc->cslices[i][0] : nullptr, 0};
+    const PrepOut trans{ops & 2u ? sc->cslices[i][1] : nullptr, sc->cx ? 1 : 0};
+    ctm_status st = prep_a_both(sc, Q[i], N, N, N, Kp, Kp, direct, trans, s, launches);
+    if (st != CTM_OK) return st;
   }
   return CTM_OK;
 }

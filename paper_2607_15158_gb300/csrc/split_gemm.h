@@ -20,9 +20,10 @@ ctm_status split_create(SplitCtx** out, bool cx, bool tf32, int N, int k, int* e
 void split_destroy(SplitCtx* sc);
 
 // Slice the fp64 corners Q[i] (N x N) whose bit i is set in mask into bf16
-// operands, in both orientations (for op(Q) = Q and op(Q) = Q^H).
+// operands, in the orientations that ops asks for: bit 0 op(Q) = Q, bit 1
+// op(Q) = Q^H.
 ctm_status split_prepare_corners(SplitCtx* sc, void* const* Q, int N, unsigned mask,
-                                 cudaStream_t s, long* launches);
+                                 unsigned ops, cudaStream_t s, long* launches);
 
 // Let sc apply the corners that src has prepared (and will prepare again): the
 // slices stay src's, and the caller orders their use.
