@@ -50,8 +50,7 @@ namespace {
 constexpr int BM = 128;          // rows per CTA (tcgen05 M)
 constexpr int BK = 64;           // bf16 K elements per stage (128 bytes)
 constexpr int KROW = 128;        // bytes of one staged K row (either format)
-constexpr int STAGES = 2;        // of the exact-digit kernel
-constexpr int MAX_STAGES = 4;    // of the slice kernel: as many as shared memory holds
+constexpr int MAX_STAGES = 4;    // K blocks staged: as many as shared memory holds
 constexpr size_t STAGE_SMEM = 225 * 1024;   // shared memory for stages
 constexpr int MAX_BNC = 160;     // columns per CTA
 constexpr int A_SLICE_BYTES = BM * KROW;     // 16 KB
@@ -160,18 +159,6 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
       "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
       : "memory");
 }
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
-      "%11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
-        "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr)
-      : "memory");
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
 // 16 columns from each of two accumulators
 __device__ __forceinline__ void tmem_ld16x2(uint32_t ta, uint32_t tb, uint32_t (&r)[16],
                                             uint32_t (&q)[16]) {
@@ -722,53 +709,75 @@ __global__ void reduce_kernel(const float* part, int nks, int M, int N, int Np, 
 //     scaled by 2^-7w, into an unevaluated fp32 pair (TwoSum) per output;
 //     the pairs of the K splits are summed the same way and the result is
 //     hi + lo scaled by 2^(E_m + E_n - 14), to about 2^-48 relative.
-// The operand digits stage through shared memory in three quarter stages
-// per K block (digits 0-3 of A with 0-3 of B, 0-3 with 4-7, 4-7 with 0-3),
-// which cover every product of weight <= 7.
+// One matrix instruction multiplies digit s of A with up to four digits t of B: B's
+// digits lie one after the other in shared memory, and so do the accumulators of
+// the weights s + t in tensor memory, so the digits of B are simply more columns
+// (N up to 256; all sums are exact integers, so their order is free).
+// The digits are staged in four groups, each with its own buffer: A's 0-3 and
+// 4-7, B's 0-3 and 4-7. A K block uses (A 0-3, B 4-7), (A 0-3, B 0-3) and
+// (A 4-7, B 0-3), in this order: every weight is started by digit 0 of A, and the
+// groups are free again one after the other, so that the next K block's loads
+// run beside the rest of this one's products.
+// A persistent grid: CTA b takes the work items b, b + gridDim.x, ... (a split of
+// a tile each), the loads running ahead into the next item. Complex, against 36
+// single digit products of N = 64 per K block from three staged quarters (a third
+// more loads), one item per CTA and four draining warps: 1024 x 1024 times 69
+// columns 64 us -> 31, 65536 x 16 times 16 63 -> 26, one K block 24 -> 14.
 constexpr int OZ_NS = 8;          // digits per operand
 constexpr int OZ_BITS = 7;        // bits per digit
-constexpr int OZ_BN = 64;         // output columns per CTA (one accumulator width)
+constexpr int OZ_BN = 64;         // output columns per CTA (one accumulator width) at most
 constexpr int OZ_KB_DRAIN = 2;    // K blocks per exact accumulation
-constexpr int OZ_Q_BYTES = 4 * A_SLICE_BYTES + 4 * OZ_BN * KROW;   // 96 KB per quarter stage
+constexpr int OZ_GA = 4 * A_SLICE_BYTES, OZ_GB = 4 * OZ_BN * KROW;   // bytes of a group
+constexpr int OZ_THREADS = 320, OZ_EPI = 8;
 
 struct OzParams {
   int M;          // output rows (real-embedded)
   int Np;         // padded output columns
+  int BNc;        // output columns per CTA, a multiple of 16, <= OZ_BN
   int kb_total;   // K blocks of 64
-  int kb_split;   // K blocks per CTA
+  int kb_split;   // K blocks per work item
+  int mt, nchunks, nks;   // work items: row tiles x column chunks x splits
   float2* part;   // [nks][M][Np] (hi, lo)
   int* err;
 };
 
-__global__ void __launch_bounds__(192, 1)
+// two_sum_acc of scale * x, scale a power of two (the product is exact)
+__device__ __forceinline__ void two_sum_scaled(float& hi, float& lo, float x, float scale) {
+  const float s = fmaf(x, scale, hi);
+  const float bb = s - hi;
+  const float e = (hi - (s - bb)) + fmaf(x, scale, -bb);
+  hi = s;
+  lo += e;
+}
+
+__global__ void __launch_bounds__(OZ_THREADS, 1)
     oz_mma_kernel(const __grid_constant__ CUtensorMap tmA,
                   const __grid_constant__ CUtensorMap tmB, OzParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STAGES * OZ_Q_BYTES);
-  // full[2], empty[2], chunk done, drained
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 2);
-  const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + STAGES),
-                 cdone = smem_u32(bars + 2 * STAGES), drained = smem_u32(bars + 2 * STAGES + 1);
+  // groups in the order of their loads: B 4-7, A 0-3, B 0-3, A 4-7
+  const uint32_t base = smem_u32(smem);
+  const uint32_t gaddr[4] = {base + 2 * OZ_GA, base, base + 2 * OZ_GA + OZ_GB, base + OZ_GA};
+  __shared__ uint64_t bars[10];
+  __shared__ uint32_t tmem_slot;
+  const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + 4), cdone = smem_u32(bars + 8),
+                 drained = smem_u32(bars + 9);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m_tile = blockIdx.x, chunk = blockIdx.y, ks = blockIdx.z;
-  const int kb0 = ks * p.kb_split;
-  const int nkb = min(p.kb_split, p.kb_total - kb0);
-  const int nchunks = (nkb + OZ_KB_DRAIN - 1) / OZ_KB_DRAIN;
+  const int BN = p.BNc;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) {
-      mbar_init(full0 + 8 * s, 1);
-      mbar_init(empty0 + 8 * s, 1);
+    for (int g = 0; g < 4; ++g) {
+      mbar_init(full0 + 8 * g, 1);
+      mbar_init(empty0 + 8 * g, 1);
     }
     mbar_init(cdone, 1);
-    mbar_init(drained, 4);
+    mbar_init(drained, OZ_EPI);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                     smem_u32(tmem_slot)),
+                     smem_u32(&tmem_slot)),
                  "r"(512)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -776,115 +785,154 @@ __global__ void __launch_bounds__(192, 1)
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = *tmem_slot;
-  __shared__ int failed;
-  if (threadIdx.x == 0) failed = 0;
-  __syncthreads();
-  // quarter q: A digits from a_off, B digits from b_off
-  const int q_a[3] = {0, 0, 4}, q_b[3] = {0, 4, 0};
+  const uint32_t tmem = tmem_slot;
+  const int items = p.mt * p.nchunks * p.nks;
+  auto kblocks = [&](int item) {
+    return min(p.kb_split, p.kb_total - item / (p.mt * p.nchunks) * p.kb_split);
+  };
 
-  if (nkb > 0 && warp == 0 && lane == 0) {
-    // TMA producer: three quarter stages per K block
-    for (int kb = 0; kb < nkb; ++kb) {
-      for (int q = 0; q < 3; ++q) {
-        const int it = 3 * kb + q, s = it % STAGES;
-        if (it >= STAGES && !mbar_wait(empty0 + 8 * s, ((it / STAGES) - 1) & 1, p.err)) {
-          failed = 1;
-          break;
+  if (warp == 0) {
+    if (lane == 0) {
+      // TMA producer
+      bool ok = true;
+      int t = 0, g = 0;   // K blocks and groups of the current one loaded
+      for (int item = blockIdx.x; item < items && ok; item += gridDim.x) {
+        const int chunk = item % p.nchunks, m_tile = item / p.nchunks % p.mt;
+        const int kb0 = item / (p.mt * p.nchunks) * p.kb_split, nkb = kblocks(item);
+        for (int kb = 0; kb < nkb && ok; ++kb) {
+          const int kx = (kb0 + kb) * BK;
+          for (g = 0; g < 4; ++g) {
+            if (t > 0 && !mbar_wait(empty0 + 8 * g, (t - 1) & 1, p.err)) {
+              ok = false;
+              break;
+            }
+            const bool is_a = g & 1;
+            const uint32_t full = full0 + 8 * g, step = is_a ? A_SLICE_BYTES : BN * KROW;
+            mbar_expect_tx(full, 4 * step);
+            const int d0 = g == 0 || g == 3 ? 4 : 0;
+            for (int i = 0; i < 4; ++i)
+              tma_load_3d(gaddr[g] + i * step, is_a ? &tmA : &tmB, kx,
+                          is_a ? m_tile * BM : chunk * BN, d0 + i, full);
+          }
+          if (ok) ++t, g = 0;
         }
-        const uint32_t full = full0 + 8 * s;
-        mbar_expect_tx(full, OZ_Q_BYTES);
-        uint8_t* st = smem + s * OZ_Q_BYTES;
-        const int kx = (kb0 + kb) * BK;
-        for (int i = 0; i < 4; ++i)
-          tma_load_3d(smem_u32(st + i * A_SLICE_BYTES), &tmA, kx, m_tile * BM, q_a[q] + i, full);
-        for (int i = 0; i < 4; ++i)
-          tma_load_3d(smem_u32(st + 4 * A_SLICE_BYTES + i * OZ_BN * KROW), &tmB, kx,
-                      chunk * OZ_BN, q_b[q] + i, full);
       }
-      if (failed) break;
+      // a CTA that gave up does not end before its copies have landed
+      for (int i = 0; !ok && i < 4; ++i) {
+        const int fills = t + (i < g ? 1 : 0);
+        if (fills > 0) mbar_wait(full0 + 8 * i, (fills - 1) & 1, p.err);
+      }
     }
-  } else if (nkb > 0 && warp == 1 && lane == 0) {
-    // MMA issuer: the products of weight <= 7 of each quarter, into the
-    // accumulator of their weight; a chunk of OZ_KB_DRAIN K blocks starts
-    // each accumulator afresh once the epilogue has drained the last one
-    const uint32_t idesc = idesc_bf16(BM, OZ_BN);
+  } else if (warp == 1) {
+    if (lane == 0) {
+      // MMA issuer; a chunk of OZ_KB_DRAIN K blocks starts each accumulator afresh
+      // once the epilogue has drained the last one
+      bool ok = true;
+      int t = 0, cc = 0;
+      // digits d of A (at a) with the first nj of a group of B (at b) into the weights from w
+      auto mma = [&](uint32_t a, uint32_t b, int nj, int w, bool fresh) {
+        const uint32_t idesc = idesc_bf16(BM, nj * BN);
+        const uint64_t da = smem_desc(a), db = smem_desc(b);
+        const uint32_t d = tmem + (uint32_t)(w * BN);
+        mma_bf16(d, da, db, idesc, fresh ? 0u : 1u);
+#pragma unroll
+        for (int kk = 1; kk < KROW / 32; ++kk) mma_bf16(d, da + 2 * kk, db + 2 * kk, idesc, 1u);
+      };
+      for (int item = blockIdx.x; item < items && ok; item += gridDim.x) {
+        const int nkb = kblocks(item);
+        for (int kb = 0; kb < nkb && ok; ++kb, ++t) {
+          const bool first = kb % OZ_KB_DRAIN == 0;
+          if (first) {
+            if (cc > 0 && !mbar_wait(drained, (cc - 1) & 1, p.err)) ok = false;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          }
+          for (int q = 0; q < 3 && ok; ++q) {
+            // groups that this quarter is the first to use
+            const int g0 = q == 0 ? 0 : q + 1;
+            for (int g = g0; g <= q + 1 && ok; ++g) ok = mbar_wait(full0 + 8 * g, t & 1, p.err);
+            if (!ok) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t a = gaddr[q == 2 ? 3 : 1], b = gaddr[q == 0 ? 0 : 2];
+#pragma unroll 1
+            for (int i = 0; i < 4; ++i)
+              mma(a + i * A_SLICE_BYTES, b, q == 1 ? 4 : 4 - i, q == 1 ? i : 4 + i,
+                  first && i == 0 && q < 2);
+            if (q == 0) {
+              mma_commit(empty0);
+            } else if (q == 1) {
+              mma_commit(empty0 + 8);
+            } else {
+              mma_commit(empty0 + 16);
+              mma_commit(empty0 + 24);
+            }
+          }
+          if (ok && (kb % OZ_KB_DRAIN == OZ_KB_DRAIN - 1 || kb == nkb - 1)) {
+            mma_commit(cdone);
+            ++cc;
+          }
+        }
+      }
+    }
+  } else {
+    // epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 and alternate groups of
+    // 16 columns
+    const int quarter = warp & 3, half = (warp - 2) >> 2;
+    const uint32_t lanes = tmem + ((uint32_t)(quarter * 32) << 16);
     bool ok = true;
-    for (int c = 0; c < nchunks && ok; ++c) {
-      if (c > 0) {
-        if (!mbar_wait(drained, (c - 1) & 1, p.err)) {
+    int cc = 0;
+    for (int item = blockIdx.x; item < items && ok; item += gridDim.x) {
+      float hi[2][16], lo[2][16];
+#pragma unroll
+      for (int g = 0; g < 2; ++g)
+#pragma unroll
+        for (int i = 0; i < 16; ++i) hi[g][i] = lo[g][i] = 0.f;
+      const int nkb = kblocks(item);
+      for (int kb = 0; kb < nkb; kb += OZ_KB_DRAIN, ++cc) {
+        if (!mbar_wait(cdone, cc & 1, p.err)) {
           ok = false;
-          failed = 1;
           break;
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      }
-      unsigned used = 0;   // accumulators written in this chunk
-      const int kbe = min(nkb, (c + 1) * OZ_KB_DRAIN);
-      for (int kb = c * OZ_KB_DRAIN; kb < kbe && ok; ++kb) {
-        for (int q = 0; q < 3; ++q) {
-          const int it = 3 * kb + q, s = it % STAGES;
-          if (!mbar_wait(full0 + 8 * s, (it / STAGES) & 1, p.err)) {
-            ok = false;
-            failed = 1;
-            break;
-          }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t st = smem_u32(smem + s * OZ_Q_BYTES);
-          for (int i = 0; i < 4; ++i) {
-            for (int j = 0; j < 4; ++j) {
-              const int w = q_a[q] + i + q_b[q] + j;
-              if (w >= OZ_NS) continue;
-              const uint32_t a0 = st + i * A_SLICE_BYTES;
-              const uint32_t b0 = st + 4 * A_SLICE_BYTES + j * OZ_BN * KROW;
-              const uint32_t d = tmem + (uint32_t)(w * OZ_BN);
-              const bool fresh = !(used >> w & 1u);
-              used |= 1u << w;
-              for (int kk = 0; kk < KROW / 32; ++kk)
-                mma_bf16(d, smem_desc(a0 + kk * 32), smem_desc(b0 + kk * 32), idesc,
-                         (fresh && kk == 0) ? 0u : 1u);
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+          const int c0 = (2 * g + half) * 16;
+          if (c0 < BN) {
+            float scale = 1.f;
+#pragma unroll 1
+            for (int w = 0; w < OZ_NS; w += 2) {
+              uint32_t r[16], q[16];
+              tmem_ld16x2(lanes + (uint32_t)(w * BN + c0), lanes + (uint32_t)((w + 1) * BN + c0), r, q);
+#pragma unroll
+              for (int i = 0; i < 16; ++i)
+                two_sum_scaled(hi[g][i], lo[g][i], __uint_as_float(r[i]), scale);
+              scale *= 0.0078125f;   // 2^-7
+#pragma unroll
+              for (int i = 0; i < 16; ++i)
+                two_sum_scaled(hi[g][i], lo[g][i], __uint_as_float(q[i]), scale);
+              scale *= 0.0078125f;
             }
           }
-          mma_commit(empty0 + 8 * s);
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(drained) : "memory");
+      }
+      const int chunk = item % p.nchunks, m_tile = item / p.nchunks % p.mt;
+      const int ks = item / (p.mt * p.nchunks);
+      const int row = m_tile * BM + quarter * 32 + lane;
+      if (ok && row < p.M) {
+        float2* out = p.part + ((size_t)ks * p.M + row) * p.Np + (size_t)chunk * BN;
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+          const int c0 = (2 * g + half) * 16;
+          if (c0 < BN) {
+            float4* o4 = reinterpret_cast<float4*>(out + c0);
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+              o4[i] = make_float4(hi[g][2 * i], lo[g][2 * i], hi[g][2 * i + 1], lo[g][2 * i + 1]);
+          }
         }
       }
-      if (ok) mma_commit(cdone);
-    }
-  } else if (warp >= 2 && nkb > 0) {
-    // epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 (its quarter)
-    const int quarter = warp & 3;
-    float hi[OZ_BN], lo[OZ_BN];
-#pragma unroll
-    for (int i = 0; i < OZ_BN; ++i) hi[i] = lo[i] = 0.f;
-    bool ok = true;
-    for (int c = 0; c < nchunks; ++c) {
-      if (!mbar_wait(cdone, c & 1, p.err)) {
-        ok = false;
-        failed = 1;
-        break;
-      }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll
-      for (int c0 = 0; c0 < OZ_BN; c0 += 16) {
-        float scale = 1.f;
-#pragma unroll 1
-        for (int w = 0; w < OZ_NS; ++w) {
-          uint32_t r[16];
-          tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(w * OZ_BN + c0), r);
-#pragma unroll
-          for (int i = 0; i < 16; ++i) two_sum_acc(hi[c0 + i], lo[c0 + i], __uint_as_float(r[i]) * scale);
-          scale *= 0.0078125f;   // 2^-7
-        }
-      }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncwarp();
-      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(drained) : "memory");
-    }
-    const int row = m_tile * BM + quarter * 32 + lane;
-    if (ok && row < p.M) {
-      float2* out = p.part + ((size_t)ks * p.M + row) * p.Np + (size_t)chunk * OZ_BN;
-#pragma unroll
-      for (int i = 0; i < OZ_BN; ++i) out[i] = make_float2(hi[i], lo[i]);
     }
   }
   __syncwarp();
@@ -1571,8 +1619,9 @@ ctm_status oz_gemm(SplitCtx* sc, int opA, const void* A, long lda, int opB, cons
   const int Kr = cx ? 2 * K : K;
   const int Kp = pad_to(Kr, BK);
   const int Nr = cx ? 2 * N : N;
-  const int Np = pad_to(Nr, OZ_BN);
-  const int nchunks = Np / OZ_BN;
+  const int nchunks = (Nr + OZ_BN - 1) / OZ_BN;
+  const int BNc = pad_to((Nr + nchunks - 1) / nchunks, 16);
+  const int Np = nchunks * BNc;
   const int mt = (M + BM - 1) / BM;
   const int kb_total = Kp / BK;
   // about two waves of CTAs, at least OZ_KB_DRAIN K blocks each
@@ -1609,20 +1658,25 @@ ctm_status oz_gemm(SplitCtx* sc, int opA, const void* A, long lda, int opB, cons
   if (launches) *launches += 4;
   CUtensorMap ta, tb;
   if (!make_map(&ta, sc->oz_a, M, Kp, BM, false, OZ_NS) ||
-      !make_map(&tb, sc->oz_b, Np, Kp, OZ_BN, false, OZ_NS))
+      !make_map(&tb, sc->oz_b, Np, Kp, BNc, false, OZ_NS))
     return sfail(sc, CTM_ECUDA, "cuTensorMapEncodeTiled failed");
   OzParams p;
   p.M = M;
   p.Np = Np;
   p.kb_total = kb_total;
   p.kb_split = kb_split;
+  p.BNc = BNc;
+  p.mt = mt;
+  p.nchunks = nchunks;
+  p.nks = nks;
   p.part = static_cast<float2*>(sc->oz_part);
   p.err = sc->err;
-  const size_t smem = 1024 + (size_t)STAGES * OZ_Q_BYTES + (2 * STAGES + 2) * 8 + 16;
+  const size_t smem = 1024 + 2 * OZ_GA + 2 * OZ_GB;
   static size_t configured = 0;
   if (raise_smem((const void*)oz_mma_kernel, configured, smem) != cudaSuccess)
     return sfail(sc, CTM_ECUDA, "cannot reserve shared memory for the fp64-accurate product");
-  oz_mma_kernel<<<dim3(mt, nchunks, nks), 192, smem, s>>>(ta, tb, p);
+  const unsigned grid = (unsigned)std::min<long>(152, tiles * nks);
+  oz_mma_kernel<<<grid, OZ_THREADS, smem, s>>>(ta, tb, p);
   ++sc->oz_launches;
   if (cx)
     oz_reduce_kernel<cplx><<<grid_cap((long)M * N), 256, 0, s>>>(

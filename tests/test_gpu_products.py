@@ -93,7 +93,7 @@ def test_corner_apply_split(d, D, chi, p, prec, cplx, herm):
     A = _normal(rng, (d, D, D, D, D), cplx)
     C = _normal(rng, (4, 1, chi, chi), cplx)
     T = _normal(rng, (4, 1, chi, chi, D, D), cplx)
-    opts = pkg.ctm_default_opts(p=p, precision=getattr(pkg, "CTM_PREC_SPLIT_" + prec))
+    opts = pkg.ctm_default_opts(p=p, prec=getattr(pkg, "CTM_PREC_SPLIT_" + prec))
     ctx = pkg.ctm_init(1, 1, [A], d, D, chi, cplx=cplx, opts=opts)
     ctx.ctm_set_env(C, T)
     Z = _normal(rng, (ctx.N, ctx.k), cplx)
@@ -106,3 +106,23 @@ def test_corner_apply_split(d, D, chi, p, prec, cplx, herm):
     tol = (3 * (38 if prec == "BF16" else 80) + 2 * D * D + 2 * d * D * D + 3) * 2.0 ** -24
     assert np.isfinite(out).all()
     assert np.max(np.abs(out - ref) / bound) < tol
+
+
+# Exact-digit products: widths of 16, 32, 48 and 64 columns per CTA, one and
+# several K blocks (an odd number among them), and more partial sums than CTAs. A
+# digit product drops 2^-53 of the row maximum times the column maximum per term
+# and sums to 2^-48 relative; of a normal sample the maxima are below twenty times
+# the mean product, so 2^-47 of the product of absolute values is a bound.
+@pytest.mark.parametrize("M,N,K,op,cplx", [
+    (20, 8, 50, 0, False),       # one K block, 8 columns
+    (130, 14, 40, 1, True),      # 28 columns, two K blocks
+    (300, 69, 333, 2, True),     # 138 columns: three CTAs of 48
+    (256, 64, 243, 0, False),    # 64 columns
+    (600, 233, 1050, 2, True),   # 466 columns, 33 K blocks: 320 partial sums
+])
+def test_exact_digit_product(M, N, K, op, cplx):
+    rng = np.random.default_rng(M + N)
+    opA, B = _normal(rng, (M, K), cplx), _normal(rng, (K, N), cplx)
+    A = {0: opA, 1: opA.T, 2: opA.conj().T}[op].copy()
+    C = pkg.ctm_gemm_fp64tc(A, B, op)
+    assert (np.abs(C - opA @ B) <= 2.0 ** -47 * (np.abs(opA) @ np.abs(B))).all()
