@@ -430,12 +430,6 @@ __device__ __forceinline__ void put_slices(T* out, long slice, long o, const T* 
 }
 
 
-__device__ __forceinline__ void put_digits(__nv_bfloat16* out, long slice, long o,
-                                           const __nv_bfloat16* d, bool neg) {
-#pragma unroll
-  for (int i = 0; i < 8; ++i) out[i * slice + o] = neg ? __hneg(d[i]) : d[i];
-}
-
 // A slices: out[s][m][kr], kr < K: Re op(A)(m, kr); K <= kr < 2K: Im
 // (complex); zero up to Kp. The stored matrix (R x C, row-major) is read once, in
 // PA x PA blocks, and each element sliced once; "direct" takes rows m = r and
@@ -948,208 +942,183 @@ __device__ __forceinline__ int bexp(double x) {
   return (int)(((unsigned)__double2hiint(x) >> 20) & 0x7ffu);
 }
 
-// the eight signed 7-bit digits of x against the exponent field eb of its
-// row / column maximum: F = trunc(|x| 2^(56 - E)), E = eb - 1022
-__device__ __forceinline__ void oz_digits(double x, int eb, __nv_bfloat16* d) {
+// One operand of an exact-digit product: V vectors (rows of op(A), columns of
+// op(B)) of K entries, stored as rows ("rows", the entries side by side) or as
+// columns of a row-major matrix.
+template <typename T>
+struct OzOperand {
+  const T* p;
+  long ld;
+  int V, K;
+  int rows;          // vectors are stored rows
+  int cj;            // conjugate
+  int* e;            // exponent field of each vector's largest entry
+  __nv_bfloat16* out;   // digits [8][rows of out][Kp]
+  int Vp;            // rows of out: V for A, the padded real columns for B
+  int tiles_c, tiles;   // 32 x 32 blocks of the stored matrix: per row, in all
+};
+constexpr int OZ_T = 32, OZ_PREP = 256, OZ_U = OZ_T * OZ_T / OZ_PREP;
+
+// this thread's four entries of block t: rows r + 8 u, column c
+template <typename T>
+__device__ __forceinline__ void oz_load(const OzOperand<T>& o, int t, int& r, int& c, T (&v)[OZ_U]) {
+  const int R = o.rows ? o.V : o.K, C = o.rows ? o.K : o.V;
+  c = t % o.tiles_c * OZ_T + threadIdx.x % OZ_T;
+  r = t / o.tiles_c * OZ_T + threadIdx.x / OZ_T;
+#pragma unroll
+  for (int u = 0; u < OZ_U; ++u)
+    v[u] = r + 8 * u < R && c < C ? o.p[(long)(r + 8 * u) * o.ld + c] : zero_of(T());
+}
+
+// exponent fields of both operands' vectors: the maximum over each block, one
+// atomicMax per vector and block
+template <typename T>
+__global__ void __launch_bounds__(OZ_PREP) oz_exp_kernel(OzOperand<T> a, OzOperand<T> b) {
+  __shared__ int part[OZ_PREP / 32][32];
+  for (int t = blockIdx.x; t < a.tiles + b.tiles; t += gridDim.x) {
+    const OzOperand<T>& o = t < a.tiles ? a : b;
+    T v[OZ_U];
+    int r, c;
+    oz_load(o, t < a.tiles ? t : t - a.tiles, r, c, v);
+    int e[OZ_U], m = 0;
+#pragma unroll
+    for (int u = 0; u < OZ_U; ++u) {
+      if constexpr (sizeof(T) == 16) e[u] = max(bexp(v[u].x), bexp(v[u].y));
+      else e[u] = bexp(v[u]);
+      m = max(m, e[u]);
+    }
+    if (o.rows) {
+#pragma unroll
+      for (int u = 0; u < OZ_U; ++u) {
+        const int x = __reduce_max_sync(0xffffffffu, e[u]);
+        if ((threadIdx.x & 31) == 0 && r + 8 * u < o.V && x > 0) atomicMax(o.e + r + 8 * u, x);
+      }
+    } else {
+      part[threadIdx.x >> 5][threadIdx.x & 31] = m;
+      __syncthreads();
+      if (threadIdx.x < 32) {
+#pragma unroll
+        for (int w = 1; w < OZ_PREP / 32; ++w) m = max(m, part[w][threadIdx.x]);
+        if (c < o.V && m > 0) atomicMax(o.e + c, m);
+      }
+      __syncthreads();
+    }
+  }
+}
+
+// the 56-bit fixed-point magnitude of x against the exponent field eb of its row /
+// column maximum: trunc(|x| 2^(56 - E)), E = eb - 1022
+__device__ __forceinline__ unsigned long long oz_fixed(double x, int eb) {
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
   const int ex = (int)((hi >> 20) & 0x7ffu);
-  unsigned long long m = ((unsigned long long)(hi & 0xfffffu) << 32) | lo;
-  unsigned long long F = 0;
-  if (ex > 0) {
-    m |= 1ull << 52;
-    const int sh = ex - eb + 3;   // <= 3 since ex <= eb
-    F = sh >= 0 ? (m << sh) : (sh > -64 ? (m >> -sh) : 0ull);
-  }
-  const bool neg = (hi >> 31) != 0;
+  if (ex == 0) return 0ull;
+  const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
+  const int sh = ex - eb + 3;   // <= 3 since ex <= eb
+  return sh >= 0 ? (m << sh) : (sh > -64 ? (m >> -sh) : 0ull);
+}
+// bits 7 (7 - s) .. + 6 of F as an fp32 integer (its low half is zero: a bf16 on top)
+__device__ __forceinline__ unsigned oz_digit(unsigned long long F, int s) {
+  const unsigned v = (unsigned)(F >> (OZ_BITS * (OZ_NS - 1 - s))) & 127u;
+  return __float_as_uint(__uint_as_float(0x4b000000u | v) - 8388608.0f);
+}
+
+// signed digits of both operands, as prep_a_kernel and prep_b_kernel lay their
+// slices out (rows of A: [Re | Im]; rows of B: [Re | -Im], then [Im | Re]). One
+// launch for both: most products here are small, and the operands' blocks fill
+// the GPU together. A value's digits are cut once, the real and imaginary one side
+// by side, and leave in eight bytes a lane. Four launches with two-byte stores
+// took 24 us of kernel time for a 69 x 69 product of 1024 rows, and an exact
+// iteration 24.4 ms at 1x2, D = 4, chi = 33 (22.2 now), 12.7 at 2x1, D = 3,
+// chi = 19 (11.9).
+template <typename T>
+__global__ void __launch_bounds__(OZ_PREP) oz_prep_kernel(OzOperand<T> a, OzOperand<T> b, int Kp) {
+  constexpr int PARTS = sizeof(T) / 8, LD = OZ_T + 1, W = 4, LPR = OZ_T / W;
+  using CellT = Cell<unsigned short, PARTS>;
+  __shared__ CellT tile[OZ_NS * OZ_T * LD];   // [digit][row][column]
+  for (int t = blockIdx.x; t < a.tiles + b.tiles; t += gridDim.x) {
+    const bool is_b = t >= a.tiles;
+    const OzOperand<T>& o = is_b ? b : a;
+    const int tt = is_b ? t - a.tiles : t;
+    T v[OZ_U];
+    int r, c;
+    oz_load(o, tt, r, c, v);
 #pragma unroll
-  for (int s = 0; s < OZ_NS; ++s) {
-    const int v = (int)((F >> (OZ_BITS * (OZ_NS - 1 - s))) & 127ull);
-    d[s] = __float2bfloat16_rn((float)(neg ? -v : v));
-  }
-}
-
-// exponent fields of the rows of op(A) (M x K): ea[m] = max over k; 32 x 32
-// tiles, one atomicMax per row and tile
-template <typename T>
-__global__ void oz_rowexp_kernel(const T* A, long lda, int op, int M, int K, int* ea) {
-  __shared__ int tile[32][33];
-  const int tiles_k = (K + 31) / 32, tiles_m = (M + 31) / 32;
-  const bool trans = (op == OP_T || op == OP_C);
-  for (int t = blockIdx.x; t < tiles_k * tiles_m; t += gridDim.x) {
-    const int k0 = (t % tiles_k) * 32, m0 = (t / tiles_k) * 32;
-    for (int yy = threadIdx.y; yy < 32; yy += 8) {
-      int e = 0;
-      if (!trans) {
-        const int m = m0 + yy, kk = k0 + threadIdx.x;
-        if (m < M && kk < K) {
-          const T v = A[(long)m * lda + kk];
-          if constexpr (sizeof(T) == 16) e = max(bexp(v.x), bexp(v.y));
-          else e = bexp(v);
-        }
-        tile[yy][threadIdx.x] = e;
+    for (int u = 0; u < OZ_U; ++u) {
+      const int vec = o.rows ? r + 8 * u : c;
+      const int eb = vec < o.V ? o.e[vec] : 0;
+      CellT* d = tile + (threadIdx.x / OZ_T + 8 * u) * LD + threadIdx.x % OZ_T;
+      if constexpr (PARTS == 2) {
+        const unsigned long long fr = oz_fixed(v[u].x, eb), fi = oz_fixed(v[u].y, eb);
+        const unsigned sign = ((unsigned)__double2hiint(v[u].x) >> 31 << 15) |
+                              ((unsigned)__double2hiint(v[u].y) & 0x80000000u);
+#pragma unroll
+        for (int s = 0; s < OZ_NS; ++s)
+          *reinterpret_cast<unsigned*>(d + s * OZ_T * LD) =
+              __byte_perm(oz_digit(fr, s), oz_digit(fi, s), 0x7632) | sign;
       } else {
-        const int kk = k0 + yy, m = m0 + threadIdx.x;
-        if (m < M && kk < K) {
-          const T v = A[(long)kk * lda + m];
-          if constexpr (sizeof(T) == 16) e = max(bexp(v.x), bexp(v.y));
-          else e = bexp(v);
-        }
-        tile[threadIdx.x][yy] = e;
+        const unsigned long long f = oz_fixed(v[u], eb);
+        const unsigned sign = (unsigned)__double2hiint(v[u]) >> 31 << 15;
+#pragma unroll
+        for (int s = 0; s < OZ_NS; ++s)
+          d[s * OZ_T * LD].p[0] = (unsigned short)((oz_digit(f, s) >> 16) | sign);
       }
     }
     __syncthreads();
-    for (int yy = threadIdx.y; yy < 32; yy += 8) {
-      int e = tile[yy][threadIdx.x];
-      for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
-      if (threadIdx.x == 0 && m0 + yy < M && e > 0) atomicMax(ea + m0 + yy, e);
-    }
-    __syncthreads();
-  }
-}
-
-// A digits: out[s][m][kr] as prep_a_kernel (real embedding [Re | Im]), with
-// the fixed-point digits of each row against ea[m]
-template <typename T>
-__global__ void oz_prep_a_kernel(const T* A, long lda, int op, int M, int K, int Kp,
-                                 const int* ea, __nv_bfloat16* out) {
-  __shared__ T tile[32][33];
-  constexpr bool cx = sizeof(T) == 16;
-  const int Kr = cx ? 2 * K : K;
-  const long slice = (long)M * Kp;
-  const int tiles_k = (K + 31) / 32, tiles_m = (M + 31) / 32;
-  const bool trans = (op == OP_T || op == OP_C);
-  const bool cj = (op == OP_C || op == OP_R);
-  for (int t = blockIdx.x; t < tiles_k * tiles_m; t += gridDim.x) {
-    const int k0 = (t % tiles_k) * 32, m0 = (t / tiles_k) * 32;
-    for (int yy = threadIdx.y; yy < 32; yy += 8) {
-      if (!trans) {
-        const int m = m0 + yy, kk = k0 + threadIdx.x;
-        tile[yy][threadIdx.x] = (m < M && kk < K) ? A[(long)m * lda + kk] : zero_of(T());
+    const int tr0 = tt / o.tiles_c * OZ_T, tc0 = tt % o.tiles_c * OZ_T;
+    const int v0 = o.rows ? tr0 : tc0, k0 = o.rows ? tc0 : tr0;
+    const int k = threadIdx.x % LPR * W, kc = k0 + k;
+    const bool whole = kc + W <= o.K, even = o.K % W == 0;
+    const long slice = (long)o.Vp * Kp;
+    // four values of a part at kc of row m, the second half (h) at K + kc
+    auto put = [&](int s, int m, int h, const CellT (&e)[W], int part, bool neg) {
+      unsigned short* dst = reinterpret_cast<unsigned short*>(o.out) + s * slice + (long)m * Kp +
+                            (h ? o.K : 0) + kc;
+      const unsigned short x = neg ? 0x8000 : 0;
+      if (whole && (!h || even)) {
+        *reinterpret_cast<ushort4*>(dst) =
+            make_ushort4(e[0].p[part] ^ x, e[1].p[part] ^ x, e[2].p[part] ^ x, e[3].p[part] ^ x);
       } else {
-        const int kk = k0 + yy, m = m0 + threadIdx.x;
-        tile[threadIdx.x][yy] = (m < M && kk < K) ? A[(long)kk * lda + m] : zero_of(T());
+#pragma unroll
+        for (int y = 0; y < W; ++y)
+          if (kc + y < o.K) dst[y] = e[y].p[part] ^ x;
       }
-    }
-    __syncthreads();
-    for (int yy = threadIdx.y; yy < 32; yy += 8) {
-      const int m = m0 + yy, kk = k0 + threadIdx.x;
-      if (m < M && kk < K) {
-        const T v = tile[yy][threadIdx.x];
-        const int eb = ea[m];
-        __nv_bfloat16 d[OZ_NS];
-        if constexpr (cx) {
-          oz_digits(v.x, eb, d);
-          put_digits(out, slice, (long)m * Kp + kk, d, false);
-          oz_digits(v.y, eb, d);
-          put_digits(out, slice, (long)m * Kp + K + kk, d, cj);
-        } else {
-          oz_digits(v, eb, d);
-          put_digits(out, slice, (long)m * Kp + kk, d, false);
+    };
+#pragma unroll 2
+    for (int i = threadIdx.x / LPR; i < OZ_NS * OZ_T; i += OZ_PREP / LPR) {
+      const int s = i / OZ_T, m = i % OZ_T;
+      CellT e[W];
+#pragma unroll
+      for (int y = 0; y < W; ++y)
+        e[y] = tile[s * OZ_T * LD + (o.rows ? m * LD + k + y : (k + y) * LD + m)];
+      if (v0 + m < o.V) {
+        put(s, v0 + m, 0, e, 0, false);
+        if constexpr (PARTS == 2) {
+          put(s, v0 + m, 1, e, 1, is_b ? !o.cj : o.cj != 0);
+          if (is_b) {
+            put(s, o.V + v0 + m, 0, e, 1, o.cj != 0);
+            put(s, o.V + v0 + m, 1, e, 0, false);
+          }
         }
       }
     }
     __syncthreads();
   }
-  const int pc = Kp - Kr;
-  const long tid = (long)blockIdx.x * blockDim.x * blockDim.y + threadIdx.y * blockDim.x + threadIdx.x;
-  const long nth = (long)gridDim.x * blockDim.x * blockDim.y;
+  // padding: the columns from PARTS K to Kp of the rows in use, then B's rows beyond them
+  const int tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
+  const int Kr = PARTS * a.K, pc = Kp - Kr, Nr = PARTS * b.V, pr = b.Vp - Nr;
   const __nv_bfloat16 z = __float2bfloat16(0.0f);
-  for (long idx = tid; idx < (long)M * pc; idx += nth)
-    for (int s = 0; s < OZ_NS; ++s) out[s * slice + (idx / pc) * Kp + Kr + idx % pc] = z;
-}
-
-// exponent fields of the columns of op(B) (K x N): eb[n] = max over k
-template <typename T>
-__global__ void oz_colexp_kernel(const T* B, long ldb, int op, int K, int N, int* eb) {
-  __shared__ int tile[32][33];
-  const int tk = (K + 31) / 32, tn = (N + 31) / 32;
-  const bool trans = (op == OP_T || op == OP_C);
-  for (int t = blockIdx.x; t < tk * tn; t += gridDim.x) {
-    const int k0 = (t % tk) * 32, n0 = (t / tk) * 32;
-    // tile[jj - n0][kk - k0]
-    for (int yy = threadIdx.y; yy < 32; yy += 8) {
-      int e = 0;
-      if (!trans) {
-        const int kk = k0 + yy, jj = n0 + threadIdx.x;
-        if (kk < K && jj < N) {
-          const T v = B[(long)kk * ldb + jj];
-          if constexpr (sizeof(T) == 16) e = max(bexp(v.x), bexp(v.y));
-          else e = bexp(v);
-        }
-        tile[threadIdx.x][yy] = e;
-      } else {
-        const int jj = n0 + yy, kk = k0 + threadIdx.x;
-        if (kk < K && jj < N) {
-          const T v = B[(long)jj * ldb + kk];
-          if constexpr (sizeof(T) == 16) e = max(bexp(v.x), bexp(v.y));
-          else e = bexp(v);
-        }
-        tile[yy][threadIdx.x] = e;
-      }
-    }
-    __syncthreads();
-    for (int yy = threadIdx.y; yy < 32; yy += 8) {
-      int e = tile[yy][threadIdx.x];
-      for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
-      if (threadIdx.x == 0 && n0 + yy < N && e > 0) atomicMax(eb + n0 + yy, e);
-    }
-    __syncthreads();
+  for (long i = tid; i < (long)OZ_NS * a.V * pc; i += nth)
+    a.out[i / pc * Kp + Kr + i % pc] = z;
+  for (long i = tid; i < (long)OZ_NS * Nr * pc; i += nth) {
+    const long row = i / pc;
+    b.out[(row / Nr * b.Vp + row % Nr) * Kp + Kr + i % pc] = z;
   }
-}
-
-// B digits: out[s][j][kr] as prep_b_kernel (B_emb = [[B_r, B_i], [-B_i, B_r]])
-template <typename T>
-__global__ void oz_prep_b_kernel(const T* B, long ldb, int op, int K, int N, int Kp, int Np,
-                                 const int* ebx, __nv_bfloat16* out) {
-  __shared__ T tile[32][33];
-  constexpr bool cx = sizeof(T) == 16;
-  const int Kr = cx ? 2 * K : K;
-  const int Nr = cx ? 2 * N : N;
-  const long slice = (long)Np * Kp;
-  const int tk = (K + 31) / 32, tn = (N + 31) / 32;
-  const bool trans = (op == OP_T || op == OP_C);
-  const bool cj = (op == OP_C || op == OP_R);
-  for (int t = blockIdx.x; t < tk * tn; t += gridDim.x) {
-    const int k0 = (t % tk) * 32, n0 = (t / tk) * 32;
-    for (int yy = threadIdx.y; yy < 32; yy += 8) {
-      if (!trans) {
-        const int kk = k0 + yy, jj = n0 + threadIdx.x;
-        tile[yy][threadIdx.x] = (kk < K && jj < N) ? B[(long)kk * ldb + jj] : zero_of(T());
-      } else {
-        const int jj = n0 + yy, kk = k0 + threadIdx.x;
-        tile[threadIdx.x][yy] = (kk < K && jj < N) ? B[(long)jj * ldb + kk] : zero_of(T());
-      }
-    }
-    __syncthreads();
-    for (int yy = threadIdx.y; yy < 32; yy += 8) {
-      const int jj = n0 + yy, kk = k0 + threadIdx.x;
-      if (jj < N && kk < K) {
-        const T v = tile[threadIdx.x][yy];
-        const int e = ebx[jj];
-        __nv_bfloat16 re[OZ_NS], im[OZ_NS];
-        if constexpr (cx) {
-          oz_digits(v.x, e, re);
-          oz_digits(v.y, e, im);
-          put_digits(out, slice, (long)jj * Kp + kk, re, false);
-          put_digits(out, slice, (long)jj * Kp + K + kk, im, !cj);
-          put_digits(out, slice, (long)(N + jj) * Kp + kk, im, cj);
-          put_digits(out, slice, (long)(N + jj) * Kp + K + kk, re, false);
-        } else {
-          oz_digits(v, e, re);
-          put_digits(out, slice, (long)jj * Kp + kk, re, false);
-        }
-      }
-    }
-    __syncthreads();
+  const int q = Kp / 8;   // sixteen bytes
+  for (long i = tid; i < (long)OZ_NS * pr * q; i += nth) {
+    const long row = i / q;
+    reinterpret_cast<uint4*>(b.out + (row / pr * b.Vp + Nr + row % pr) * Kp)[i % q] =
+        make_uint4(0u, 0u, 0u, 0u);
   }
-  const __nv_bfloat16 z = __float2bfloat16(0.0f);
-  const long tid = (long)blockIdx.x * blockDim.x * blockDim.y + threadIdx.y * blockDim.x + threadIdx.x;
-  const long nth = (long)gridDim.x * blockDim.x * blockDim.y;
-  for (long idx = tid; idx < (long)(Np - Nr) * Kp; idx += nth)
-    for (int s = 0; s < OZ_NS; ++s) out[s * slice + (long)Nr * Kp + idx] = z;
-  const int pc = Kp - Kr;
-  for (long idx = tid; idx < (long)Nr * pc; idx += nth)
-    for (int s = 0; s < OZ_NS; ++s) out[s * slice + (idx / pc) * Kp + Kr + idx % pc] = z;
 }
 
 // C[m][j] = (sum over K splits of the pairs) 2^(E_m + E_j - 14), complex
@@ -1639,23 +1608,37 @@ ctm_status oz_gemm(SplitCtx* sc, int opA, const void* A, long lda, int opB, cons
   int* ebx = sc->oz_e + M;
   if (cudaMemsetAsync(sc->oz_e, 0, (size_t)(M + N) * sizeof(int), s) != cudaSuccess)
     return sfail(sc, CTM_ECUDA, "exponent reset failed");
-  const dim3 blk(32, 8);
-  const unsigned ga = (unsigned)std::max<long>(1, std::min<long>((long)((K + 31) / 32) * ((M + 31) / 32), 152L * 16));
-  const unsigned gb = (unsigned)std::max<long>(1, std::min<long>((long)((K + 31) / 32) * ((N + 31) / 32), 152L * 16));
-  __nv_bfloat16* da = static_cast<__nv_bfloat16*>(sc->oz_a);
-  __nv_bfloat16* db = static_cast<__nv_bfloat16*>(sc->oz_b);
-  if (cx) {
-    oz_rowexp_kernel<cplx><<<ga, blk, 0, s>>>((const cplx*)A, lda, opA, M, K, ea);
-    oz_colexp_kernel<cplx><<<gb, blk, 0, s>>>((const cplx*)B, ldb, opB, K, N, ebx);
-    oz_prep_a_kernel<cplx><<<ga, blk, 0, s>>>((const cplx*)A, lda, opA, M, K, Kp, ea, da);
-    oz_prep_b_kernel<cplx><<<gb, blk, 0, s>>>((const cplx*)B, ldb, opB, K, N, Kp, Np, ebx, db);
-  } else {
-    oz_rowexp_kernel<double><<<ga, blk, 0, s>>>((const double*)A, lda, opA, M, K, ea);
-    oz_colexp_kernel<double><<<gb, blk, 0, s>>>((const double*)B, ldb, opB, K, N, ebx);
-    oz_prep_a_kernel<double><<<ga, blk, 0, s>>>((const double*)A, lda, opA, M, K, Kp, ea, da);
-    oz_prep_b_kernel<double><<<gb, blk, 0, s>>>((const double*)B, ldb, opB, K, N, Kp, Np, ebx, db);
-  }
-  if (launches) *launches += 4;
+  auto prepare = [&](auto zero) {
+    using T = decltype(zero);
+    OzOperand<T> a, b;
+    a.p = static_cast<const T*>(A);
+    a.ld = lda;
+    a.V = M;
+    a.rows = opA == OP_N || opA == OP_R;
+    a.cj = opA == OP_C || opA == OP_R;
+    a.e = ea;
+    a.out = static_cast<__nv_bfloat16*>(sc->oz_a);
+    a.Vp = M;
+    b.p = static_cast<const T*>(B);
+    b.ld = ldb;
+    b.V = N;
+    b.rows = opB == OP_T || opB == OP_C;
+    b.cj = opB == OP_C || opB == OP_R;
+    b.e = ebx;
+    b.out = static_cast<__nv_bfloat16*>(sc->oz_b);
+    b.Vp = Np;
+    for (OzOperand<T>* o : {&a, &b}) {
+      o->K = K;
+      o->tiles_c = ((o->rows ? K : o->V) + OZ_T - 1) / OZ_T;
+      o->tiles = o->tiles_c * (((o->rows ? o->V : K) + OZ_T - 1) / OZ_T);
+    }
+    const unsigned g = (unsigned)std::min<long>((long)a.tiles + b.tiles, 152L * 16);
+    oz_exp_kernel<T><<<g, OZ_PREP, 0, s>>>(a, b);
+    oz_prep_kernel<T><<<g, OZ_PREP, 0, s>>>(a, b, Kp);
+  };
+  if (cx) prepare(cplx());
+  else prepare(0.0);
+  if (launches) *launches += 2;
   CUtensorMap ta, tb;
   if (!make_map(&ta, sc->oz_a, M, Kp, BM, false, OZ_NS) ||
       !make_map(&tb, sc->oz_b, Np, Kp, BNc, false, OZ_NS))
