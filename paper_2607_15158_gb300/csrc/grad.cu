@@ -311,6 +311,18 @@ struct Tape {
     adj[v] = a;
     return a;
   }
+  // where a contribution to the adjoint of v is written: the adjoint itself, not
+  // yet zeroed, for the first one (*first), a temporary to be added for a later one.
+  // Most values have one use, so most contributions need neither a memset nor an
+  // addition: 522 of the 2150 kernels of a gradient at D = 3, chi = 27 were such
+  // additions.
+  void* contribution(void* v, long n, bool* first) {
+    *first = adj.find(v) == adj.end();
+    if (!*first) return tmpbuf(n);
+    void* a = adjs.get((size_t)n * 8);
+    if (a) adj[v] = a;
+    return a;
+  }
   void* adj_if(void* v) const {
     auto it = adj.find(v);
     return it == adj.end() ? nullptr : it->second;
@@ -328,6 +340,11 @@ ctm_status axpy(Tape& T, long n, double a, const void* x, void* y) {
   ++T.c->launches;
   CTM_CUDA_OK(cudaGetLastError());
   return CTM_OK;
+}
+
+// a contribution written by Tape::contribution joins the adjoint of v
+ctm_status add_in(Tape& T, void* v, long n, const void* t, bool first) {
+  return first ? CTM_OK : axpy(T, n, 1.0, t, T.adj_if(v));
 }
 
 // ---------------------------------------------------------- forward ops
@@ -493,19 +510,19 @@ ctm_status backward(Tape& T) {
         g.p = go;
         if (!T.constant.count(nd.a.p)) {
           Tn t = nd.a;
-          t.p = T.tmpbuf(nd.a.size());
-          void* ga = T.adj_of(nd.a.p, nd.a.size());
-          if (!t.p || !ga) return nomem(c);
+          bool first;
+          t.p = T.contribution(nd.a.p, nd.a.size(), &first);
+          if (!t.p) return nomem(c);
           CK(ein(c, (lo + "," + lb + "->" + la).c_str(), g, false, nd.b, false, t));
-          CK(axpy(T, nd.a.size(), 1.0, t.p, ga));
+          CK(add_in(T, nd.a.p, nd.a.size(), t.p, first));
         }
         if (!T.constant.count(nd.b.p)) {
           Tn t = nd.b;
-          t.p = T.tmpbuf(nd.b.size());
-          void* gb = T.adj_of(nd.b.p, nd.b.size());
-          if (!t.p || !gb) return nomem(c);
+          bool first;
+          t.p = T.contribution(nd.b.p, nd.b.size(), &first);
+          if (!t.p) return nomem(c);
           CK(ein(c, (la + "," + lo + "->" + lb).c_str(), nd.a, false, g, false, t));
-          CK(axpy(T, nd.b.size(), 1.0, t.p, gb));
+          CK(add_in(T, nd.b.p, nd.b.size(), t.p, first));
         }
         break;
       }
@@ -514,11 +531,11 @@ ctm_status backward(Tape& T) {
         if (!go || T.constant.count(nd.a.p)) break;
         int inv[8];
         for (int j = 0; j < nd.a.r; ++j) inv[nd.perm[j]] = j;
-        void* t = T.tmpbuf(nd.a.size());
-        void* ga = T.adj_of(nd.a.p, nd.a.size());
-        if (!t || !ga) return nomem(c);
+        bool first;
+        void* t = T.contribution(nd.a.p, nd.a.size(), &first);
+        if (!t) return nomem(c);
         CTM_CUDA_OK(permute(go, t, nd.o.r, nd.o.d, inv, false, false, T.st(), &c->launches));
-        CK(axpy(T, nd.a.size(), 1.0, t, ga));
+        CK(add_in(T, nd.a.p, nd.a.size(), t, first));
         break;
       }
       case K_QR: {
@@ -531,9 +548,9 @@ ctm_status backward(Tape& T) {
         void* R = T.tmpbuf((long)k * k);
         void* Ri = T.tmpbuf((long)k * k);
         void* G = T.tmpbuf(nk);
-        void* t = T.tmpbuf(nk);
-        void* gz = T.adj_of(Z, nk);
-        if (!P || !S || !R || !Ri || !G || !t || !gz) return nomem(c);
+        bool first;
+        void* t = T.contribution(Z, nk, &first);
+        if (!P || !S || !R || !Ri || !G || !t) return nomem(c);
         // P = Q^T dQ, S = sym(triu P), G = dQ - Q S
         CK(mm_small(c, OP_T, OP_N, k, k, N, Q, k, gq, k, P, k));
         sym_upper_kernel<<<blocks_for((long)k * k), 256, 0, T.st()>>>(k, (const double*)P, (double*)S);
@@ -544,7 +561,7 @@ ctm_status backward(Tape& T) {
         inv_upper_kernel<<<(k + 127) / 128, 128, 0, T.st()>>>(k, (const double*)R, (double*)Ri);
         c->launches += 3;
         CK(mm_small(c, OP_N, OP_T, N, k, k, G, k, Ri, k, t, k));
-        CK(axpy(T, nk, 1.0, t, gz));
+        CK(add_in(T, Z, nk, t, first));
         break;
       }
       case K_SVD: {
@@ -558,9 +575,9 @@ ctm_status backward(Tape& T) {
         void* K = gv ? T.tmpbuf((long)k * k) : nullptr;
         void* inner = T.tmpbuf((long)k * k);
         void* t1 = T.tmpbuf((long)k * k);
-        void* t2 = T.tmpbuf((long)k * k);
-        void* grho = T.adj_of(nd.p[0], (long)k * k);
-        if (!inner || !t1 || !t2 || !grho || (gu && !J) || (gv && !K)) return nomem(c);
+        bool first;
+        void* t2 = T.contribution(nd.p[0], (long)k * k, &first);
+        if (!inner || !t1 || !t2 || (gu && !J) || (gv && !K)) return nomem(c);
         if (gu) CK(mm_small(c, OP_T, OP_N, k, k, k, U, k, gu, k, J, k));
         if (gv) CK(mm_small(c, OP_T, OP_N, k, k, k, V, k, gv, k, K, k));
         svd_inner_kernel<<<blocks_for((long)k * k), 256, 0, T.st()>>>(
@@ -569,7 +586,7 @@ ctm_status backward(Tape& T) {
         ++c->launches;
         CK(mm_small(c, OP_N, OP_N, k, k, k, U, k, inner, k, t1, k));
         CK(mm_small(c, OP_N, OP_T, k, k, k, t1, k, V, k, t2, k));
-        CK(axpy(T, (long)k * k, 1.0, t2, grho));
+        CK(add_in(T, nd.p[0], (long)k * k, t2, first));
         break;
       }
       case K_SCALE: {
