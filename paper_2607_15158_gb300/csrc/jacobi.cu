@@ -17,6 +17,8 @@
 // Result: A = U diag(s) V^H with s descending (ties keep the lower column
 // first); exactly-zero columns of U are completed to a unitary by
 // Gram-Schmidt against unit vectors.
+#include <cooperative_groups.h>
+
 #include <cfloat>
 
 #include "common.cuh"
@@ -25,6 +27,8 @@
 namespace ctm {
 
 namespace {
+
+namespace cg = cooperative_groups;
 
 constexpr int JT = 64;   // threads per block (two warps)
 
@@ -159,6 +163,78 @@ __device__ __forceinline__ cplx rot_hi(cplx x, cplx y, double s, cplx ce) {
                       fma(ce.x, y.y, fma(ce.y, y.x, s * x.y)));
 }
 
+// The rotation of a pair of columns with squared norms al, be and overlap ga, by the
+// whole warp: every fp64 instruction costs the SM's narrow fp64 pipe the same for
+// one lane as for 32 and the chain of square roots and divisions is what a round
+// waits for, so the independent ones (the three roots; zeta, 1 / |gamma| and the
+// ratio) are taken side by side in lanes 0, 1 and 2.
+template <typename T>
+struct Rotation {
+  double c, s, tt, gm, ratio;   // ratio (lane 2): |gamma| / sqrt(alpha beta), at most 1
+  T se, ce;
+  // whether the pair is rotated: |gamma| > tol sqrt(alpha beta)
+  __device__ __forceinline__ bool find(T ga, double al, double be, double tol, int lane) {
+    double v = lane == 0 ? absq(ga) : lane == 1 ? al : be;
+    v = sqrt(v);
+    gm = __shfl_sync(0xffffffffu, v, 0);
+    const double nrm = __shfl_sync(0xffffffffu, v, 1) * __shfl_sync(0xffffffffu, v, 2);
+    if (!(gm > tol * nrm && gm != 0.0)) return false;
+    v = (lane == 0 ? be - al : lane == 1 ? 1.0 : gm) /
+        (lane == 0 ? 2.0 * gm : lane == 1 ? gm : nrm);
+    ratio = nrm > 0.0 ? fmin(v, 1.0) : 1.0;
+    const double zeta = __shfl_sync(0xffffffffu, v, 0);
+    const double ig = __shfl_sync(0xffffffffu, v, 1);
+    tt = copysign(1.0, zeta) / (fabs(zeta) + hypot(1.0, zeta));
+    c = 1.0 / hypot(1.0, tt);
+    s = c * tt;
+    // conj(gamma) / |gamma|
+    T eph;
+    if constexpr (sizeof(T) == 8) eph = ga * ig;
+    else eph = make_double2(ga.x * ig, -ga.y * ig);
+    se = scalev(eph, s);
+    ce = scalev(eph, c);
+    return true;
+  }
+};
+
+// exactly-zero columns of U (the last nzero), completed to a unitary by
+// Gram-Schmidt against unit vectors; one warp, tmp: k elements
+template <typename T>
+__device__ void complete_columns(int k, int nzero, T* Ub, T* tmp, int lane) {
+  const T one = [] {
+    if constexpr (sizeof(T) == 8) return T(1.0);
+    else return make_double2(1.0, 0.0);
+  }();
+  int cand = 0;
+  for (int col = k - nzero; col < k; ++col) {
+    for (; cand < k; ++cand) {
+      for (int r = lane; r < k; r += 32) stcg(tmp + r, (r == cand) ? one : zero_of(T()));
+      __syncwarp();
+      for (int rep = 0; rep < 2; ++rep) {
+        for (int j = 0; j < col; ++j) {
+          T dd = zero_of(T());
+          for (int r = lane; r < k; r += 32) fmacv(dd, ldcg(Ub + (size_t)r * k + j), ldcg(tmp + r));
+          dd = warp_sum(dd);
+          __syncwarp();
+          for (int r = lane; r < k; r += 32)
+            stcg(tmp + r, subv(ldcg(tmp + r), mulv(ldcg(Ub + (size_t)r * k + j), dd)));
+          __syncwarp();
+        }
+      }
+      double nn = 0.0;
+      for (int r = lane; r < k; r += 32) nn += absq(ldcg(tmp + r));
+      nn = warp_sum(nn);
+      if (nn > 0.25) {
+        const double inv = 1.0 / sqrt(nn);
+        for (int r = lane; r < k; r += 32) stcg(Ub + (size_t)r * k + col, scalev(ldcg(tmp + r), inv));
+        __syncwarp();
+        ++cand;
+        break;
+      }
+    }
+  }
+}
+
 template <typename T, int R>
 __global__ void __launch_bounds__(JT) jacobi_coop(JacobiArgs a) {
   // R: elements of a column held per lane (k <= 32 R); the pair's columns
@@ -257,39 +333,12 @@ __global__ void __launch_bounds__(JT) jacobi_coop(JacobiArgs a) {
             if (lane + 32 * e < k) fmacv(ga, xr[e], yr[e]);
           ga = warp_sum(ga);
           const double al = __ldcg(nsq + p), be = __ldcg(nsq + q);
-          // the rotation's scalars: every fp64 instruction costs the SM's
-          // narrow fp64 pipe the same for one lane as for 32 and the chain of
-          // square roots and divisions is what a round waits for, so the
-          // independent ones (the three roots; zeta, 1 / |gamma| and the
-          // ratio) are taken side by side in lanes 0, 1 and 2
-          double v = lane == 0 ? absq(ga) : lane == 1 ? al : be;
-          v = sqrt(v);
-          const double gm = __shfl_sync(0xffffffffu, v, 0);
-          const double nrm = __shfl_sync(0xffffffffu, v, 1) * __shfl_sync(0xffffffffu, v, 2);
-          // rotate when |gamma| > tol sqrt(alpha beta)
-          if (gm > tol * nrm && gm != 0.0) {
-            v = (lane == 0 ? be - al : lane == 1 ? 1.0 : gm) /
-                (lane == 0 ? 2.0 * gm : lane == 1 ? gm : nrm);
+          Rotation<T> ro;
+          if (ro.find(ga, al, be, tol, lane)) {
             if (lane == 2)
-              atomicMax(offb, (unsigned long long)__double_as_longlong(
-                                  nrm > 0.0 ? fmin(v, 1.0) : 1.0));   // this sweep rotated
-            const double zeta = __shfl_sync(0xffffffffu, v, 0);
-            const double ig = __shfl_sync(0xffffffffu, v, 1);
-            const double tt = copysign(1.0, zeta) / (fabs(zeta) + hypot(1.0, zeta));
-            const double c = 1.0 / hypot(1.0, tt);
-            const double s = c * tt;
-            // conj(gamma) / |gamma|
-            double ex = 0.0, ey = 0.0;
-            if constexpr (sizeof(T) == 8) {
-              ex = ga * ig;
-            } else {
-              ex = ga.x * ig;
-              ey = -ga.y * ig;
-            }
-            T eph;
-            if constexpr (sizeof(T) == 8) eph = ex;
-            else eph = make_double2(ex, ey);
-            const T se = scalev(eph, s), ce = scalev(eph, c);
+              atomicMax(offb, (unsigned long long)__double_as_longlong(ro.ratio));   // this sweep rotated
+            const double c = ro.c, s = ro.s;
+            const T se = ro.se, ce = ro.ce;
 #pragma unroll
             for (int e = 0; e < R; ++e) {
               const int r = lane + 32 * e;
@@ -299,8 +348,8 @@ __global__ void __launch_bounds__(JT) jacobi_coop(JacobiArgs a) {
               }
             }
             if (lane == 0) {
-              __stcg(nsq + p, al - tt * gm);
-              __stcg(nsq + q, be + tt * gm);
+              __stcg(nsq + p, al - ro.tt * ro.gm);
+              __stcg(nsq + q, be + ro.tt * ro.gm);
             }
             if (a.want_uv) {
 #pragma unroll
@@ -437,38 +486,234 @@ __global__ void __launch_bounds__(JT) jacobi_coop(JacobiArgs a) {
   int nzero = 0;
   for (int c = 0; c < k; ++c) nzero += (__ldcg(nb + c) == 0.0);
   if (nzero == 0) return;
-  T* Ub = static_cast<T*>(a.U) + (size_t)b * k * k;
-  T* tmp = wa;
-  int cand = 0;
-  for (int col = k - nzero; col < k; ++col) {
-    for (; cand < k; ++cand) {
-      for (int r = lane; r < k; r += 32) stcg(tmp + r, (r == cand) ? one : zero_of(T()));
-      __syncwarp();
-      for (int rep = 0; rep < 2; ++rep) {
-        for (int j = 0; j < col; ++j) {
-          T dd = zero_of(T());
-          for (int r = lane; r < k; r += 32) fmacv(dd, ldcg(Ub + (size_t)r * k + j), ldcg(tmp + r));
-          dd = warp_sum(dd);
-          __syncwarp();
-          for (int r = lane; r < k; r += 32)
-            stcg(tmp + r, subv(ldcg(tmp + r), mulv(ldcg(Ub + (size_t)r * k + j), dd)));
-          __syncwarp();
+  complete_columns(k, nzero, static_cast<T*>(a.U) + (size_t)b * k * k, wa, lane);
+}
+
+// 1b. The same iteration for k <= 64 on one cluster per matrix: A's and V's columns
+// stay in shared memory (column c in block c % C), a pair's warp reads and writes
+// them there, over the cluster's network, and a cluster barrier ends a round. Four
+// pairs per block, one per sub-partition: a pair's scalar chain fills a
+// sub-partition's fp64 pipe by itself. In jacobi_coop a round passes its columns
+// and versions through L2 (a poll, a load, a fence and a store one after the
+// other, about 2900 clocks beside the 5000 of the arithmetic); here it is a remote
+// load and the barrier, 640. The rotations are the same ones in the same order, so
+// the results are the same bits. Real k = 32: 1.24 ms -> 1.08 an SVD (1x1, D = 3,
+// chi = 27, an iteration: 6.95 ms -> 6.33); above k = 64 a cluster of eight has two
+// pairs per sub-partition, whose scalars then wait for one another.
+constexpr int JC_T = 128, JC_MAX_C = 8;
+
+template <typename T, int R>
+__global__ void __launch_bounds__(JC_T) jacobi_cluster(JacobiArgs a) {
+  cg::cluster_group cl = cg::this_cluster();
+  const int k = a.k, C = (int)cl.num_blocks(), me = (int)cl.block_rank();
+  const int b = blockIdx.x / C, nc = (k + C - 1) / C;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* wa = reinterpret_cast<T*>(smem_raw);          // [nc][k]
+  T* wv = wa + (size_t)nc * k;
+  double* nsq = reinterpret_cast<double*>(wv + (a.want_uv ? (size_t)nc * k : 0));   // [nc]
+  double* off = nsq + nc;                          // block 0: a slot per warp
+  auto colA = [&](int c) { return cl.map_shared_rank(wa, c % C) + (size_t)(c / C) * k; };
+  auto colV = [&](int c) { return cl.map_shared_rank(wv, c % C) + (size_t)(c / C) * k; };
+  auto norm = [&](int c) { return cl.map_shared_rank(nsq, c % C) + c / C; };
+  auto barrier = [&] {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::
+                     : "memory");
+  };
+  const T* Ab = static_cast<const T*>(a.A) + (size_t)b * a.strideA;
+  const T* Vi = a.Vinit ? static_cast<const T*>(a.Vinit) + (size_t)b * k * k : nullptr;
+  const T one = [] {
+    if constexpr (sizeof(T) == 8) return T(1.0);
+    else return make_double2(1.0, 0.0);
+  }();
+  const int mine = me < k ? (k - me + C - 1) / C : 0;   // columns of this block
+  for (int i = threadIdx.x; i < mine * k; i += JC_T) {
+    const int j = i % mine, r = i / mine, c = me + C * j;
+    wa[j * k + r] = Ab[(size_t)r * k + c];
+    if (a.want_uv) wv[j * k + r] = Vi ? Vi[(size_t)r * k + c] : (r == c ? one : zero_of(T()));
+  }
+  __syncthreads();
+  const double tol = fmax(1.0, (double)k) * DBL_EPSILON;
+  const int kk = k + (k & 1), m = kk - 1, npairs = kk / 2;
+  const int gw = me * (JC_T / 32) + warp, nw = C * (JC_T / 32);
+  auto norms = [&] {
+    for (int j = warp; j < mine; j += JC_T / 32) {
+      double acc = 0.0;
+      for (int r = lane; r < k; r += 32) acc += absq(wa[j * k + r]);
+      acc = warp_sum(acc);
+      if (lane == 0) nsq[j] = acc;
+    }
+  };
+  // the largest of the warps' values, to all threads
+  auto cluster_max = [&](double v) {
+    if (lane == 0) cl.map_shared_rank(off, 0)[gw] = v;
+    barrier();
+    const double* o = cl.map_shared_rank(off, 0);
+    double x = lane < nw ? o[lane] : 0.0;
+    for (int sft = 16; sft > 0; sft >>= 1) x = fmax(x, __shfl_xor_sync(0xffffffffu, x, sft));
+    return x;
+  };
+  bool converged = false;
+  for (int sweep = 0; sweep < a.max_sweeps && !converged; ++sweep) {
+    norms();   // exact squared norms at the start of the sweep
+    barrier();
+    double mx = 0.0;   // lane 2: the largest ratio rotated
+    for (int t = 0; t < m; ++t) {
+      for (int pr = gw; pr < npairs; pr += nw) {
+        int p = player(pr, t, m), q = player(kk - 1 - pr, t, m);
+        if (p > q) { const int tmp = p; p = q; q = tmp; }
+        if (q >= k) continue;
+        T *ap = colA(p), *aq = colA(q), *vp = nullptr, *vq = nullptr;
+        T xr[R], yr[R], vxr[R], vyr[R];
+        if (a.want_uv) {
+          vp = colV(p);
+          vq = colV(q);
+        }
+        double *np_ = norm(p), *nq_ = norm(q);
+        const double al = *np_, be = *nq_;
+        T ga = zero_of(T());
+#pragma unroll
+        for (int e = 0; e < R; ++e) {
+          const int r = lane + 32 * e;
+          if (r < k) {
+            xr[e] = ap[r];
+            yr[e] = aq[r];
+            if (a.want_uv) {
+              vxr[e] = vp[r];
+              vyr[e] = vq[r];
+            }
+          }
+        }
+#pragma unroll
+        for (int e = 0; e < R; ++e)
+          if (lane + 32 * e < k) fmacv(ga, xr[e], yr[e]);
+        ga = warp_sum(ga);
+        Rotation<T> ro;
+        if (ro.find(ga, al, be, tol, lane)) {
+          mx = fmax(mx, ro.ratio);
+#pragma unroll
+          for (int e = 0; e < R; ++e) {
+            const int r = lane + 32 * e;
+            if (r < k) {
+              ap[r] = rot_lo(xr[e], yr[e], ro.c, ro.se);
+              aq[r] = rot_hi(xr[e], yr[e], ro.s, ro.ce);
+              if (a.want_uv) {
+                vp[r] = rot_lo(vxr[e], vyr[e], ro.c, ro.se);
+                vq[r] = rot_hi(vxr[e], vyr[e], ro.s, ro.ce);
+              }
+            }
+          }
+          if (lane == 0) {
+            *np_ = al - ro.tt * ro.gm;
+            *nq_ = be + ro.tt * ro.gm;
+          }
         }
       }
-      double nn = 0.0;
-      for (int r = lane; r < k; r += 32) nn += absq(ldcg(tmp + r));
-      nn = warp_sum(nn);
-      if (nn > 0.25) {
-        const double inv = 1.0 / sqrt(nn);
-        for (int r = lane; r < k; r += 32) stcg(Ub + (size_t)r * k + col, scalev(ldcg(tmp + r), inv));
-        __syncwarp();
-        ++cand;
-        break;
+      barrier();
+    }
+    const double mxr = cluster_max(__shfl_sync(0xffffffffu, mx, 2));
+    converged = mxr <= tol;
+    if (!converged && mxr < 1e-6 && sweep + 1 < a.max_sweeps) {
+      // quadratic regime: whether another sweep would rotate anything, decided at
+      // once from every pair's exact ratio on the current columns
+      norms();
+      barrier();   // (and the slots have been read)
+      bool bad = false;
+      for (int f = gw; 2 * f <= k - 2 && !bad; f += nw) {
+        for (int side = 0; side < 2 && !bad; ++side) {
+          const int p = side == 0 ? f : k - 2 - f;
+          if (side == 1 && p == f) break;
+          T xr[R];
+          const T* ap = colA(p);
+#pragma unroll
+          for (int e = 0; e < R; ++e) {
+            const int r = lane + 32 * e;
+            xr[e] = r < k ? ap[r] : zero_of(T());
+          }
+          const double np_ = *norm(p);
+          for (int q = p + 1; q < k && !bad; ++q) {
+            const T* aq = colA(q);
+            T ga = zero_of(T());
+#pragma unroll
+            for (int e = 0; e < R; ++e) {
+              const int r = lane + 32 * e;
+              if (r < k) fmacv(ga, xr[e], aq[r]);
+            }
+            ga = warp_sum(ga);
+            bad = absq(ga) > tol * tol * np_ * *norm(q) && absq(ga) != 0.0;
+          }
+        }
+      }
+      converged = cluster_max(bad ? 1.0 : 0.0) == 0.0;
+    }
+    barrier();   // the slots have been read
+  }
+  if (!converged && me == 0 && threadIdx.x == 0) atomicOr(a.err, DEV_JACOBI_NOCONV);
+  // singular values: column norms
+  for (int j = warp; j < mine; j += JC_T / 32) {
+    double acc = 0.0;
+    for (int r = lane; r < k; r += 32) acc += absq(wa[j * k + r]);
+    acc = warp_sum(acc);
+    if (lane == 0) nsq[j] = sqrt(acc);
+  }
+  barrier();
+  // descending order, ties to the lower index; s, U, V, a column per warp
+  T* Ub = static_cast<T*>(a.U) + (size_t)b * k * k;
+  T* Vb = static_cast<T*>(a.V) + (size_t)b * k * k;
+  int nzero = 0;
+  for (int j = warp; j < mine; j += JC_T / 32) {
+    const int c = me + C * j;
+    const double x = nsq[j];
+    int rk = 0;
+    for (int i = lane; i < k; i += 32) {
+      const double y = *norm(i);
+      rk += (y > x) || (y == x && i < c);
+    }
+    rk = __reduce_add_sync(0xffffffffu, rk);
+    if (lane == 0) {
+      a.s_out[(size_t)b * k + rk] = x;
+      if (!isfinite(x)) atomicOr(a.err, DEV_NONFINITE);
+    }
+    if (a.want_uv) {
+      const double inv = x > 0.0 ? 1.0 / x : 0.0;
+      for (int r = lane; r < k; r += 32) {
+        stcg(Ub + (size_t)r * k + rk, x > 0.0 ? scalev(wa[j * k + r], inv) : zero_of(T()));
+        stcg(Vb + (size_t)r * k + rk, wv[j * k + r]);
       }
     }
   }
+  if (a.want_uv && me == 0)
+    for (int i = 0; i < k; ++i) nzero += *norm(i) == 0.0;
+  __threadfence();
+  barrier();   // U is written; no block leaves while its columns are read
+  if (a.want_uv && me == 0 && warp == 0 && nzero > 0)
+    complete_columns(k, nzero, Ub, static_cast<T*>(a.work) + (size_t)b * 2 * k * k, lane);
 }
 
+template <typename T, int R>
+cudaError_t launch_jacobi_cluster(const JacobiArgs& a, cudaStream_t s) {
+  int C = 1;
+  while (C < JC_MAX_C && 4 * C < (a.k + 1) / 2) C *= 2;
+  const size_t nc = (a.k + C - 1) / C;
+  const size_t smem = nc * a.k * sizeof(T) * (a.want_uv ? 2 : 1) + (nc + 4 * JC_MAX_C) * sizeof(double);
+  static size_t configured = 0;
+  cudaError_t e = raise_smem((const void*)jacobi_cluster<T, R>, configured, smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(a.batch * C);
+  cfg.blockDim = dim3(JC_T);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = C;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, jacobi_cluster<T, R>, a);
+}
 // ------------------------------------------------------------------------
 // 2. Blocked right-looking Cholesky G = L L^H (optionally shifted, with the
 // dead-column detection of CholeskyQR) and the triangular inverse L^-1.
@@ -746,6 +991,14 @@ cudaError_t jacobi_svd_coop(bool cx, int k, const void* A, long strideA, double*
   w += (size_t)batch * k * sizeof(unsigned);
   a.bar = reinterpret_cast<unsigned*>((reinterpret_cast<uintptr_t>(w) + 15) & ~(uintptr_t)15);
   a.err = err;
+  if (k <= 64) {
+    if (cx)
+      e = k <= 32 ? launch_jacobi_cluster<cplx, 1>(a, s) : launch_jacobi_cluster<cplx, 2>(a, s);
+    else
+      e = k <= 32 ? launch_jacobi_cluster<double, 1>(a, s) : launch_jacobi_cluster<double, 2>(a, s);
+    if (launches) ++*launches;
+    return e;
+  }
   e = cudaMemsetAsync(a.bar, 0, 65 * sizeof(unsigned), s);
   if (e != cudaSuccess) return e;
   void* args[] = {&a};
