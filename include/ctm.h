@@ -458,9 +458,11 @@ void ctm_debug_fail_alloc(int after);
  * callers that cannot let a library allocate device memory (an application
  * that owns all device memory through its own allocator, or a loop in which a
  * cudaMalloc / cudaFree would stall on a device-wide synchronisation). It runs
- * the same one-sided Jacobi kernel as ctm_spectrum, but keeps all of its
- * scratch in one fixed array of 2 MiB + 8 KiB reserved in device memory for
- * every GPU that loads the library, for the life of the process.
+ * the same one-sided Jacobi kernels as ctm_spectrum: up to k = 128 (CTM_F64) or
+ * 96 (CTM_C128) one that works in shared memory, above one whose scratch, like
+ * the error word of both, lies in one fixed array of 2 MiB + 8 KiB reserved in
+ * device memory for every GPU that loads the library, for the life of the
+ * process.
  *
  *   A       device pointer, the matrix in column-major order, k*k elements of
  *           double (CTM_F64) or interleaved (re, im) double pairs (CTM_C128);

@@ -12,7 +12,8 @@
 // round that wrote its columns (per-column version counters, release /
 // acquire), and grid barriers separate the sweeps. Every wait is bounded
 // (2 s of %globaltimer); a timeout sets DEV_MBAR_TIMEOUT and a global abort
-// flag after which every block leaves.
+// flag after which every block leaves. For k <= 64 the same iteration runs on a
+// cluster per matrix (1b).
 //
 // Result: A = U diag(s) V^H with s descending (ties keep the lower column
 // first); exactly-zero columns of U are completed to a unitary by

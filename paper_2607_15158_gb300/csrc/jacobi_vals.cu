@@ -4,9 +4,9 @@
 //
 // What bounds it is the chain of a round of disjoint rotations: dot product,
 // warp reduction, rotation angle, rotation, hand-over of the columns. The
-// kernel that also returns vectors (jacobi.cu) keeps the columns in global
-// memory and takes the angle with fp64 roots, divisions and hypots, a chain
-// of about 8300 clocks a round. Here
+// kernels that also return vectors (jacobi.cu) take the angle with fp64 roots,
+// divisions and hypots, a chain of about 5000 clocks a round (8300 with the
+// columns passed through global memory, as above k = 64). Here
 //   * each matrix lives in the shared memory of a cluster of up to eight CTAs,
 //     two blocks of B columns in each. A CTA rotates every column of one
 //     block against every column of the other (B rounds of B pairs, one pair

@@ -4,10 +4,11 @@
 // application that owns all device memory through its own allocator and
 // forbids plug-ins from calling cudaMalloc, or a latency-sensitive loop in
 // which cudaMalloc / cudaFree would stall on an implicit device-wide
-// synchronisation. ctm_svdvals_noalloc serves them: it runs the same
-// cooperative one-sided Jacobi kernel as the rest of the library, but its
-// scratch (the kernel's work area, grid-barrier words and error word) lives
-// in the fixed array g_noalloc_scratch below, reserved once in device memory
+// synchronisation. ctm_svdvals_noalloc serves them: it runs the same one-sided
+// Jacobi kernels as ctm_spectrum (in shared memory up to k = 128 real or 96
+// complex, on a cooperative grid above), but the scratch (the error word, and the
+// cooperative kernel's work area and grid-barrier words) lives in the fixed array
+// g_noalloc_scratch below, reserved once in device memory
 // for every GPU that loads the library and kept until the process exits.
 #include <cuda_runtime.h>
 
