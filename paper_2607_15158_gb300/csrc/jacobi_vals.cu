@@ -114,14 +114,19 @@ __global__ void __launch_bounds__(32 * VMAXW) jacobi_vals_kernel(ValsArgs a) {
   __shared__ int mxs[2][VMAXG];    // those of all CTAs
   __shared__ int exs[VMAXG];            // largest exponent field of every CTA's entries
   __shared__ int exm;
+  auto arrive = [&]() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); };
+  auto wait = [&]() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); };
   auto sync = [&]() {
     if (G > 1) {
-      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-      asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+      arrive();
+      wait();
     } else {
       __syncthreads();
     }
   };
+  // every CTA of the cluster must run before its shared memory is written: arrive
+  // here, wait before the first remote store, the loads in between
+  if (G > 1) arrive();
   auto remote = [&](auto* p, int cta) { return G > 1 ? cl.map_shared_rank(p, cta) : p; };
   // block position q of the round-robin table: CTA q's first block for q < G,
   // CTA 2 G - 1 - q's second block above
@@ -148,6 +153,7 @@ __global__ void __launch_bounds__(32 * VMAXW) jacobi_vals_kernel(ValsArgs a) {
   em = __reduce_max_sync(0xffffffffu, em);
   if (lane == 0) atomicMax(&exm, em);
   __syncthreads();
+  if (G > 1) wait();
   if (threadIdx.x < G) remote(&exs[rank], threadIdx.x)[0] = exm;
   sync();
   for (int g = 0; g < G; ++g) em = max(em, exs[g]);
