@@ -19,8 +19,16 @@
 //     root by Newton steps): the rotation is orthogonal to fp64 rounding, and
 //     an angle off by 1e-7 leaves 1e-7 of the overlap, which does not slow the
 //     quadratic convergence;
-//   * a sweep whose largest rotated overlap is below 1e-9 of the norms is the
-//     last: the next would meet overlaps of its square.
+//   * the sweep is the last that either rotates nothing, or whose rotated overlaps
+//     are below 7e-10 of the norms and so small beside its angles that (largest
+//     overlap) x (largest tangent) is below eps. A rotation returns to a pair that
+//     was already orthogonal its tangent times another overlap, at most 2 (k - 1)
+//     such terms a sweep, so what is left is of the order of the threshold k eps.
+//     The overlaps alone do not decide that: columns of nearly equal norm turn by up
+//     to 45 degrees however small their overlap, and their cluster converges only as
+//     a matrix of its own would (a spectrum within 1e-9 of one value takes seven
+//     sweeps at k = 64; one leaves errors of 1e-10). On random and on graded
+//     spectra the rule costs no sweep (k = 8 to 128), one without rotations one.
 // The matrix is scaled by a power of two so that its largest entry is about
 // 1; overlaps below 1e-140 then are left alone (their squares leave the fp64
 // range). The squared norms are exact at the start of each sweep and updated
@@ -110,8 +118,9 @@ __global__ void __launch_bounds__(32 * VMAXW) jacobi_vals_kernel(ValsArgs a) {
   T* cols = reinterpret_cast<T*>(smem);                               // [2 buffers][2 blocks][B][k]
   double* nsq = reinterpret_cast<double*>(cols + (size_t)4 * B * k);  // [2][2][B]
   double* vals = nsq + 4 * B;                                         // [2 G B]
-  __shared__ int mx[2];            // largest exponent of the sweep's rotated |gamma|^2 / (alpha beta)
-  __shared__ int mxs[2][VMAXG];    // those of all CTAs
+  // largest exponent of the sweep's rotated |gamma|^2 / (alpha beta) and of its tangents
+  __shared__ int mx[2][2];
+  __shared__ int mxs[2][2][VMAXG];   // those of all CTAs
   __shared__ int exs[VMAXG];            // largest exponent field of every CTA's entries
   __shared__ int exm;
   auto arrive = [&]() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); };
@@ -136,7 +145,7 @@ __global__ void __launch_bounds__(32 * VMAXW) jacobi_vals_kernel(ValsArgs a) {
   // position 1 to the end
   const int d0 = q0 == 0 ? 0 : q0 == 1 ? 2 * G - 1 : q0 - 1;
   const int d1 = G == 1 ? 1 : q1 - 1;
-  if (threadIdx.x < 2) mx[threadIdx.x] = NONE;
+  if (threadIdx.x < 4) mx[threadIdx.x / 2][threadIdx.x % 2] = NONE;
   if (threadIdx.x == 0) exm = 0;
   __syncthreads();
   const T* A = static_cast<const T*>(a.A) + (size_t)b * a.strideA;
@@ -194,7 +203,6 @@ __global__ void __launch_bounds__(32 * VMAXW) jacobi_vals_kernel(ValsArgs a) {
     const double g2 = absq(ga);
     const bool rot = g2 > thr && exf(g2) > 1023 - 930;   // above 1e-280
     if (rot) {
-      if (lane == 0) atomicMax(&mx[par], exf(g2) + 1023 - exf(al) - exf(be));
       double g;
       if constexpr (sizeof(T) == 8) {
         g = ga;
@@ -208,6 +216,10 @@ __global__ void __launch_bounds__(32 * VMAXW) jacobi_vals_kernel(ValsArgs a) {
       }
       double c;
       const double tt = tangent(d, g, c);
+      if (lane == 0) {
+        atomicMax(&mx[par][0], exf(g2) + 1023 - exf(al) - exf(be));
+        atomicMax(&mx[par][1], exf(tt) - 1023);
+      }
       c = rsqrt_from(fma(tt, tt, 1.0), c);
       const double s = c * tt;
 #pragma unroll
@@ -278,13 +290,21 @@ __global__ void __launch_bounds__(32 * VMAXW) jacobi_vals_kernel(ValsArgs a) {
       buf ^= 1;
       sync();
     }
-    // the largest ratio of the sweep over all CTAs
-    if (threadIdx.x < G) remote(&mxs[par][rank], threadIdx.x)[0] = mx[par];
-    if (threadIdx.x == 0) mx[par ^ 1] = NONE;
+    // the largest ratio and tangent of the sweep over all CTAs
+    if (threadIdx.x < 2 * G) {
+      const int g = threadIdx.x / 2, i = threadIdx.x % 2;
+      remote(&mxs[par][i][rank], g)[0] = mx[par][i];
+    }
+    if (threadIdx.x < 2) mx[par ^ 1][threadIdx.x] = NONE;
     sync();
-    int mm = NONE;
-    for (int g = 0; g < G; ++g) mm = max(mm, mxs[par][g]);
-    converged = mm < -61;   // below 2^-60 = 9e-19
+    int mm = NONE, mt = NONE;
+    for (int g = 0; g < G; ++g) {
+      mm = max(mm, mxs[par][0][g]);
+      mt = max(mt, mxs[par][1][g]);
+    }
+    // the overlap is below 2^((mm + 1) / 2), the tangent below 2^(mt + 1): the
+    // first below 2^-30, the product below 2^-52 (NONE: nothing was rotated)
+    converged = mm == NONE || (mm < -61 && mm + 2 * mt <= -107);
   }
   if (!converged && rank == 0 && threadIdx.x == 0) atomicOr(a.err, DEV_JACOBI_NOCONV);
   // norms of the columns to every CTA
