@@ -17,8 +17,13 @@
 //   * the tangent of the rotation is taken in fp32 and only the cosine that
 //     belongs to it in fp64 (from the hardware's approximate reciprocal square
 //     root by Newton steps): the rotation is orthogonal to fp64 rounding, and
-//     an angle off by 1e-7 leaves 1e-7 of the overlap, which does not slow the
-//     quadratic convergence;
+//     an angle off by 5e-7 leaves 5e-7 of the overlap. In the last sweep, whose
+//     overlaps are below 7e-10, that is less than the threshold k eps; in every other
+//     the next sweep meets it. Against an extended-precision Jacobi (k = 8 to 128,
+//     real and complex, singular values falling to e^-16) the errors are 5e-16 to
+//     4e-15 of the largest value; with a Newton step in fp64 on the tangent 3e-16 to
+//     5e-15 and a tenth more time; from the vector kernels, whose angles are fp64,
+//     1e-15 to 4e-14;
 //   * the sweep is the last that either rotates nothing, or whose rotated overlaps
 //     are below 7e-10 of the norms and so small beside its angles that (largest
 //     overlap) x (largest tangent) is below eps. A rotation returns to a pair that
