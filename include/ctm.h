@@ -452,6 +452,10 @@ const char* ctm_last_error(const ctm_ctx* ctx);
  * the hook then disarms itself. after < 0 disarms it. Process-wide. */
 void ctm_debug_fail_alloc(int after);
 
+/* For tests: the moves of this context that ran kernel by kernel, and those
+ * that were replayed from a CUDA graph (small cells past their warm-up). */
+ctm_status ctm_debug_moves(const ctm_ctx* ctx, long* direct, long* replayed);
+
 /* Singular values of one k x k matrix, with no device allocation.
  *
  * The paper has no counterpart to this call: it is a library service for

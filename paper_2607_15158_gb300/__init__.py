@@ -93,6 +93,7 @@ def load():
         "ctm_si_stats": (I, [ctx_p, P(C.c_long), P(C.c_long)]),
         "ctm_transfer_spectrum": (I, [ctx_p, I, I, I, P(D), P(D)]),
         "ctm_debug_fail_alloc": (None, [I]),
+        "ctm_debug_moves": (I, [ctx_p, P(C.c_long), P(C.c_long)]),
         "ctm_record": (I, [ctx_p, I]),
         "ctm_grad": (I, [ctx_p, VP, P(D), VP]),
         "ctm_grad_fixed_point": (I, [ctx_p, VP, D, I, P(D), VP, P(I), P(D)]),
@@ -316,6 +317,12 @@ class Context:
         u, sk = C.c_long(), C.c_long()
         _check(self.lib, self.ptr, self.lib.ctm_si_stats(self.ptr, C.byref(u), C.byref(sk)))
         return u.value, sk.value
+
+    def ctm_debug_moves(self):
+        """(moves run kernel by kernel, moves replayed from a graph)."""
+        d, r = C.c_long(), C.c_long()
+        _check(self.lib, self.ptr, self.lib.ctm_debug_moves(self.ptr, C.byref(d), C.byref(r)))
+        return d.value, r.value
 
     def ctm_profile_enable(self, on=True):
         _check(self.lib, self.ptr, self.lib.ctm_profile_enable(self.ptr, 1 if on else 0))

@@ -1152,12 +1152,16 @@ void drop_graph(ctm_ctx::MoveGraph& g) {
 // size), past its warm-up, and only where the host decides nothing from move
 // to move (no recycling policy, no recording for gradients, no profiling).
 constexpr int GRAPH_MAX_N = 2048;
+ctm_status run_direct(ctm_ctx* c, int r) {
+  ++c->n_direct;
+  return move_impl(c, r);
+}
 ctm_status run_move(ctm_ctx* c, int r) {
   bool ok = !c->graphs_off && c->opts.method == CTM_PROJ_SI && c->N <= GRAPH_MAX_N && !c->prof &&
             !grad_recording(c) && c->moves_done[r] >= c->opts.warmup_iters &&
             !(c->opts.recycle_sin2 > 0.0);
   for (int i = 0; ok && i < c->S; ++i) ok = c->rf_ready[r * c->S + i] != 0;
-  if (!ok) return move_impl(c, r);
+  if (!ok) return run_direct(c, r);
   auto key_now = [&]() {
     long k = 0;
     for (SplitCtx* sp : split_states(c)) k += split_generation(sp);
@@ -1166,7 +1170,7 @@ ctm_status run_move(ctm_ctx* c, int r) {
   ctm_ctx::MoveGraph& g = c->graphs[r][c->exact ? 1 : 0];
   if (g.exec && g.key != key_now()) drop_graph(g);
   if (!g.exec && g.ran != key_now()) {
-    const ctm_status st = move_impl(c, r);
+    const ctm_status st = run_direct(c, r);
     g.ran = key_now();
     return st;
   }
@@ -1215,7 +1219,7 @@ ctm_status run_move(ctm_ctx* c, int r) {
       c->n_updates = up0;
       c->n_skipped = sk0;
       c->si_updates = su0;
-      return move_impl(c, r);
+      return run_direct(c, r);
     }
     g.key = key_now();
     g.launches = c->launches - l0;
@@ -1223,6 +1227,7 @@ ctm_status run_move(ctm_ctx* c, int r) {
   }
   CTM_CUDA_OK(set_u64(c->qr_base, qr0, c->stream, &c->launches));
   CTM_CUDA_OK(cudaGraphLaunch(g.exec, c->stream));
+  ++c->n_replayed;
   return CTM_OK;
 }
 
@@ -2485,6 +2490,13 @@ ctm_status ctm_transfer_spectrum(ctm_ctx* c, int dir, int row, int nvals, double
   if (xi_out) *xi_out = ratio > 0.0 ? -(double)Lxf / std::log(ratio) : 0.0;
   c->scratch_off = mark;
   if (!conv) return fail(c, CTM_ENOCONV, "transfer-matrix eigenvalues did not converge");
+  return CTM_OK;
+}
+
+ctm_status ctm_debug_moves(const ctm_ctx* c, long* direct, long* replayed) {
+  if (!c) return CTM_EINVAL;
+  if (direct) *direct = c->n_direct;
+  if (replayed) *replayed = c->n_replayed;
   return CTM_OK;
 }
 

@@ -134,6 +134,7 @@ struct ctm_ctx {
   void* Xraw = nullptr;        // initial raw blocks (randomized-SVD warm-up)
   void* Wraw = nullptr;
   long n_updates = 0, n_skipped = 0;
+  long n_direct = 0, n_replayed = 0;   // moves run directly, replayed (run_move)
   int moves_done[4] = {0, 0, 0, 0};
   int num_sms = 1;
   bool spectra_init = false;
