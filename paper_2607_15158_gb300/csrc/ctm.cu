@@ -1150,7 +1150,9 @@ void drop_graph(ctm_ctx::MoveGraph& g) {
 // the line lies where nothing is left to gain. A direction is recorded after
 // it has run once directly with the same buffers (so that all have their
 // size), past its warm-up, and only where the host decides nothing from move
-// to move (no recycling policy, no recording for gradients, no profiling).
+// to move (no recycling policy, no recording for gradients, no profiling). It is
+// recorded on a stream of its own: c->stream may be the caller's (opts.stream),
+// and what others put on it in the meantime must run, not become part of the graph.
 constexpr int GRAPH_MAX_N = 2048;
 ctm_status run_direct(ctm_ctx* c, int r) {
   ++c->n_direct;
@@ -1195,12 +1197,17 @@ ctm_status run_move(ctm_ctx* c, int r) {
     const std::string msg0 = c->msg;
     cudaGraph_t graph = nullptr;
     ctm_status st = CTM_ECUDA;
-    if (cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+    const cudaStream_t s0 = c->stream;
+    if ((c->rec_stream ||
+         cudaStreamCreateWithFlags(&c->rec_stream, cudaStreamNonBlocking) == cudaSuccess) &&
+        cudaStreamBeginCapture(c->rec_stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+      c->stream = c->lanes[0].stream = c->rec_stream;
       c->recording_move = true;
       c->qr_start = qr0;
       st = move_impl(c, r);
       c->recording_move = false;
-      if (cudaStreamEndCapture(c->stream, &graph) != cudaSuccess) st = CTM_ECUDA;
+      c->stream = c->lanes[0].stream = s0;
+      if (cudaStreamEndCapture(c->rec_stream, &graph) != cudaSuccess) st = CTM_ECUDA;
     }
     if (st == CTM_OK && cudaGraphInstantiate(&g.exec, graph, 0) != cudaSuccess) {
       g.exec = nullptr;
@@ -2621,6 +2628,7 @@ void ctm_free(ctm_ctx* c) {
   if (c->stream) cudaStreamSynchronize(c->stream);
   for (auto& d : c->graphs)
     for (auto& g : d) drop_graph(g);
+  if (c->rec_stream) cudaStreamDestroy(c->rec_stream);
   destroy_helpers(c);
   for (auto& e : c->pev) cudaEventDestroy(e);
   if (c->stream) cudaStreamSynchronize(c->stream);

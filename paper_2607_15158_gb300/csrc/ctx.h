@@ -122,6 +122,7 @@ struct ctm_ctx {
   MoveGraph graphs[4][2];      // per direction; [1]: with exact-digit products
   bool graphs_off = false;     // recording failed once: every move runs directly
   bool recording_move = false;
+  cudaStream_t rec_stream = nullptr;   // lane 0's stream while a move is recorded
   uint64_t qr_start = 0;       // qr_calls at the start of the recorded move
   uint64_t* qr_base = nullptr; // device copy of qr_calls at the start of a replay
   // recycling policy (opts.recycle_sin2): per direction and cut, the number of
