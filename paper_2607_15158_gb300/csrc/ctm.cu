@@ -115,22 +115,39 @@ char* at(void* base, size_t elems, const ctm_ctx* c) {
 // remaining successful allocations before an injected failure (< 0: off)
 std::atomic<int> g_fail_alloc_after{-1};
 
+// device memory of the context: allocations may be refused by the fault hook, and
+// every change is counted (ctm_ctx::buffers)
+bool refused_by_hook() {
+  int left = g_fail_alloc_after.load();
+  while (left >= 0)
+    if (g_fail_alloc_after.compare_exchange_weak(left, left - 1)) return left == 0;
+  return false;
+}
+cudaError_t ctx_alloc(ctm_ctx* c, void** p, size_t bytes) {
+  *p = nullptr;
+  c->alloc_injected = refused_by_hook();
+  if (c->alloc_injected) return cudaErrorMemoryAllocation;
+  const cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaSuccess) ++c->buffers;
+  return e;
+}
+void ctx_release(ctm_ctx* c, void* p, size_t) {
+  ++c->buffers;
+  cudaFree(p);
+}
+SplitMemory split_memory(ctm_ctx* c) {
+  SplitMemory m;
+  m.owner = c;
+  m.alloc = [](void* o, void** p, size_t n) { return ctx_alloc(static_cast<ctm_ctx*>(o), p, n); };
+  m.release = [](void* o, void* p, size_t n) { ctx_release(static_cast<ctm_ctx*>(o), p, n); };
+  return m;
+}
+
 ctm_status dalloc(ctm_ctx* c, void** p, size_t bytes) {
   if (bytes == 0) bytes = 16;
-  {
-    int left = g_fail_alloc_after.load();
-    while (left >= 0) {
-      if (g_fail_alloc_after.compare_exchange_weak(left, left - 1)) {
-        if (left == 0) {
-          *p = nullptr;
-          c->alloc_injected = true;
-          return fail(c, CTM_ENOMEM, "device allocation failed (injected by ctm_debug_fail_alloc)");
-        }
-        break;
-      }
-    }
-  }
-  cudaError_t e = cudaMalloc(p, bytes);
+  cudaError_t e = ctx_alloc(c, p, bytes);
+  if (c->alloc_injected)
+    return fail(c, CTM_ENOMEM, "device allocation failed (injected by ctm_debug_fail_alloc)");
   if (e != cudaSuccess) {
     cudaGetLastError();
     char buf[256];
@@ -1164,16 +1181,11 @@ ctm_status run_move(ctm_ctx* c, int r) {
             !(c->opts.recycle_sin2 > 0.0);
   for (int i = 0; ok && i < c->S; ++i) ok = c->rf_ready[r * c->S + i] != 0;
   if (!ok) return run_direct(c, r);
-  auto key_now = [&]() {
-    long k = 0;
-    for (SplitCtx* sp : split_states(c)) k += split_generation(sp);
-    return k;
-  };
   ctm_ctx::MoveGraph& g = c->graphs[r][c->exact ? 1 : 0];
-  if (g.exec && g.key != key_now()) drop_graph(g);
-  if (!g.exec && g.ran != key_now()) {
+  if (g.exec && g.key != c->buffers) drop_graph(g);
+  if (!g.exec && g.ran != c->buffers) {
     const ctm_status st = run_direct(c, r);
-    g.ran = key_now();
+    g.ran = c->buffers;
     return st;
   }
   const uint64_t qr0 = c->qr_calls;
@@ -1228,7 +1240,7 @@ ctm_status run_move(ctm_ctx* c, int r) {
       c->si_updates = su0;
       return run_direct(c, r);
     }
-    g.key = key_now();
+    g.key = c->buffers;
     g.launches = c->launches - l0;
     g.qrs = c->qr_calls - qr0;
   }
@@ -1430,11 +1442,11 @@ ctm_status create_helpers(ctm_ctx* c) {
     al(H.Us, k * chi * es);
     if (st == CTM_OK && c->opts.prec != CTM_PREC_FP64 &&
         split_create(&H.split, c->cx, c->opts.prec == CTM_PREC_SPLIT_TF32, (int)N, (int)k, c->err,
-                     H.stream) != CTM_OK)
+                     H.stream, split_memory(c)) != CTM_OK)
       return fail(c, CTM_ECUDA, "split-precision setup failed");
   }
   if (st != CTM_ENOMEM || c->alloc_injected) return st;
-  for (size_t i = mark; i < c->allocs.size(); ++i) cudaFree(c->allocs[i]);
+  for (size_t i = mark; i < c->allocs.size(); ++i) ctx_release(c, c->allocs[i], 0);
   c->allocs.resize(mark);
   destroy_helpers(c);
   c->msg.clear();
@@ -1620,7 +1632,7 @@ ctm_status create(ctm_ctx** out, int Lx, int Ly, int d, int Dk, int Db, int chi,
     return bail(st);
   if (c->opts.prec != CTM_PREC_FP64) {
     st = split_create(&c->split, cx, c->opts.prec == CTM_PREC_SPLIT_TF32, (int)N, (int)k, c->err,
-                      c->stream);
+                      c->stream, split_memory(c));
     if (st != CTM_OK) {
       c->msg = "split-precision setup failed";
       return bail(st);
@@ -1688,7 +1700,7 @@ ctm_status create(ctm_ctx** out, int Lx, int Ly, int d, int Dk, int Db, int chi,
         return bail(st);
       if (c->opts.prec != CTM_PREC_FP64 &&
           (st = split_create(&M.split, cx, c->opts.prec == CTM_PREC_SPLIT_TF32, (int)N, (int)k,
-                             c->err, M.stream)) != CTM_OK) {
+                             c->err, M.stream, split_memory(c))) != CTM_OK) {
         c->msg = "split-precision setup failed";
         return bail(st);
       }

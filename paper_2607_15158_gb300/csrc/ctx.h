@@ -110,8 +110,9 @@ struct ctm_ctx {
   // Moves of small cells, whose kernels are as short as their launches, are
   // recorded as CUDA graphs once their direction is past its warm-up, and
   // replayed (run_move). A graph holds while the buffers that its kernels
-  // were given stay (key: the growth of the split buffers); the QR counter
-  // reaches its kernels through qr_base.
+  // were given stay (key: buffers, which counts every device buffer of the
+  // context allocated or freed, so that a freed one is never replayed into); the
+  // QR counter reaches its kernels through qr_base.
   struct MoveGraph {
     cudaGraphExec_t exec = nullptr;
     long key = -1;        // of the graph
@@ -119,6 +120,7 @@ struct ctm_ctx {
     long launches = 0;
     uint64_t qrs = 0;
   };
+  long buffers = 0;
   MoveGraph graphs[4][2];      // per direction; [1]: with exact-digit products
   bool graphs_off = false;     // recording failed once: every move runs directly
   bool recording_move = false;

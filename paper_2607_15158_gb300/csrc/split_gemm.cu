@@ -1207,6 +1207,7 @@ struct SplitCtx {
   bool tf32 = false;        // 3xTF32 slices instead of bf16 x3
   int N = 0, k = 0;
   std::string msg;
+  SplitMemory mem;
   // cached corner operands: [corner][op N / op H] slices, and their sources
   void* corner_src[4] = {nullptr};
   void* cslices[4][2] = {{nullptr}};
@@ -1229,7 +1230,6 @@ struct SplitCtx {
   void* oz_part = nullptr;
   size_t oz_part_bytes = 0;
   long oz_launches = 0;
-  long generation = 0;      // buffers allocated or replaced
   int* err = nullptr;       // device error flag of the owning context
   // per-launch CUDA events around the tensor-core kernel (profiling)
   bool prof = false;
@@ -1246,19 +1246,32 @@ ctm_status sfail(SplitCtx* sc, ctm_status st, const char* m) {
   return st;
 }
 
+bool mem_alloc(SplitCtx* sc, void** p, size_t bytes) {
+  const cudaError_t e =
+      sc->mem.alloc ? sc->mem.alloc(sc->mem.owner, p, bytes) : cudaMalloc(p, bytes);
+  if (e == cudaSuccess) return true;
+  cudaGetLastError();
+  *p = nullptr;
+  return false;
+}
+
+void mem_release(SplitCtx* sc, void** p, size_t bytes) {
+  if (!*p) return;
+  if (sc->mem.release) sc->mem.release(sc->mem.owner, *p, bytes);
+  else cudaFree(*p);
+  *p = nullptr;
+}
+
 ctm_status grow(SplitCtx* sc, void** p, size_t* have, size_t need) {
   if (*have >= need) return CTM_OK;
-  if (*p) cudaFree(*p);
-  *p = nullptr;
+  mem_release(sc, p, *have);
   *have = 0;
-  if (cudaMalloc(p, need) != cudaSuccess) {
-    cudaGetLastError();
+  if (!mem_alloc(sc, p, need))
     return sfail(sc, CTM_ENOMEM, "split-precision buffer allocation failed");
-  }
   *have = need;
-  ++sc->generation;
   return CTM_OK;
 }
+
 
 int pad_to(int x, int m) { return (x + m - 1) / m * m; }
 
@@ -1296,6 +1309,11 @@ inline double Kr_used(int Kp, const SplitCtx*) { return g_kr_real > 0 ? g_kr_rea
 inline int ns_of(const SplitCtx* sc) { return sc->tf32 ? 2 : 3; }
 inline int ke_of(const SplitCtx* sc) { return sc->tf32 ? 32 : 64; }
 inline int eb_of(const SplitCtx* sc) { return sc->tf32 ? 4 : 2; }
+
+// bytes of a corner's slices in one orientation
+size_t slice_bytes(const SplitCtx* sc, int N, int Kp) {
+  return (size_t)ns_of(sc) * N * Kp * eb_of(sc);
+}
 
 // run the tensor-core kernel on prepared slices: A [ns][M][Kp], B [ns][Np][Kp]
 ctm_status run_mma(SplitCtx* sc, const void* As, const void* Bs, int M, int Kp,
@@ -1443,7 +1461,7 @@ ctm_status prep_b(SplitCtx* sc, const void* B, long ldb, int op, int K, int N, i
 }  // namespace
 
 ctm_status split_create(SplitCtx** out, bool cx, bool tf32, int N, int k, int* err,
-                        cudaStream_t s) {
+                        cudaStream_t s, const SplitMemory& mem) {
   (void)s;
   *out = nullptr;
   if (!get_encoder()) return CTM_EUNSUPPORTED;
@@ -1453,6 +1471,7 @@ ctm_status split_create(SplitCtx** out, bool cx, bool tf32, int N, int k, int* e
   sc->N = N;
   sc->k = k;
   sc->err = err;
+  sc->mem = mem;
   *out = sc;
   return CTM_OK;
 }
@@ -1492,14 +1511,14 @@ void split_destroy(SplitCtx* sc) {
   for (auto& e : sc->ev) cudaEventDestroy(e);
   for (int i = 0; i < 4 && !sc->borrowed; ++i)
     for (int o = 0; o < 2; ++o)
-      if (sc->cslices[i][o]) cudaFree(sc->cslices[i][o]);
-  if (sc->abuf) cudaFree(sc->abuf);
-  if (sc->bbuf) cudaFree(sc->bbuf);
-  if (sc->part) cudaFree(sc->part);
-  if (sc->oz_a) cudaFree(sc->oz_a);
-  if (sc->oz_b) cudaFree(sc->oz_b);
-  if (sc->oz_e) cudaFree(sc->oz_e);
-  if (sc->oz_part) cudaFree(sc->oz_part);
+      mem_release(sc, &sc->cslices[i][o], slice_bytes(sc, sc->N, sc->corner_Kp));
+  mem_release(sc, &sc->abuf, sc->abuf_bytes);
+  mem_release(sc, &sc->bbuf, sc->bbuf_bytes);
+  mem_release(sc, (void**)&sc->part, sc->part_bytes);
+  mem_release(sc, &sc->oz_a, sc->oz_a_bytes);
+  mem_release(sc, &sc->oz_b, sc->oz_b_bytes);
+  mem_release(sc, (void**)&sc->oz_e, sc->oz_e_bytes);
+  mem_release(sc, &sc->oz_part, sc->oz_part_bytes);
   delete sc;
 }
 
@@ -1512,13 +1531,9 @@ ctm_status split_prepare_corners(SplitCtx* sc, void* const* Q, int N, unsigned m
     if (!(mask >> i & 1u)) continue;
     sc->corner_src[i] = Q[i];
     for (int o = 0; o < 2; ++o)
-      if ((ops >> o & 1u) && !sc->cslices[i][o]) {
-        if (cudaMalloc(&sc->cslices[i][o], (size_t)ns_of(sc) * N * Kp * eb_of(sc)) != cudaSuccess) {
-          cudaGetLastError();
-          return sfail(sc, CTM_ENOMEM, "corner slice allocation failed");
-        }
-        ++sc->generation;
-      }
+      if ((ops >> o & 1u) && !sc->cslices[i][o] &&
+          !mem_alloc(sc, &sc->cslices[i][o], slice_bytes(sc, N, Kp)))
+        return sfail(sc, CTM_ENOMEM, "corner slice allocation failed");
     // both orientations from one reading
     const PrepOut direct{ops & 1u ? sc->cslices[i][0] : nullptr, 0};
     const PrepOut trans{ops & 2u ? sc->cslices[i][1] : nullptr, sc->cx ? 1 : 0};
@@ -1676,8 +1691,6 @@ size_t split_partial_splits(size_t N, bool cx) {
   const size_t kb = ((cx ? 2 : 1) * N + BK - 1) / BK;
   return std::max<size_t>(32, (kb + KB_SPLIT_MAX - 1) / KB_SPLIT_MAX);
 }
-
-long split_generation(const SplitCtx* sc) { return sc->generation; }
 
 const char* split_last_error(const SplitCtx* sc) {
   return sc ? sc->msg.c_str() : "split precision not initialised";

@@ -10,13 +10,21 @@ namespace ctm {
 
 struct SplitCtx;
 
+// Where a state's device buffers come from: the owner's allocator (null: cudaMalloc
+// and cudaFree).
+struct SplitMemory {
+  void* owner = nullptr;
+  cudaError_t (*alloc)(void* owner, void** p, size_t bytes) = nullptr;
+  void (*release)(void* owner, void* p, size_t bytes) = nullptr;
+};
+
 // State for N x N corners and N x k blocks of real (cx = false) or complex
 // data; err is the owner's device error flag (bounded waits report there).
 // Buffers are allocated on first use.
 // tf32: 3xTF32 slices (two tf32 slices, three products, kind::tf32) instead
 // of bf16 x3 (three bf16 slices, six products, kind::f16).
 ctm_status split_create(SplitCtx** out, bool cx, bool tf32, int N, int k, int* err,
-                        cudaStream_t s);
+                        cudaStream_t s, const SplitMemory& mem = SplitMemory());
 void split_destroy(SplitCtx* sc);
 
 // Slice the fp64 corners Q[i] (N x N) whose bit i is set in mask into bf16
@@ -60,9 +68,6 @@ ctm_status split_profile(SplitCtx* sc, int on, double* ms, long* launches, doubl
 // Largest number of split-K partials a product with inner dimension N (2N
 // for complex) uses: each partial covers a bounded number of K blocks.
 size_t split_partial_splits(size_t N, bool cx);
-
-// Number of times a buffer of the state was allocated or replaced.
-long split_generation(const SplitCtx* sc);
 
 const char* split_last_error(const SplitCtx* sc);
 

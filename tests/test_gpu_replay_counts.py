@@ -59,3 +59,25 @@ def test_a_grown_buffer_is_followed_by_one_direct_move_per_direction():
         c.ctm_converge(0.0, 3)
     _same(a, b)
     assert a.ctm_debug_moves() == (12, 16)
+
+
+def test_no_replay_into_a_buffer_that_was_freed_and_could_not_be_replaced():
+    """An observable frees an operand buffer of the recorded moves to allocate a
+    larger one, and the allocation is refused: the observable fails, the next move
+    of each direction runs directly (and allocates again), and the environment goes
+    on as in a context that never asked for the observable."""
+    a, b = _pair(1, 1, 3, 32, True, **SPLIT)
+    for c in (a, b):
+        c.ctm_converge(0.0, 4)
+    assert a.ctm_debug_moves() == (8, 8)
+    pkg.ctm_debug_fail_alloc(0)
+    with pytest.raises(pkg.CTMError) as e:
+        a.ctm_rdm2(0, 0, 0)
+    assert e.value.status == pkg.CTM_ENOMEM
+    for c in (a, b):
+        c.ctm_converge(0.0, 2)
+        c.ctm_rdm2(0, 0, 0)
+        c.ctm_converge(0.0, 2)
+    _same(a, b)
+    direct, replayed = a.ctm_debug_moves()
+    assert direct == 16 and replayed == 16
