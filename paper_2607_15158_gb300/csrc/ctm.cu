@@ -248,10 +248,22 @@ struct Halves {
   }
 };
 
-// returns c to lane 0 when a move leaves early
+// Returns c to lane 0. When a move leaves early (done not set), the other lanes and the
+// helpers may still work on corners and blocks: what follows on lane 0 waits for them.
+// (The recording of a move that fails is thrown away, and nothing of it has run.)
 struct LaneReset {
   ctm_ctx* c;
-  ~LaneReset() { use_lane(c, 0); }
+  bool done = false;
+  ~LaneReset() {
+    use_lane(c, 0);
+    if (done || c->recording_move) return;
+    auto join = [&](const ctm_ctx::Lane& L) {
+      if (L.ev && cudaEventRecord(L.ev, L.stream) == cudaSuccess)
+        cudaStreamWaitEvent(c->lanes[0].stream, L.ev, 0);
+    };
+    for (size_t l = 1; l < c->lanes.size(); ++l) join(c->lanes[l]);
+    for (const auto& H : c->helpers) join(H);
+  }
 };
 
 void* scratch_alloc(ctm_ctx* c, size_t bytes) {
@@ -1136,6 +1148,7 @@ ctm_status move_impl(ctm_ctx* c, int r) {
       CTM_CUDA_OK(cudaMemcpyAsync(fC(c, r, 3, x + 1, y), at(c->stC4, y * elems_C(c), c),
                                   elems_C(c) * c->es, cudaMemcpyDeviceToDevice, c->stream));
     }
+    lane_reset.done = true;
   }
   c->moves_done[r] += 1;
   c->last_dir = r;
