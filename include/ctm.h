@@ -377,7 +377,8 @@ ctm_status ctm_profile_phases(ctm_ctx* ctx, double ms[CTM_NPHASES]);
 
 /* Device bytes a context of these dimensions and options allocates (an
  * upper estimate: the context's arrays, split-precision slice caches and
- * partial sums, dense-SVD buffers, plus 5 % and 64 MB). */
+ * partial sums, dense-SVD buffers, plus 5 % and 64 MB). Halves of cuts that run
+ * side by side take buffers of their own only as far as this leaves room. */
 ctm_status ctm_footprint(int Lx, int Ly, int d, int D, int chi, ctm_dtype dtype,
                          const ctm_opts* opts, size_t* bytes);
 
@@ -455,6 +456,10 @@ void ctm_debug_fail_alloc(int after);
 /* For tests: the moves of this context that ran kernel by kernel, and those
  * that were replayed from a CUDA graph (small cells past their warm-up). */
 ctm_status ctm_debug_moves(const ctm_ctx* ctx, long* direct, long* replayed);
+
+/* For tests: the device memory that the context holds, and the helpers on which
+ * it runs halves of cuts side by side (0: it runs them one after the other). */
+ctm_status ctm_debug_memory(const ctm_ctx* ctx, size_t* used, int* helpers);
 
 /* Singular values of one k x k matrix, with no device allocation.
  *

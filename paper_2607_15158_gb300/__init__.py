@@ -93,6 +93,7 @@ def load():
         "ctm_si_stats": (I, [ctx_p, P(C.c_long), P(C.c_long)]),
         "ctm_transfer_spectrum": (I, [ctx_p, I, I, I, P(D), P(D)]),
         "ctm_debug_fail_alloc": (None, [I]),
+        "ctm_debug_memory": (I, [ctx_p, P(C.c_size_t), P(I)]),
         "ctm_debug_moves": (I, [ctx_p, P(C.c_long), P(C.c_long)]),
         "ctm_record": (I, [ctx_p, I]),
         "ctm_grad": (I, [ctx_p, VP, P(D), VP]),
@@ -317,6 +318,12 @@ class Context:
         u, sk = C.c_long(), C.c_long()
         _check(self.lib, self.ptr, self.lib.ctm_si_stats(self.ptr, C.byref(u), C.byref(sk)))
         return u.value, sk.value
+
+    def ctm_debug_memory(self):
+        """(device bytes held, helpers)."""
+        n, h = C.c_size_t(), C.c_int()
+        _check(self.lib, self.ptr, self.lib.ctm_debug_memory(self.ptr, C.byref(n), C.byref(h)))
+        return n.value, h.value
 
     def ctm_debug_moves(self):
         """(moves run kernel by kernel, moves replayed from a graph)."""

@@ -123,16 +123,36 @@ bool refused_by_hook() {
     if (g_fail_alloc_after.compare_exchange_weak(left, left - 1)) return left == 0;
   return false;
 }
+void drop_helpers(ctm_ctx* c);
+bool helpers_idle(const ctm_ctx* c) {
+  return !c->helpers.empty() && !c->helpers_busy && !c->recording_move;
+}
+// cudaMalloc, once more without the helpers if there is no room beside them
+cudaError_t malloc_or_shed(ctm_ctx* c, void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e != cudaSuccess && helpers_idle(c)) {
+    cudaGetLastError();
+    drop_helpers(c);
+    e = cudaMalloc(p, bytes);
+  }
+  return e;
+}
 cudaError_t ctx_alloc(ctm_ctx* c, void** p, size_t bytes) {
   *p = nullptr;
   c->alloc_injected = refused_by_hook();
   if (c->alloc_injected) return cudaErrorMemoryAllocation;
-  const cudaError_t e = cudaMalloc(p, bytes);
-  if (e == cudaSuccess) ++c->buffers;
+  const size_t held = device_bytes(bytes);
+  if (c->mem_used + held > c->mem_cap && helpers_idle(c)) drop_helpers(c);
+  const cudaError_t e = malloc_or_shed(c, p, bytes);
+  if (e == cudaSuccess) {
+    ++c->buffers;
+    c->mem_used += held;
+  }
   return e;
 }
-void ctx_release(ctm_ctx* c, void* p, size_t) {
+void ctx_release(ctm_ctx* c, void* p, size_t bytes) {
   ++c->buffers;
+  c->mem_used -= device_bytes(bytes);
   cudaFree(p);
 }
 SplitMemory split_memory(ctm_ctx* c) {
@@ -218,14 +238,27 @@ void use_helper(ctm_ctx* c, int i) {
 
 // The W half of a cut beside its X half: from a fork on, w() points c at the
 // helper of the cut's lane and x() back at the lane; join() makes the lane wait
-// for the helper. Without a helper all of it runs on the lane.
+// for the helper. Without a helper all of it runs on the lane. In a split context it
+// also does until a section of the same plan (the kinds of its products) has run on
+// this lane alone: the helper's operand buffers get the sizes that it noted.
 struct Halves {
   ctm_ctx* c;
-  int lane;
-  bool on;
-  Halves(ctm_ctx* c_, bool want) : c(c_), lane(c_->cur_lane), on(want && !c_->helpers.empty()) {}
+  int lane, plan;
+  bool want, on;
+  Halves(ctm_ctx* c_, bool want_, int plan_)
+      : c(c_), lane(c_->cur_lane), plan(plan_), want(want_ && !c_->helpers_off),
+        on(want && !c_->helpers.empty() &&
+           (!c_->split || (c_->lanes[lane].matched >> plan & 1u))) {}
+  ~Halves() {
+    if (on) c->helpers_busy = false;
+    else if (want && c->lanes[lane].split) split_note(c->lanes[lane].split, false);
+  }
   ctm_status fork() {
-    if (!on) return CTM_OK;
+    if (!on) {
+      if (want && c->split) split_note(c->split, true);
+      return CTM_OK;
+    }
+    c->helpers_busy = true;
     const ctm_ctx::Lane &L = c->lanes[lane], &H = c->helpers[lane];
     if (H.split) split_borrow_corners(H.split, L.split);
     CTM_CUDA_OK(cudaEventRecord(L.ev, L.stream));
@@ -233,7 +266,10 @@ struct Halves {
     return CTM_OK;
   }
   ctm_status join() {
-    if (!on) return CTM_OK;
+    if (!on) {
+      if (want) c->lanes[lane].plans |= 1u << plan;
+      return CTM_OK;
+    }
     const ctm_ctx::Lane &L = c->lanes[lane], &H = c->helpers[lane];
     CTM_CUDA_OK(cudaEventRecord(H.ev, H.stream));
     CTM_CUDA_OK(cudaStreamWaitEvent(L.stream, H.ev, 0));
@@ -688,8 +724,13 @@ ctm_status si_rho(ctm_ctx* c, int r, int cut, int y) {
                                 cudaMemcpyDeviceToDevice, c->stream));
     ready = 0;
   }
+  const int rc = r * c->S + cut;
+  // recycling policy (paper step 4): a cut whose leading subspace stopped
+  // moving only recycles its bases, with no update round
+  const int rounds = warm ? c->opts.warmup_rounds
+                          : (c->si_skip[rc] ? 0 : c->opts.si_rounds);
   // the coupled update alternates between X and W: nothing runs side by side
-  Halves half(c, !c->opts.si_coupled);
+  Halves half(c, !c->opts.si_coupled, c->exact + 2 * warm + 4 * !ready + 8 * (rounds == 0));
   CK(half.fork());
   if (!ready) {
     CK(qr_inplace(c, X, Z[0], false));
@@ -698,11 +739,6 @@ ctm_status si_rho(ctm_ctx* c, int r, int cut, int y) {
     half.x();
     ready = 1;
   }
-  const int rc = r * c->S + cut;
-  // recycling policy (paper step 4): a cut whose leading subspace stopped
-  // moving only recycles its bases, with no update round
-  const int rounds = warm ? c->opts.warmup_rounds
-                          : (c->si_skip[rc] ? 0 : c->opts.si_rounds);
   c->si_rounds_used[rc] = rounds > 0;
   if (rounds > 0) {
     ++c->si_updates[rc];
@@ -863,7 +899,7 @@ ctm_status si_finish(ctm_ctx* c, int r, int cut, int y, void* Pl, void* PrH) {
     CTM_CUDA_OK(scale_columns_conj(c->cx, k, k, k, u, c->ph, c->stream, &c->launches));
     CTM_CUDA_OK(scale_columns_conj(c->cx, k, k, k, v, c->ph, c->stream, &c->launches));
   }
-  Halves half(c, true);
+  Halves half(c, !c->opts.si_coupled, 16 + c->exact);
   CK(half.fork());
   // recycled bases X v, W u (the next update re-orthonormalises them, so in
   // split contexts they run on the tensor cores) and the projectors
@@ -1184,9 +1220,11 @@ void drop_graph(ctm_ctx::MoveGraph& g) {
 // recorded on a stream of its own: c->stream may be the caller's (opts.stream),
 // and what others put on it in the meantime must run, not become part of the graph.
 constexpr int GRAPH_MAX_N = 2048;
+ctm_status ensure_helpers(ctm_ctx* c);
 ctm_status run_direct(ctm_ctx* c, int r) {
   ++c->n_direct;
-  return move_impl(c, r);
+  CK(move_impl(c, r));
+  return ensure_helpers(c);
 }
 ctm_status run_move(ctm_ctx* c, int r) {
   bool ok = !c->graphs_off && c->opts.method == CTM_PROJ_SI && c->N <= GRAPH_MAX_N && !c->prof &&
@@ -1415,6 +1453,73 @@ ctm_status update_recycling(ctm_ctx* c) {
   return CTM_OK;
 }
 
+// ------------------------------------------------------------ footprint
+// Device bytes a context of these dimensions allocates (the list of create(),
+// plus the split-precision slice caches and partial sums and the dense-SVD
+// buffers), rounded up by 5 % + 64 MB for allocator granularity. The helpers of a
+// context live within that rounding (ensure_helpers).
+size_t footprint_bytes(int Lx, int Ly, int d, int Dk, int Db, int chi, bool cx,
+                       const ctm_opts* o) {
+  const size_t S = (size_t)Lx * Ly, es = cx ? 16 : 8;
+  const size_t N = (size_t)chi * Dk * Db;
+  const size_t k = std::min<size_t>((size_t)chi + o->p, N);
+  const size_t NN = N * N, maxT = (size_t)d * d * NN + 64;
+  const size_t Lmax = std::max(Lx, Ly);
+  const size_t eC = (size_t)chi * chi, eT = eC * Dk * Db;
+  const size_t nk = (size_t)d * Dk * Dk * Dk * Dk, nb = (size_t)d * Db * Db * Db * Db;
+  size_t b = 0;
+  b += 4 * S * (nk + nb) * es;                     // kets, bras
+  b += 4 * S * (eC + eT) * es;                     // C, T
+  b += 2 * 4 * S * N * k * es;                     // X, W
+  b += 4 * NN * es + 2 * maxT * es;                // Q, pipes
+  b += 3 * maxT * es + ((size_t)64 << 20);         // scratch
+  b += 2 * Lmax * N * chi * es + 2 * S * N * chi * es;   // Pl, PrH, last*
+  b += 6 * N * k * es + 2 * k * k * es;            // Z, Xn, Wn, G, Linv
+  b += 2 * Lmax * N * k * es + 3 * Lmax * k * k * es;    // ZR, ZL, rho, u, v
+  b += 4 * std::max(Lmax * k * k, 4 * S * (size_t)chi * chi) * es;   // pre-solve
+  b += std::max(jacobi_coop_work_bytes(cx, (int)k, (int)Lmax),
+                jacobi_coop_work_bytes(cx, chi, 4 * (int)S));
+  b += (std::max(k, (size_t)chi) + 2 * k * chi) * es;
+  b += std::max(Lmax * k, 4 * S * (size_t)chi) * sizeof(double);
+  b += Lmax * (2 * eC + eT) * es + 8 * S * chi * sizeof(double);
+  b += 2 * (size_t)d * d * d * d * es + 2 * nk * es + ((size_t)1 << 20);
+  b += Lmax * k * k * es + 4 * S * sizeof(double);   // recycling policy
+  if (o->warmup_rsvd) b += 2 * 4 * S * N * k * es;    // raw blocks
+  if (o->prec != CTM_PREC_FP64) {
+    // slices: 3 bf16 (6 bytes) or 2 tf32 (8 bytes) per element
+    const size_t Kp = ((cx ? 2 : 1) * N + 63) / 64 * 64;
+    const size_t sb = o->prec == CTM_PREC_SPLIT_TF32 ? 8 : 6;
+    b += 8 * N * Kp * sb;                          // corner slices, both orientations
+    b += 2 * N * Kp * sb;                          // operand slices of general products
+    b += split_partial_splits(N, cx) * N * ((cx ? 2 : 1) * k + 160) * 4;   // split-K partials
+  }
+  // refinement: eight 2-byte digits per real component of the operands
+  // (complex B operands as 2 x 2 real blocks, K padded to at most twice) and
+  // fp32-pair partials, for operands of up to d N^2 elements on the lanes and
+  // d^2 N^2 for the two-site observables of lane 0
+  const bool refine = o->prec != CTM_PREC_FP64 && o->split_refine > 0.0;
+  const size_t oz_refine = refine ? 12 * (size_t)d * NN * es : 0;
+  b += (size_t)d * oz_refine;
+  if (o->method == CTM_PROJ_SVD) b += 3 * NN * es + 2 * N * chi * es + (size_t)64 * N * es;
+  if (o->method == CTM_PROJ_SI) {
+    // lanes 1 .. nl-1: corners, pipes, scratch, N x k blocks, QR work, split state
+    const bool fused =
+        !(o->split_refine > 0.0) && use_fused_absorb(cx, o->prec != CTM_PREC_FP64, *o, Dk, Db, d);
+    const size_t laneT = (size_t)(fused ? 1 : d) * NN + 64;
+    size_t lane = 4 * NN * es + 4 * laneT * es + ((size_t)64 << 20) + 4 * N * k * es +
+                  2 * k * k * es + 12 * k + chol_coop_work_bytes((int)k, 1) +
+                  (2 * N * k + 2 * k * chi + std::max(k, (size_t)chi)) * es;   // si_finish
+    if (o->prec != CTM_PREC_FP64) {
+      const size_t Kp = ((cx ? 2 : 1) * N + 63) / 64 * 64;
+      const size_t sb = o->prec == CTM_PREC_SPLIT_TF32 ? 8 : 6;
+      lane += 10 * N * Kp * sb + split_partial_splits(N, cx) * N * ((cx ? 2 : 1) * k + 160) * 4;
+    }
+    lane += oz_refine;
+    b += (size_t)(lanes_for(Lx, Ly) - 1) * lane;
+  }
+  return b + b / 20 + ((size_t)64 << 20);
+}
+
 void destroy_helpers(ctm_ctx* c) {
   for (auto& H : c->helpers) {
     if (H.split) split_destroy(H.split);
@@ -1422,47 +1527,85 @@ void destroy_helpers(ctm_ctx* c) {
     if (H.stream) cudaStreamDestroy(H.stream);
   }
   c->helpers.clear();
+  for (auto& a : c->helper_allocs) ctx_release(c, a.first, a.second);
+  c->helper_allocs.clear();
+}
+
+// give the helpers up for good (idle ones: nothing is enqueued between fork and join)
+void drop_helpers(ctm_ctx* c) {
+  cudaStreamSynchronize(c->lanes[0].stream);
+  for (auto& H : c->helpers)
+    if (H.stream) cudaStreamSynchronize(H.stream);
+  destroy_helpers(c);
+  for (auto& L : c->lanes) L.matched = 0;
+  c->helpers_off = true;
 }
 
 // scratch of a helper: the partial sums of a tall-skinny fp64 product
 size_t helper_scratch(size_t N) { return N >= 4096 ? (size_t)16 << 20 : (size_t)64 << 10; }
 
-// Helpers of the lanes that run cuts. A context runs without them, one half of
-// a cut after the other, when the device has no room for them.
-ctm_status create_helpers(ctm_ctx* c) {
-  const size_t N = c->N, k = c->k, chi = c->chi, es = c->es, mark = c->allocs.size();
-  const int nl = (int)c->lanes.size();
-  c->helpers.resize(nl);
-  ctm_status st = CTM_OK;
-  for (int l = nl > 1 ? 1 : 0; l < nl && st == CTM_OK; ++l) {
-    ctm_ctx::Lane& H = c->helpers[l];
-    for (int q = 0; q < 4; ++q) H.Q[q] = c->lanes[l].Q[q];
-    if (cudaStreamCreateWithFlags(&H.stream, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaEventCreateWithFlags(&H.ev, cudaEventDisableTiming) != cudaSuccess)
-      return fail(c, CTM_ECUDA, "helper stream creation failed");
-    H.scratch_bytes = helper_scratch(N);
-    auto al = [&](auto& p, size_t bytes) {
-      if (st == CTM_OK) st = dalloc(c, (void**)&p, bytes);
-    };
-    al(H.scratch, H.scratch_bytes);
-    for (int q = 0; q < 3; ++q) al(H.Z[q], N * k * es);
-    al(H.G, k * k * es);
-    al(H.Linv, k * k * es);
-    al(H.dsc, k * sizeof(double));
-    al(H.dead, k * sizeof(int));
-    al(H.chol_work, chol_coop_work_bytes((int)k, 1));
-    al(H.Wn, N * k * es);
-    al(H.Us, k * chi * es);
-    if (st == CTM_OK && c->opts.prec != CTM_PREC_FP64 &&
-        split_create(&H.split, c->cx, c->opts.prec == CTM_PREC_SPLIT_TF32, (int)N, (int)k, c->err,
-                     H.stream, split_memory(c)) != CTM_OK)
-      return fail(c, CTM_ECUDA, "split-precision setup failed");
+// Helpers of the lanes that run cuts, as far as they are wanted and there is room: a
+// context never holds more than its footprint, which does not count them
+// (HELPER_SLACK below it, for what is not tracked: graphs, events, driver pages). What
+// the helpers take is the part of the footprint that its rounding leaves, 5 % and 64
+// MB; where that does not do, where the device refuses, and as soon as the context
+// itself needs the room, it runs one half of a cut after the other.
+constexpr size_t HELPER_SLACK = (size_t)24 << 20;
+ctm_status ensure_helpers(ctm_ctx* c) {
+  if (c->helpers_off) return CTM_OK;
+  const size_t N = c->N, k = c->k, chi = c->chi, es = c->es;
+  const int nl = (int)c->lanes.size(), l0 = nl > 1 ? 1 : 0;
+  bool stale = c->helpers.empty() && !c->split;
+  for (int l = l0; l < nl; ++l) stale |= c->lanes[l].matched != c->lanes[l].plans;
+  if (!stale) return CTM_OK;
+  // the blocks of one helper, in bytes
+  const size_t sizes[] = {helper_scratch(N), N * k * es, N * k * es, N * k * es, k * k * es, k * k * es,
+                          k * sizeof(double), k * sizeof(int), chol_coop_work_bytes((int)k, 1),
+                          N * k * es, k * chi * es};
+  size_t need = 0;
+  for (int l = l0; l < nl; ++l) {
+    if (c->helpers.empty())
+      for (size_t b : sizes) need += device_bytes(std::max<size_t>(b, 16));
+    if (c->split)
+      need += split_reserve_bytes(c->helpers.empty() ? nullptr : c->helpers[l].split,
+                                  c->lanes[l].split);
   }
-  if (st != CTM_ENOMEM || c->alloc_injected) return st;
-  for (size_t i = mark; i < c->allocs.size(); ++i) ctx_release(c, c->allocs[i], 0);
-  c->allocs.resize(mark);
-  destroy_helpers(c);
-  c->msg.clear();
+  struct Busy {
+    ctm_ctx* c;
+    explicit Busy(ctm_ctx* cc) : c(cc) { c->helpers_busy = true; }
+    ~Busy() { c->helpers_busy = false; }
+  };
+  bool room = c->mem_used + need + HELPER_SLACK <= c->mem_cap;
+  {
+    Busy busy(c);
+    if (room && c->helpers.empty()) {
+      c->helpers.resize(nl);
+      for (int l = l0; l < nl && room; ++l) {
+        ctm_ctx::Lane& H = c->helpers[l];
+        for (int q = 0; q < 4; ++q) H.Q[q] = c->lanes[l].Q[q];
+        H.scratch_bytes = sizes[0];
+        void** const ptrs[] = {(void**)&H.scratch, &H.Z[0], &H.Z[1], &H.Z[2], &H.G, &H.Linv,
+                               (void**)&H.dsc, (void**)&H.dead, &H.chol_work, &H.Wn, &H.Us};
+        for (int i = 0; i < 11 && room; ++i) {
+          const size_t b = std::max<size_t>(sizes[i], 16);
+          room = ctx_alloc(c, ptrs[i], b) == cudaSuccess;
+          if (room) c->helper_allocs.push_back({*ptrs[i], b});
+        }
+        room = room && cudaStreamCreateWithFlags(&H.stream, cudaStreamNonBlocking) == cudaSuccess &&
+               cudaEventCreateWithFlags(&H.ev, cudaEventDisableTiming) == cudaSuccess &&
+               (!c->split || split_create(&H.split, c->cx, c->opts.prec == CTM_PREC_SPLIT_TF32, (int)N,
+                                          (int)k, c->err, H.stream, split_memory(c)) == CTM_OK);
+      }
+    }
+    for (int l = l0; l < nl && room && c->split; ++l) {
+      room = split_reserve(c->helpers[l].split, c->lanes[l].split) == CTM_OK;
+      if (room) c->lanes[l].matched = c->lanes[l].plans;
+    }
+  }
+  if (!room) {
+    cudaGetLastError();
+    drop_helpers(c);
+  }
   return CTM_OK;
 }
 
@@ -1529,6 +1672,7 @@ ctm_status create(ctm_ctx** out, int Lx, int Ly, int d, int Dk, int Db, int chi,
   const size_t S = c->S, N = c->N, k = c->k, es = c->es;
   const size_t nk = elems_ket(c), nb = elems_bra(c);
   const size_t NN = N * N;
+  c->mem_cap = footprint_bytes(Lx, Ly, d, Dk, Db, chi, cx, &c->opts);
   const size_t maxT = (size_t)d * d * NN + 64;
   c->pipe_elems = maxT;
   ctm_status st = CTM_OK;
@@ -1719,9 +1863,9 @@ ctm_status create(ctm_ctx** out, int Lx, int Ly, int d, int Dk, int Db, int chi,
       }
     }
   }
-  if (c->opts.method == CTM_PROJ_SI && !c->opts.si_coupled &&
-      (st = create_helpers(c)) != CTM_OK)
-    return bail(st);
+  // (a split context gets its helpers once a move has run: ensure_helpers)
+  c->helpers_off = c->opts.method != CTM_PROJ_SI || c->opts.si_coupled;
+  if (!c->split && (st = ensure_helpers(c)) != CTM_OK) return bail(st);
   if (c->opts.method == CTM_PROJ_SVD) {
     st = svd_create(&c->svd, cx, (int)N, chi);
     if (st != CTM_OK) {
@@ -1933,82 +2077,6 @@ ctm_status ctm_set_rangefinders(ctm_ctx* c, const void* X, const void* W) {
   std::fill(c->rf_ready.begin(), c->rf_ready.end(), 0);
   for (int r = 0; r < 4; ++r) c->moves_done[r] = 0;
   return reset_recycling(c);
-}
-
-// ------------------------------------------------------------ footprint
-// Device bytes a context of these dimensions allocates (the list of create(),
-// plus the split-precision slice caches and partial sums and the dense-SVD
-// buffers), rounded up by 5 % + 64 MB for allocator granularity.
-static size_t footprint_bytes(int Lx, int Ly, int d, int Dk, int Db, int chi, bool cx,
-                       const ctm_opts* o) {
-  const size_t S = (size_t)Lx * Ly, es = cx ? 16 : 8;
-  const size_t N = (size_t)chi * Dk * Db;
-  const size_t k = std::min<size_t>((size_t)chi + o->p, N);
-  const size_t NN = N * N, maxT = (size_t)d * d * NN + 64;
-  const size_t Lmax = std::max(Lx, Ly);
-  const size_t eC = (size_t)chi * chi, eT = eC * Dk * Db;
-  const size_t nk = (size_t)d * Dk * Dk * Dk * Dk, nb = (size_t)d * Db * Db * Db * Db;
-  size_t b = 0;
-  b += 4 * S * (nk + nb) * es;                     // kets, bras
-  b += 4 * S * (eC + eT) * es;                     // C, T
-  b += 2 * 4 * S * N * k * es;                     // X, W
-  b += 4 * NN * es + 2 * maxT * es;                // Q, pipes
-  b += 3 * maxT * es + ((size_t)64 << 20);         // scratch
-  b += 2 * Lmax * N * chi * es + 2 * S * N * chi * es;   // Pl, PrH, last*
-  b += 6 * N * k * es + 2 * k * k * es;            // Z, Xn, Wn, G, Linv
-  b += 2 * Lmax * N * k * es + 3 * Lmax * k * k * es;    // ZR, ZL, rho, u, v
-  b += 4 * std::max(Lmax * k * k, 4 * S * (size_t)chi * chi) * es;   // pre-solve
-  b += std::max(jacobi_coop_work_bytes(cx, (int)k, (int)Lmax),
-                jacobi_coop_work_bytes(cx, chi, 4 * (int)S));
-  b += (std::max(k, (size_t)chi) + 2 * k * chi) * es;
-  b += std::max(Lmax * k, 4 * S * (size_t)chi) * sizeof(double);
-  b += Lmax * (2 * eC + eT) * es + 8 * S * chi * sizeof(double);
-  b += 2 * (size_t)d * d * d * d * es + 2 * nk * es + ((size_t)1 << 20);
-  b += Lmax * k * k * es + 4 * S * sizeof(double);   // recycling policy
-  if (o->warmup_rsvd) b += 2 * 4 * S * N * k * es;    // raw blocks
-  if (o->prec != CTM_PREC_FP64) {
-    // slices: 3 bf16 (6 bytes) or 2 tf32 (8 bytes) per element
-    const size_t Kp = ((cx ? 2 : 1) * N + 63) / 64 * 64;
-    const size_t sb = o->prec == CTM_PREC_SPLIT_TF32 ? 8 : 6;
-    b += 8 * N * Kp * sb;                          // corner slices, both orientations
-    b += 2 * N * Kp * sb;                          // operand slices of general products
-    b += split_partial_splits(N, cx) * N * ((cx ? 2 : 1) * k + 160) * 4;   // split-K partials
-  }
-  // refinement: eight 2-byte digits per real component of the operands
-  // (complex B operands as 2 x 2 real blocks, K padded to at most twice) and
-  // fp32-pair partials, for operands of up to d N^2 elements on the lanes and
-  // d^2 N^2 for the two-site observables of lane 0
-  const bool refine = o->prec != CTM_PREC_FP64 && o->split_refine > 0.0;
-  const size_t oz_refine = refine ? 12 * (size_t)d * NN * es : 0;
-  b += (size_t)d * oz_refine;
-  if (o->method == CTM_PROJ_SVD) b += 3 * NN * es + 2 * N * chi * es + (size_t)64 * N * es;
-  if (o->method == CTM_PROJ_SI) {
-    // lanes 1 .. nl-1: corners, pipes, scratch, N x k blocks, QR work, split state
-    const bool fused =
-        !(o->split_refine > 0.0) && use_fused_absorb(cx, o->prec != CTM_PREC_FP64, *o, Dk, Db, d);
-    const size_t laneT = (size_t)(fused ? 1 : d) * NN + 64;
-    size_t lane = 4 * NN * es + 4 * laneT * es + ((size_t)64 << 20) + 4 * N * k * es +
-                  2 * k * k * es + 12 * k + chol_coop_work_bytes((int)k, 1) +
-                  (2 * N * k + 2 * k * chi + std::max(k, (size_t)chi)) * es;   // si_finish
-    if (o->prec != CTM_PREC_FP64) {
-      const size_t Kp = ((cx ? 2 : 1) * N + 63) / 64 * 64;
-      const size_t sb = o->prec == CTM_PREC_SPLIT_TF32 ? 8 : 6;
-      lane += 10 * N * Kp * sb + split_partial_splits(N, cx) * N * ((cx ? 2 : 1) * k + 160) * 4;
-    }
-    lane += oz_refine;
-    const int nl = lanes_for(Lx, Ly);
-    b += (size_t)(nl - 1) * lane;
-    if (!o->si_coupled) {
-      // helpers of the lanes that run cuts: blocks, QR work, split state
-      size_t help = helper_scratch(N) + 4 * N * k * es + 2 * k * k * es + k * chi * es + 12 * k +
-                    chol_coop_work_bytes((int)k, 1) + ((size_t)1 << 20);
-      if (o->prec != CTM_PREC_FP64)
-        help += split_partial_splits(N, cx) * N * ((cx ? 2 : 1) * k + 160) * 4 + 40 * N * k * es;
-      if (refine) help += 4 * NN * es;
-      b += (size_t)std::max(1, nl - 1) * help;
-    }
-  }
-  return b + b / 20 + ((size_t)64 << 20);
 }
 
 // ---------------------------------------------------- checkpoint / resume
@@ -2522,6 +2590,16 @@ ctm_status ctm_transfer_spectrum(ctm_ctx* c, int dir, int row, int nvals, double
   if (xi_out) *xi_out = ratio > 0.0 ? -(double)Lxf / std::log(ratio) : 0.0;
   c->scratch_off = mark;
   if (!conv) return fail(c, CTM_ENOCONV, "transfer-matrix eigenvalues did not converge");
+  return CTM_OK;
+}
+
+ctm_status ctm_debug_memory(const ctm_ctx* c, size_t* used, int* helpers) {
+  if (!c) return CTM_EINVAL;
+  if (used) *used = c->mem_used;
+  if (helpers) {
+    *helpers = 0;
+    for (const auto& H : c->helpers) *helpers += H.stream != nullptr;
+  }
   return CTM_OK;
 }
 

@@ -171,14 +171,23 @@ struct ctm_ctx {
     void* Vs = nullptr;
     void* Us = nullptr;
     void* ph = nullptr;
+    // sections of a cut that have run on this lane alone, one bit per plan (si_rho,
+    // si_finish), and those whose buffers its helper has too
+    unsigned plans = 0, matched = 0;
   };
   std::vector<Lane> lanes;   // lane 0 = the context's own buffers and stream
   int cur_lane = 0;          // -1 - i: the helper of lane i
   // helper of a lane that runs cuts: the W half of a cut's subspace iteration
   // and projector step (independent of the X half but for the corners) on its
   // own stream, with the lane's corners and its own blocks and QR work. Empty
-  // when the device had no room for them: then both halves run on the lane.
+  // when there is no room for them (see ensure_helpers): then both halves run on
+  // the lane.
   std::vector<Lane> helpers; // one per lane (those of lanes without cuts unused)
+  std::vector<std::pair<void*, size_t>> helper_allocs;
+  bool helpers_off = false;  // not wanted, or given up for good
+  bool helpers_busy = false; // being made, or in use between a fork and its join
+  size_t mem_used = 0;       // device memory held (device_bytes of every allocation)
+  size_t mem_cap = 0;        // that the context may hold (footprint)
   bool alloc_injected = false;   // the last allocation failure was injected
   // standard truncated-SVD projectors (CTM_PROJ_SVD)
   SvdCtx* svd = nullptr;
@@ -228,6 +237,7 @@ size_t elems_ket(const ctm_ctx* c);
 size_t elems_bra(const ctm_ctx* c);
 char* at(void* base, size_t elems, const ctm_ctx* c);
 ctm_status dalloc(ctm_ctx* c, void** p, size_t bytes);
+cudaError_t malloc_or_shed(ctm_ctx* c, void** p, size_t bytes);
 int frame_site(const ctm_ctx* c, int r, int x, int y);
 int frame_label(int r, int i);
 void* Cp(ctm_ctx* c, int label, int site);

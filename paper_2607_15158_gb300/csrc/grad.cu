@@ -239,6 +239,7 @@ __global__ void diff_norm_kernel(long n, const double* a, const double* b, doubl
 // Device bump allocator in large chunks; released as a whole.
 class Arena {
  public:
+  explicit Arena(ctm_ctx* c) : c_(c) {}
   ~Arena() { release(); }
   void* get(size_t bytes) {
     bytes = (bytes + 255) & ~(size_t)255;
@@ -246,7 +247,7 @@ class Arena {
     if (chunks_.empty() || off_ + bytes > caps_.back()) {
       const size_t cap = std::max(bytes, (size_t)256 << 20);
       void* p = nullptr;
-      if (cudaMalloc(&p, cap) != cudaSuccess) {
+      if (malloc_or_shed(c_, &p, cap) != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
       }
@@ -266,6 +267,7 @@ class Arena {
   }
 
  private:
+  ctm_ctx* c_;
   std::vector<void*> chunks_;
   std::vector<size_t> caps_;
   size_t off_ = 0;
@@ -291,7 +293,7 @@ struct Tape {
   std::unordered_map<void*, long> len;      // elements of each recorded value
   std::unordered_set<void*> constant;       // values with no adjoint
   double* dwork = nullptr;                  // reduction scratch (>= 2 + 2432)
-  explicit Tape(ctm_ctx* cc) : c(cc) {}
+  explicit Tape(ctm_ctx* cc) : c(cc), vals(cc), adjs(cc), tmp(cc) {}
 
   cudaStream_t st() const { return c->stream; }
 
@@ -928,8 +930,10 @@ ctm_status grad_checkpoint(ctm_ctx* c, int r) {
   cp.r = r;
   const size_t nC = 4 * (size_t)c->S * elems_C(c) * 8, nT = 4 * (size_t)c->S * elems_T(c) * 8;
   const size_t nX = (size_t)c->S * c->N * c->k * 8;
-  if (cudaMalloc(&cp.C, nC) != cudaSuccess || cudaMalloc(&cp.T, nT) != cudaSuccess ||
-      cudaMalloc(&cp.X, nX) != cudaSuccess || cudaMalloc(&cp.W, nX) != cudaSuccess) {
+  if (malloc_or_shed(c, &cp.C, nC) != cudaSuccess ||
+      malloc_or_shed(c, &cp.T, nT) != cudaSuccess ||
+      malloc_or_shed(c, &cp.X, nX) != cudaSuccess ||
+      malloc_or_shed(c, &cp.W, nX) != cudaSuccess) {
     cudaGetLastError();
     cudaFree(cp.C);
     cudaFree(cp.T);
@@ -980,7 +984,7 @@ ctm_status ctm_grad(ctm_ctx* c, const void* op, double* E_out, void* dA_out) {
   if (!c->grad) return fail(c, CTM_EINVAL, "no recorded moves: call ctm_record(ctx, 1) first");
   use_lane(c, 0);
   const int S = c->S, d2 = c->d * c->d;
-  Arena keep;
+  Arena keep(c);
   void* dop = keep.get((size_t)d2 * d2 * 8);
   double* dw = static_cast<double*>(keep.get((2 + 2432) * 8));
   AdjState g;
@@ -1085,7 +1089,7 @@ ctm_status ctm_grad_fixed_point(ctm_ctx* c, const void* op, double tol, int max_
     if (!rd) return fail(c, CTM_EINVAL, "converge the environment first");
   use_lane(c, 0);
   const int S = c->S, d2 = c->d * c->d;
-  Arena keep;
+  Arena keep(c);
   void* dop = keep.get((size_t)d2 * d2 * 8);
   double* dw = static_cast<double*>(keep.get((2 + 2432) * 8));
   double* nrm = static_cast<double*>(keep.get(16));

@@ -1213,22 +1213,16 @@ struct SplitCtx {
   void* cslices[4][2] = {{nullptr}};
   int corner_Kp = 0;
   bool borrowed = false;    // cslices belong to another context
-  // generic operand buffers (grown on demand)
-  void* abuf = nullptr;
-  size_t abuf_bytes = 0;
-  void* bbuf = nullptr;
-  size_t bbuf_bytes = 0;
-  float* part = nullptr;
-  size_t part_bytes = 0;
-  // fp64-accurate products: digits of both operands, exponent fields, partials
-  void* oz_a = nullptr;
-  size_t oz_a_bytes = 0;
-  void* oz_b = nullptr;
-  size_t oz_b_bytes = 0;
-  int* oz_e = nullptr;
-  size_t oz_e_bytes = 0;
-  void* oz_part = nullptr;
-  size_t oz_part_bytes = 0;
+  // operand and partial-sum buffers (grown on demand). fp64-accurate products: digits
+  // of both operands, exponent fields, partials
+  struct Buf {
+    void* p = nullptr;
+    size_t bytes = 0;
+    size_t want = 0;        // the most that a product asked for while noting
+  };
+  enum { ABUF, BBUF, PART, OZ_A, OZ_B, OZ_E, OZ_PART, NBUF };
+  Buf buf[NBUF];
+  bool noting = false;
   long oz_launches = 0;
   int* err = nullptr;       // device error flag of the owning context
   // per-launch CUDA events around the tensor-core kernel (profiling)
@@ -1262,16 +1256,17 @@ void mem_release(SplitCtx* sc, void** p, size_t bytes) {
   *p = nullptr;
 }
 
-ctm_status grow(SplitCtx* sc, void** p, size_t* have, size_t need) {
-  if (*have >= need) return CTM_OK;
-  mem_release(sc, p, *have);
-  *have = 0;
-  if (!mem_alloc(sc, p, need))
+ctm_status grow(SplitCtx* sc, int which, size_t need) {
+  SplitCtx::Buf& b = sc->buf[which];
+  if (sc->noting) b.want = std::max(b.want, need);
+  if (b.bytes >= need) return CTM_OK;
+  mem_release(sc, &b.p, b.bytes);
+  b.bytes = 0;
+  if (!mem_alloc(sc, &b.p, need))
     return sfail(sc, CTM_ENOMEM, "split-precision buffer allocation failed");
-  *have = need;
+  b.bytes = need;
   return CTM_OK;
 }
-
 
 int pad_to(int x, int m) { return (x + m - 1) / m * m; }
 
@@ -1326,7 +1321,7 @@ ctm_status run_mma(SplitCtx* sc, const void* As, const void* Bs, int M, int Kp,
   const int nks = choose_splits(mt * nchunks, kb_total, KB_SPLIT_MAX * BK / ke_of(sc));
   const int kb_split = (kb_total + nks - 1) / nks;
   {
-    ctm_status st = grow(sc, (void**)&sc->part, &sc->part_bytes, (size_t)nks * M * Np * 4);
+    ctm_status st = grow(sc, SplitCtx::PART, (size_t)nks * M * Np * 4);
     if (st != CTM_OK) return st;
   }
   CUtensorMap ta, tb;
@@ -1341,7 +1336,8 @@ ctm_status run_mma(SplitCtx* sc, const void* As, const void* Bs, int M, int Kp,
   p.mt = mt;
   p.nchunks = nchunks;
   p.nks = nks;
-  p.part = sc->part;
+  float* const part = static_cast<float*>(sc->buf[SplitCtx::PART].p);
+  p.part = part;
   p.err = sc->err;
   const int ns = ns_of(sc);
   const size_t stage = ns * A_SLICE_BYTES + ns * (size_t)BNc * KROW;
@@ -1381,10 +1377,10 @@ ctm_status run_mma(SplitCtx* sc, const void* As, const void* Bs, int M, int Kp,
   }
   if (launches) ++*launches;
   if (sc->cx)
-    reduce_kernel<cplx><<<grid_cap((long)M * Nout), 256, 0, s>>>(sc->part, nks, M, Nout, Np,
+    reduce_kernel<cplx><<<grid_cap((long)M * Nout), 256, 0, s>>>(part, nks, M, Nout, Np,
                                                                  (cplx*)C, ldc);
   else
-    reduce_kernel<double><<<grid_cap((long)M * Nout), 256, 0, s>>>(sc->part, nks, M, Nout, Np,
+    reduce_kernel<double><<<grid_cap((long)M * Nout), 256, 0, s>>>(part, nks, M, Nout, Np,
                                                                    (double*)C, ldc);
   if (launches) ++*launches;
   if (cudaGetLastError() != cudaSuccess) return sfail(sc, CTM_ECUDA, "split GEMM launch failed");
@@ -1512,13 +1508,7 @@ void split_destroy(SplitCtx* sc) {
   for (int i = 0; i < 4 && !sc->borrowed; ++i)
     for (int o = 0; o < 2; ++o)
       mem_release(sc, &sc->cslices[i][o], slice_bytes(sc, sc->N, sc->corner_Kp));
-  mem_release(sc, &sc->abuf, sc->abuf_bytes);
-  mem_release(sc, &sc->bbuf, sc->bbuf_bytes);
-  mem_release(sc, (void**)&sc->part, sc->part_bytes);
-  mem_release(sc, &sc->oz_a, sc->oz_a_bytes);
-  mem_release(sc, &sc->oz_b, sc->oz_b_bytes);
-  mem_release(sc, (void**)&sc->oz_e, sc->oz_e_bytes);
-  mem_release(sc, &sc->oz_part, sc->oz_part_bytes);
+  for (auto& b : sc->buf) mem_release(sc, &b.p, b.bytes);
   delete sc;
 }
 
@@ -1552,6 +1542,23 @@ void split_borrow_corners(SplitCtx* sc, const SplitCtx* src) {
   }
 }
 
+void split_note(SplitCtx* sc, bool on) { sc->noting = on; }
+
+size_t split_reserve_bytes(const SplitCtx* sc, const SplitCtx* like) {
+  size_t n = 0;
+  for (int i = 0; i < SplitCtx::NBUF; ++i)
+    if (like->buf[i].want > (sc ? sc->buf[i].bytes : 0)) n += device_bytes(like->buf[i].want);
+  return n;
+}
+
+ctm_status split_reserve(SplitCtx* sc, const SplitCtx* like) {
+  for (int i = 0; i < SplitCtx::NBUF; ++i) {
+    const ctm_status st = grow(sc, i, like->buf[i].want);
+    if (st != CTM_OK) return st;
+  }
+  return CTM_OK;
+}
+
 ctm_status split_apply(SplitCtx* sc, const void* Q, bool herm, const void* Zin, void* Zout, int N,
                        int k, cudaStream_t s, long* launches) {
   int ci = -1;
@@ -1564,12 +1571,12 @@ ctm_status split_apply(SplitCtx* sc, const void* Q, bool herm, const void* Zin, 
   int nchunks, BNc;
   chunking(Nr, &nchunks, &BNc);
   const int Np = nchunks * BNc;
-  ctm_status st = grow(sc, (void**)&sc->bbuf, &sc->bbuf_bytes,
-                       (size_t)ns_of(sc) * Np * Kp * eb_of(sc));
+  ctm_status st = grow(sc, SplitCtx::BBUF, (size_t)ns_of(sc) * Np * Kp * eb_of(sc));
   if (st != CTM_OK) return st;
-  st = prep_b(sc, Zin, k, OP_N, N, k, Kp, Np, sc->bbuf, s, launches);
+  void* const bbuf = sc->buf[SplitCtx::BBUF].p;
+  st = prep_b(sc, Zin, k, OP_N, N, k, Kp, Np, bbuf, s, launches);
   if (st != CTM_OK) return st;
-  return run_mma(sc, sc->cslices[ci][herm ? 1 : 0], sc->bbuf, N, Kp, Nr, nchunks, BNc, Zout, k, k,
+  return run_mma(sc, sc->cslices[ci][herm ? 1 : 0], bbuf, N, Kp, Nr, nchunks, BNc, Zout, k, k,
                  s, launches);
 }
 
@@ -1584,15 +1591,16 @@ ctm_status split_gemm(SplitCtx* sc, int opA, const void* A, long lda, int opB, c
   chunking(Nr, &nchunks, &BNc);
   const int Np = nchunks * BNc;
   const size_t per = (size_t)ns_of(sc) * eb_of(sc);
-  ctm_status st = grow(sc, (void**)&sc->abuf, &sc->abuf_bytes, per * M * Kp);
+  ctm_status st = grow(sc, SplitCtx::ABUF, per * M * Kp);
   if (st != CTM_OK) return st;
-  st = grow(sc, (void**)&sc->bbuf, &sc->bbuf_bytes, per * Np * Kp);
+  st = grow(sc, SplitCtx::BBUF, per * Np * Kp);
   if (st != CTM_OK) return st;
-  st = prep_a(sc, A, lda, opA, M, K, Kp, sc->abuf, s, launches);
+  void *const abuf = sc->buf[SplitCtx::ABUF].p, *const bbuf = sc->buf[SplitCtx::BBUF].p;
+  st = prep_a(sc, A, lda, opA, M, K, Kp, abuf, s, launches);
   if (st != CTM_OK) return st;
-  st = prep_b(sc, B, ldb, opB, K, N, Kp, Np, sc->bbuf, s, launches);
+  st = prep_b(sc, B, ldb, opB, K, N, Kp, Np, bbuf, s, launches);
   if (st != CTM_OK) return st;
-  return run_mma(sc, sc->abuf, sc->bbuf, M, Kp, Nr, nchunks, BNc, C, ldc, N, s, launches);
+  return run_mma(sc, abuf, bbuf, M, Kp, Nr, nchunks, BNc, C, ldc, N, s, launches);
 }
 
 ctm_status oz_gemm(SplitCtx* sc, int opA, const void* A, long lda, int opB, const void* B,
@@ -1614,14 +1622,15 @@ ctm_status oz_gemm(SplitCtx* sc, int opA, const void* A, long lda, int opB, cons
                                                   (kb_total + OZ_KB_DRAIN - 1) / OZ_KB_DRAIN));
   const int kb_split = (kb_total + nks - 1) / nks;
   nks = (kb_total + kb_split - 1) / kb_split;
-  ctm_status st = grow(sc, &sc->oz_a, &sc->oz_a_bytes, (size_t)OZ_NS * M * Kp * 2);
-  if (st == CTM_OK) st = grow(sc, &sc->oz_b, &sc->oz_b_bytes, (size_t)OZ_NS * Np * Kp * 2);
-  if (st == CTM_OK) st = grow(sc, (void**)&sc->oz_e, &sc->oz_e_bytes, (size_t)(M + N) * sizeof(int));
-  if (st == CTM_OK) st = grow(sc, &sc->oz_part, &sc->oz_part_bytes, (size_t)nks * M * Np * 8);
+  ctm_status st = grow(sc, SplitCtx::OZ_A, (size_t)OZ_NS * M * Kp * 2);
+  if (st == CTM_OK) st = grow(sc, SplitCtx::OZ_B, (size_t)OZ_NS * Np * Kp * 2);
+  if (st == CTM_OK) st = grow(sc, SplitCtx::OZ_E, (size_t)(M + N) * sizeof(int));
+  if (st == CTM_OK) st = grow(sc, SplitCtx::OZ_PART, (size_t)nks * M * Np * 8);
   if (st != CTM_OK) return st;
-  int* ea = sc->oz_e;
-  int* ebx = sc->oz_e + M;
-  if (cudaMemsetAsync(sc->oz_e, 0, (size_t)(M + N) * sizeof(int), s) != cudaSuccess)
+  void *const oz_a = sc->buf[SplitCtx::OZ_A].p, *const oz_b = sc->buf[SplitCtx::OZ_B].p;
+  int* const ea = static_cast<int*>(sc->buf[SplitCtx::OZ_E].p);
+  int* const ebx = ea + M;
+  if (cudaMemsetAsync(ea, 0, (size_t)(M + N) * sizeof(int), s) != cudaSuccess)
     return sfail(sc, CTM_ECUDA, "exponent reset failed");
   auto prepare = [&](auto zero) {
     using T = decltype(zero);
@@ -1632,7 +1641,7 @@ ctm_status oz_gemm(SplitCtx* sc, int opA, const void* A, long lda, int opB, cons
     a.rows = opA == OP_N || opA == OP_R;
     a.cj = opA == OP_C || opA == OP_R;
     a.e = ea;
-    a.out = static_cast<__nv_bfloat16*>(sc->oz_a);
+    a.out = static_cast<__nv_bfloat16*>(oz_a);
     a.Vp = M;
     b.p = static_cast<const T*>(B);
     b.ld = ldb;
@@ -1640,7 +1649,7 @@ ctm_status oz_gemm(SplitCtx* sc, int opA, const void* A, long lda, int opB, cons
     b.rows = opB == OP_T || opB == OP_C;
     b.cj = opB == OP_C || opB == OP_R;
     b.e = ebx;
-    b.out = static_cast<__nv_bfloat16*>(sc->oz_b);
+    b.out = static_cast<__nv_bfloat16*>(oz_b);
     b.Vp = Np;
     for (OzOperand<T>* o : {&a, &b}) {
       o->K = K;
@@ -1655,8 +1664,8 @@ ctm_status oz_gemm(SplitCtx* sc, int opA, const void* A, long lda, int opB, cons
   else prepare(0.0);
   if (launches) *launches += 2;
   CUtensorMap ta, tb;
-  if (!make_map(&ta, sc->oz_a, M, Kp, BM, false, OZ_NS) ||
-      !make_map(&tb, sc->oz_b, Np, Kp, BNc, false, OZ_NS))
+  if (!make_map(&ta, oz_a, M, Kp, BM, false, OZ_NS) ||
+      !make_map(&tb, oz_b, Np, Kp, BNc, false, OZ_NS))
     return sfail(sc, CTM_ECUDA, "cuTensorMapEncodeTiled failed");
   OzParams p;
   p.M = M;
@@ -1667,7 +1676,7 @@ ctm_status oz_gemm(SplitCtx* sc, int opA, const void* A, long lda, int opB, cons
   p.mt = mt;
   p.nchunks = nchunks;
   p.nks = nks;
-  p.part = static_cast<float2*>(sc->oz_part);
+  p.part = static_cast<float2*>(sc->buf[SplitCtx::OZ_PART].p);
   p.err = sc->err;
   const size_t smem = 1024 + 2 * OZ_GA + 2 * OZ_GB;
   static size_t configured = 0;

@@ -37,6 +37,21 @@ ctm_status split_prepare_corners(SplitCtx* sc, void* const* Q, int N, unsigned m
 // slices stay src's, and the caller orders their use.
 void split_borrow_corners(SplitCtx* sc, const SplitCtx* src);
 
+// While noting, sc keeps the largest size that its products ask of each operand
+// buffer. split_reserve gives another state buffers of those sizes, so that it runs
+// the same products without an allocation; split_reserve_bytes is the device memory
+// that this would add (sc null: to a new one).
+void split_note(SplitCtx* sc, bool on);
+size_t split_reserve_bytes(const SplitCtx* sc, const SplitCtx* like);
+ctm_status split_reserve(SplitCtx* sc, const SplitCtx* like);
+
+// device memory that an allocation of this many bytes occupies: whole pages of 2 MiB
+// from half a page on, below that its share of one
+inline size_t device_bytes(size_t bytes) {
+  const size_t unit = bytes >= ((size_t)1 << 20) ? (size_t)2 << 20 : (size_t)512;
+  return (bytes + unit - 1) / unit * unit;
+}
+
 // Zout = op(Q) Zin for one of the prepared corners (identified by pointer),
 // Zin, Zout fp64 N x k row-major.
 ctm_status split_apply(SplitCtx* sc, const void* Q, bool herm, const void* Zin, void* Zout,
