@@ -457,6 +457,10 @@ void ctm_debug_fail_alloc(int after);
  * that were replayed from a CUDA graph (small cells past their warm-up). */
 ctm_status ctm_debug_moves(const ctm_ctx* ctx, long* direct, long* replayed);
 
+/* For tests: sqrt(x), 1 / sqrt(x) (of the rounded root) and 1 / x of n host
+ * values as the Cholesky kernels take them. */
+ctm_status ctm_debug_roots(long n, const double* x, double* root, double* rroot, double* rcp);
+
 /* For tests: the device memory that the context holds, and the helpers on which
  * it runs halves of cuts side by side (0: it runs them one after the other). */
 ctm_status ctm_debug_memory(const ctm_ctx* ctx, size_t* used, int* helpers);

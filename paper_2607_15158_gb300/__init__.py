@@ -93,6 +93,7 @@ def load():
         "ctm_si_stats": (I, [ctx_p, P(C.c_long), P(C.c_long)]),
         "ctm_transfer_spectrum": (I, [ctx_p, I, I, I, P(D), P(D)]),
         "ctm_debug_fail_alloc": (None, [I]),
+        "ctm_debug_roots": (I, [C.c_long, VP, VP, VP, VP]),
         "ctm_debug_memory": (I, [ctx_p, P(C.c_size_t), P(I)]),
         "ctm_debug_moves": (I, [ctx_p, P(C.c_long), P(C.c_long)]),
         "ctm_record": (I, [ctx_p, I]),
@@ -475,6 +476,15 @@ def ctm_debug_fail_alloc(after):
     """Make the device allocation after `after` successful ones fail (test
     hook of the error paths); after < 0 disarms it."""
     load().ctm_debug_fail_alloc(int(after))
+
+
+def ctm_debug_roots(x):
+    """(sqrt(x), 1 / sqrt(x), 1 / x) as the Cholesky kernels take them."""
+    lib = load()
+    x = np.ascontiguousarray(x, dtype=np.float64)
+    out = [np.empty_like(x) for _ in range(3)]
+    _check(lib, None, lib.ctm_debug_roots(x.size, x.ctypes.data, *[o.ctypes.data for o in out]))
+    return tuple(out)
 
 
 def ctm_init(Lx, Ly, A, d, D, chi, cplx=None, bra=None, opts=None):

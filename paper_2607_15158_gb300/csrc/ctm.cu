@@ -2593,6 +2593,29 @@ ctm_status ctm_transfer_spectrum(ctm_ctx* c, int dir, int row, int nvals, double
   return CTM_OK;
 }
 
+ctm_status ctm_debug_roots(long n, const double* x, double* root, double* rroot, double* rcp) {
+  if (n < 1 || !x || !root || !rroot || !rcp)
+    return fail(nullptr, CTM_EINVAL, "bad arguments of ctm_debug_roots");
+  const size_t bytes = (size_t)n * sizeof(double);
+  double* d = nullptr;   // x, root, rroot, rcp
+  cudaStream_t s = nullptr;
+  ctm_status st = CTM_OK;
+  if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaMalloc(&d, 4 * bytes) != cudaSuccess)
+    st = CTM_ENOMEM;
+  else if (cudaMemcpyAsync(d, x, bytes, cudaMemcpyHostToDevice, s) != cudaSuccess ||
+           pivot_roots(n, d, d + n, d + 2 * n, d + 3 * n, s) != cudaSuccess ||
+           cudaMemcpyAsync(root, d + n, bytes, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+           cudaMemcpyAsync(rroot, d + 2 * n, bytes, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+           cudaMemcpyAsync(rcp, d + 3 * n, bytes, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+           cudaStreamSynchronize(s) != cudaSuccess)
+    st = CTM_ECUDA;
+  cudaGetLastError();
+  if (d) cudaFree(d);
+  if (s) cudaStreamDestroy(s);
+  return st == CTM_OK ? CTM_OK : fail(nullptr, st, "ctm_debug_roots failed on the device");
+}
+
 ctm_status ctm_debug_memory(const ctm_ctx* c, size_t* used, int* helpers) {
   if (!c) return CTM_EINVAL;
   if (used) *used = c->mem_used;

@@ -121,6 +121,10 @@ cudaError_t sub_inplace(bool cx, long n, void* z, const void* d, cudaStream_t s,
 // receives D (k doubles). W may alias G. Supported up to k ~ 390 complex,
 // 576 real (chol_cluster_supported).
 bool chol_cluster_supported(bool cx, int k);
+// the square root, its reciprocal and the reciprocal of x[0 .. n - 1] as the factor
+// takes them (for tests)
+cudaError_t pivot_roots(long n, const double* x, double* root, double* rroot, double* rcp,
+                        cudaStream_t s);
 cudaError_t chol_cluster(bool cx, int k, long rows, bool shift, bool scale, const void* G,
                          void* L, double* dsc, int* dead, void* W, int* err, cudaStream_t s,
                          long* launches);
