@@ -369,9 +369,9 @@ template <typename T>
 cudaError_t dispatch_vals(const ValsArgs& a, int batch, size_t shm, cudaStream_t s) {
   if (a.k <= 32) return launch_vals<T, 1>(a, batch, shm, s);
   if (a.k <= 64) return launch_vals<T, 2>(a, batch, shm, s);
-  if (a.k <= 96) return launch_vals<T, 3>(a, batch, shm, s);
-  if (a.k <= 128) return launch_vals<T, 4>(a, batch, shm, s);
-  return launch_vals<T, 5>(a, batch, shm, s);
+  if constexpr (sizeof(T) == 8)
+    if (a.k > 96) return launch_vals<T, 4>(a, batch, shm, s);
+  return launch_vals<T, 3>(a, batch, shm, s);
 }
 
 }  // namespace
