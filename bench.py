@@ -35,9 +35,10 @@ WARM_ITERS, WARM_ROUNDS = 2, 4
 # DRAM bytes (read + write) per launch of split_mma_kernel<FmtBF16> over the
 # kernel's algorithmic bytes (all slices of both operands + the fp32 split-K
 # partials), from a one-pass ncu capture of a corner x block launch at
-# N = 5184, k = 149 (469.2 MB / 501.7 MB); only valid for the bf16 kernel as
-# captured, so it is set to None whenever that kernel changes
-TRAFFIC_PER_OPERAND_BYTE = 0.935
+# N = 5184, k = 149 (460.3 MB / 501.7 MB); only valid for the bf16 kernel as
+# captured (persistent grid of 320-thread CTAs), so it is set to None whenever
+# that kernel changes
+TRAFFIC_PER_OPERAND_BYTE = 0.917
 SLICE_PRODUCTS = 6   # bf16 slice products per algorithmic product
 METRIC = "CTMRG moves/s & tensor TFLOP/s at D=6, chi=144"
 UNIT = "moves/s"
