@@ -357,8 +357,8 @@ def run_ours(args, rank, world, local_rank):
                     "frac": round(achieved / peak, 4), "traffic": traffic,
                     "traffic_basis": "bytes per launch: ncu dram read + write of one "
                                      "corner x block launch (N = 5184, k = 149) over its "
-                                     "algorithmic bytes (0.935) x this run's algorithmic "
-                                     "bytes per launch",
+                                     f"algorithmic bytes ({TRAFFIC_PER_OPERAND_BYTE}) x this "
+                                     "run's algorithmic bytes per launch",
                     "achieved_basis": "algorithmic flops (8 per complex multiply-add) per "
                                       "launch / CUDA-event duration on the launching stream",
                     "tensor_pipe_achieved": round(pipe, 2),
